@@ -381,8 +381,16 @@ __global__ void __launch_bounds__(32 * lanes_per_rhs<BP>()) k_dir_b(DevLevel L, 
             if (!*flag) return;
             __threadfence();
             double t = 0.0;
-            if (act)
-                for (int sb = warp; sb < L.nsub; sb += kDW) t += __ldcg(&rz.part[(int64_t)sb * K + lane]);
+            if (act) {
+                for (int sb = warp; sb < L.nsub; sb += 8 * kDW) {   // eight loads in flight
+                    double v[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        v[u] = sb + u * kDW < L.nsub ? __ldcg(&rz.part[(int64_t)(sb + u * kDW) * K + lane]) : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) t += v[u];
+                }
+            }
             red[warp * 32 + lane] = t;
             __syncthreads();
             if (warp == 0 && act) {
@@ -1122,8 +1130,18 @@ __global__ void __launch_bounds__(kSBMaxT, 1) k_dir_bs(DevLevel L, BatchLevel B,
             // bucket of the finishing block: the same order in every run
             for (int g = w; g < 8; g += nw) {
                 double t = 0.0;
-                if (lane < K)
-                    for (int sb = g; sb < L.nsub; sb += 8) t += __ldcg(&rz.part[(int64_t)sb * K + lane]);
+                if (lane < K) {
+                    // sixteen loads in flight (one at a time, this tail took
+                    // 25 us more at 1024 substructures)
+                    for (int sb = g; sb < L.nsub; sb += 8 * 16) {
+                        double v[16];
+#pragma unroll
+                        for (int u = 0; u < 16; ++u)
+                            v[u] = sb + 8 * u < L.nsub ? __ldcg(&rz.part[(int64_t)(sb + 8 * u) * K + lane]) : 0.0;
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) t += v[u];
+                    }
+                }
                 red[g * 32 + lane] = t;
             }
             __syncthreads();

@@ -553,7 +553,14 @@ __global__ void __launch_bounds__(kTcThreads, 2)
                         __threadfence();
                         double tsum = 0.0;
                         if (lane < K)
-                            for (int sb = ew; sb < L.nsub; sb += 4) tsum += __ldcg(&rz.part[(int64_t)sb * K + lane]);
+                            for (int sb = ew; sb < L.nsub; sb += 4 * 16) {   // sixteen loads in flight
+                                double v[16];
+#pragma unroll
+                                for (int u = 0; u < 16; ++u)
+                                    v[u] = sb + 4 * u < L.nsub ? __ldcg(&rz.part[(int64_t)(sb + 4 * u) * K + lane]) : 0.0;
+#pragma unroll
+                                for (int u = 0; u < 16; ++u) tsum += v[u];
+                            }
                         red[ew * 32 + lane] = tsum;
                         bar_sync(2, 128);
                         if (ew == 0 && lane < K) {
