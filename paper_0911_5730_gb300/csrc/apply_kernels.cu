@@ -310,13 +310,26 @@ __global__ void __launch_bounds__(kSB) k_dir_s(DevLevel L, const double *r, doub
 }
 
 // (6)-(8): f = D_i r_B on Gamma; w = N_i f; r_c += Psi_i^T f.
+// Latency of the loads of N_i (from L2) bounds this: a block takes kNRows
+// rows of one substructure (blockIdx.y), a lane per row, and its warps share
+// the columns, so that few large substructures still fill the GPU and a
+// thread's chain is nG / 8 loads, four in flight.  (With one block per
+// substructure and a thread per row, the two levels of the three-level
+// elasticity problem at 384^2, nine substructures on level 2, took 113 us of
+// an iteration: an FP32 solve 8.03 ms, now 5.54.)
+constexpr int kNRows = 32, kNWarps = 8;
 template <class T, class ACC>
-__global__ void k_neumann(DevLevel L, const double *r, const int *skip) {
+__global__ void __launch_bounds__(32 * kNWarps) k_neumann(DevLevel L, const double *r, const int *skip) {
     if (skip && *skip) return;
     extern __shared__ unsigned char smem_raw[];
+    __shared__ ACC part[kNWarps][kNRows];
     ACC *f = reinterpret_cast<ACC *>(smem_raw);
     const int sub = blockIdx.x;
     const int nG = L.nG[sub], nc = L.ncl[sub];
+    const int q0 = blockIdx.y * kNRows;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // blocks past the rows of a small substructure may still hold coarse rows
+    if (q0 >= nG && (int)(blockIdx.y * kNWarps) >= nc) return;
     const OpSet<T> &O = Ops<T>::get(L);
     const int64_t g0 = L.offG[sub];
     for (int q = threadIdx.x; q < nG; q += blockDim.x) {
@@ -324,15 +337,28 @@ __global__ void k_neumann(DevLevel L, const double *r, const int *skip) {
         f[q] = ld<T, ACC>(O.wg + g0 + q) * (ACC)(r[L.ifaceDof[id]] + L.rB[id]);
     }
     __syncthreads();
-    const T *N = O.nmat + L.offN[sub];
-    for (int q = threadIdx.x; q < nG; q += blockDim.x) {
-        ACC s = 0;
-        for (int p = 0; p < nG; ++p) s += ld<T, ACC>(N + (int64_t)p * nG + q) * f[p];
-        L.w[g0 + q] = (double)s;
+    if (q0 < nG) {
+        const int q = q0 + lane;
+        const T *N = O.nmat + L.offN[sub] + (q < nG ? q : nG - 1);
+        ACC s[4] = {0, 0, 0, 0};
+        int p = warp;
+        for (; p + 3 * kNWarps < nG; p += 4 * kNWarps) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                s[u] += ld<T, ACC>(N + (int64_t)(p + u * kNWarps) * nG) * f[p + u * kNWarps];
+        }
+        for (; p < nG; p += kNWarps) s[0] += ld<T, ACC>(N + (int64_t)p * nG) * f[p];
+        part[warp][lane] = (s[0] + s[1]) + (s[2] + s[3]);
+        __syncthreads();
+        if (warp == 0 && q < nG) {
+            ACC t = 0;
+#pragma unroll
+            for (int w = 0; w < kNWarps; ++w) t += part[w][lane];
+            L.w[g0 + q] = (double)t;
+        }
     }
     const T *P = O.psit + L.offP[sub];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int k = warp; k < nc; k += nw) {
+    for (int k = blockIdx.y * kNWarps + warp; k < nc; k += kNWarps * gridDim.y) {
         ACC s = 0;
         for (int q = lane; q < nG; q += 32) s += ld<T, ACC>(P + (int64_t)k * nG + q) * f[q];
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -1299,6 +1325,12 @@ template <class T, class ACC> void pre_t(const DevLevel &L, const double *r, con
     }
     launch_k(false, k_pre<T, ACC>, L.nsub, kGT, generic_smem<ACC>(L), s, L, r, skip);
 }
+template <class T, class ACC> void neumann_t(const DevLevel &L, const double *r, const int *skip, cudaStream_t s) {
+    const int rows = (L.max_nG + kNRows - 1) / kNRows;
+    const dim3 grid((unsigned)L.nsub, (unsigned)(rows > 0 ? rows : 1));
+    launch_grid(false, k_neumann<T, ACC>, grid, 32 * kNWarps, sizeof(ACC) * (size_t)(L.max_nG > 0 ? L.max_nG : 1), s, L, r,
+              skip);
+}
 template <class T, class ACC> void post_t(const DevLevel &L, const double *r, double *z,
                                           const int *skip, cudaStream_t s) {
     if (stream_fits<T, ACC>(L)) {
@@ -1482,10 +1514,9 @@ void apply_level_neumann(const DevLevel &L, int prec, const double *r, const int
         else neu_launch<__nv_bfloat16, float>(L, prec, r, skip, s);
         return;
     }
-    const size_t smn = sizeof(double) * (size_t)(L.max_nG > L.max_nc ? L.max_nG : L.max_nc);
-    if (prec == BDDC_PREC_FP64) launch_k(false, k_neumann<double, double>, L.nsub, 128, smn, s, L, r, skip);
-    else if (prec == BDDC_PREC_FP32) launch_k(false, k_neumann<float, float>, L.nsub, 128, smn, s, L, r, skip);
-    else launch_k(false, k_neumann<__nv_bfloat16, float>, L.nsub, 128, smn, s, L, r, skip);
+    if (prec == BDDC_PREC_FP64) neumann_t<double, double>(L, r, skip, s);
+    else if (prec == BDDC_PREC_FP32) neumann_t<float, float>(L, r, skip, s);
+    else neumann_t<__nv_bfloat16, float>(L, r, skip, s);
 }
 
 void apply_level_average(const DevLevel &L, int prec, const int *skip, cudaStream_t s) {

@@ -137,10 +137,10 @@ inline bool pdl_enabled() {
 
 // Launch with (pdl) or without programmatic stream serialisation.
 template <class... KArgs, class... Args>
-inline void launch_k(bool pdl, void (*k)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
-                     Args... args) {
+inline void launch_grid(bool pdl, void (*k)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s,
+                        Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -153,10 +153,16 @@ inline void launch_k(bool pdl, void (*k)(KArgs...), int grid, int block, size_t 
     if (e != cudaSuccess) {
         const char *name = nullptr;
         if (cudaFuncGetName(&name, reinterpret_cast<const void *>(k)) != cudaSuccess || !name) name = "?";
-        throw Error(BDDC_E_CUDA, std::string("launch of ") + name + " (grid " + std::to_string(grid) +
-                                     ", block " + std::to_string(block) + ", shared " + std::to_string(smem) +
+        throw Error(BDDC_E_CUDA, std::string("launch of ") + name + " (grid " + std::to_string(grid.x) + " x " +
+                                     std::to_string(grid.y) + ", block " + std::to_string(block) + ", shared " + std::to_string(smem) +
                                      "): " + cudaGetErrorString(e));
     }
+}
+
+template <class... KArgs, class... Args>
+inline void launch_k(bool pdl, void (*k)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                     Args... args) {
+    launch_grid(pdl, k, dim3((unsigned)grid), block, smem, s, args...);
 }
 
 template <class... KArgs, class... Args>
