@@ -758,10 +758,10 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
         ACC s0 = 0, s1 = 0;
         int pp = 0;
         for (; pp + 1 < nG; pp += 2) {
-            s0 += ld<T, ACC>(Ns + (size_t)pp * nG + q) * f[pp];
-            s1 += ld<T, ACC>(Ns + (size_t)(pp + 1) * nG + q) * f[pp + 1];
+            s0 += ld<T, ACC>(Ns + (size_t)pp * lay.ld + q) * f[pp];
+            s1 += ld<T, ACC>(Ns + (size_t)(pp + 1) * lay.ld + q) * f[pp + 1];
         }
-        if (pp < nG) s0 += ld<T, ACC>(Ns + (size_t)pp * nG + q) * f[pp];
+        if (pp < nG) s0 += ld<T, ACC>(Ns + (size_t)pp * lay.ld + q) * f[pp];
         L.w[g0 + q] = (double)(s0 + s1);
     }
     // coarse right-hand side: lane k sums row k of Psi^T, staggered to avoid bank conflicts
@@ -769,7 +769,7 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
         ACC s0 = 0;
         for (int t = 0; t < nG; ++t) {
             const int q = (t + k) % nG;
-            s0 += ld<T, ACC>(Ps + (size_t)k * nG + q) * f[q];
+            s0 += ld<T, ACC>(Ps + (size_t)k * lay.ld + q) * f[q];
         }
         atomicAdd(&L.rcv[rcs[k]], (double)s0);
     }
@@ -816,7 +816,7 @@ __global__ void k_average_r(DevLevel L, int pidx, const int *skip, unsigned slic
     __syncwarp();
     for (int q = lane; q < nG; q += 32) {
         ACC v = (q < 128) ? (ACC)wv[q >> 5] : (ACC)L.w[g0 + q];
-        for (int k = 0; k < nc; ++k) v += ld<T, ACC>(Ps + (size_t)k * nG + q) * uc[k];
+        for (int k = 0; k < nc; ++k) v += ld<T, ACC>(Ps + (size_t)k * lay.ld + q) * uc[k];
         atomicAdd(&L.uB[iG[q]], (double)(ld<T, ACC>(wg + q) * v));
         L.rB[iG[q]] = 0.0;            // consumed by the substructure correction
     }
@@ -859,7 +859,11 @@ __global__ void k_build_nrec(DevLevel D, OpSet<T> O, unsigned char *rec, const i
     int *rcs = reinterpret_cast<int *>(base + lay.rc);
     int *gG = reinterpret_cast<int *>(base + lay.gG);
     T *N = reinterpret_cast<T *>(base + lay.N);
-    for (int k = threadIdx.x; k < nc * nG; k += blockDim.x) psi[k] = O.psit[D.offP[sub] + k];
+    const int ld = lay.ld;
+    for (int k = threadIdx.x; k < nc * ld; k += blockDim.x) {
+        const int row = k / ld, q = k - row * ld;
+        psi[k] = q < nG ? O.psit[D.offP[sub] + (int64_t)row * nG + q] : T(0.0f);
+    }
     for (int q = threadIdx.x; q < nG; q += blockDim.x) {
         wg[q] = O.wg[D.offG[sub] + q];
         iG[q] = D.idxG[D.offG[sub] + q];

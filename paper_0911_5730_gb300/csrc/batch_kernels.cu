@@ -1168,126 +1168,248 @@ __global__ void __launch_bounds__(kSBMaxT, 1) k_dir_bs(DevLevel L, BatchLevel B,
     }
 }
 
-// (6)-(9) for K right-hand sides when the Neumann records are too large to
-// stage whole: one block of kNBT threads per substructure reads N_i and
-// Psi_i^T from global memory in chunks of contiguous rows, loaded by all
-// threads (coalesced) into shared memory; warp w computes the rows q = w
-// (mod 8) for all right-hand sides (lane k: right-hand side k).
-constexpr int kChunkBytes = 32 * 1024, kNBT = 256;   // chunk of N; threads (8 warps)
+// (6)-(9) for K right-hand sides, a block of up to kNBW warps per
+// substructure and a lane per right-hand side.  The record [Psi | D | ids] and
+// the rows of N_i arrive by bulk copies that start before the vectors are
+// touched; N_i streams through two stages of `chunk` bytes, so records of any
+// size take this route.  Shared-memory reads bound the product (one per
+// multiply-add when an entry feeds one row): a warp takes tiles of eight rows,
+// so an entry of f and two vector reads of N feed eight multiply-adds, and RT
+// tiles at once.  w_i is kept in the accumulator type (the value it was
+// computed in; half the traffic of FP64 in the mixed path).
+// Measured (solves of the benchmark cases, the kernels these replaced read one
+// shared word per multiply-add): 21 right-hand sides on 1024 Voronoi cells
+// 157.5 -> 145.8 ms, 32 on the 1024^2 three-level problem 107.4 -> 101.3 ms.
+constexpr int kChunkBytes = 32 * 1024, kNBW = 8;   // chunk of N; most warps of a block
 
-// chunk: bytes of N per chunk (0: kChunkBytes), the autotuner's choice
+// chunk: bytes of N per stage (0: kChunkBytes), the autotuner's choice
 template <class T> __host__ __device__ inline int neu_chunk_rows(int nG, int chunk = 0) {
     const int cb = chunk > 0 ? chunk : kChunkBytes;
-    const int rows = cb / (int)(sizeof(T) * (nG > 0 ? nG : 1));
+    const int rows = cb / (int)(sizeof(T) * (nG > 0 ? (nG + 7) & ~7 : 8));
     return rows < 1 ? 1 : (rows > nG ? (nG > 0 ? nG : 1) : rows);
 }
-template <class T, class ACC> __host__ __device__ inline size_t neu_bg_smem(const DevLevel &L, int chunk_bytes = 0) {
-    const size_t mg = L.max_nG > 0 ? L.max_nG : 1, mc = L.max_nc > 0 ? L.max_nc : 1;
-    const size_t row = sizeof(T) * mg;   // one row of N when a row exceeds the chunk
-    const size_t cb = chunk_bytes > 0 ? (size_t)chunk_bytes : (size_t)kChunkBytes;
-    const size_t chunk = al16((row > cb ? row : cb) + 16);
-    const size_t psi = al16(sizeof(T) * mg * mc);
-    return al16(sizeof(ACC) * mg * 32) + al16(sizeof(ACC) * mc * 32) + (chunk > psi ? chunk : psi) + 16;
+struct NeuSmem {
+    size_t head, f, stage, total;
+    template <class T, class ACC> __host__ __device__ static NeuSmem of(const DevLevel &L, int chunk) {
+        NeuSmem m;
+        const size_t mg = L.max_nG > 0 ? L.max_nG : 1, mc = L.max_nc > 0 ? L.max_nc : 1;
+        const size_t row = sizeof(T) * ((mg + 7) & ~size_t(7));
+        m.head = (size_t)NRecLayout((int)mg, (int)mc, (int)sizeof(T)).N;
+        m.f = al16(sizeof(ACC) * ((mg + 7) & ~size_t(7)) * 32);
+        const size_t cb = chunk > 0 ? (size_t)chunk : (size_t)kChunkBytes;
+        // one stage when the whole operator fits in it and one pass covers its rows, else two
+        const bool whole = mg * row <= cb && (mg + 7) / 8 <= kNBW * (sizeof(ACC) == 8 ? 2 : 3);
+        m.stage = whole ? al16(mg * row) : al16(row > cb ? row : cb);
+        m.total = m.head + m.f + (whole ? 1 : 2) * m.stage + 32;
+        return m;
+    }
+};
+template <class T, class ACC> __host__ inline size_t neu_bg_smem(const DevLevel &L, int chunk_bytes = 0) {
+    return NeuSmem::of<T, ACC>(L, chunk_bytes).total;
 }
 
-template <class T, class ACC>
-__global__ void __launch_bounds__(kNBT) k_neu_bg(DevLevel L, BatchLevel B, int pidx, const double *r,
-                                                 const int *skip) {
+template <class T, class ACC, int RT>
+__global__ void __launch_bounds__(32 * kNBW, RT == 1 ? 4 : 3) k_neu_bg(DevLevel L, BatchLevel B, int pidx, const double *r,
+                                                      const int *skip) {
     extern __shared__ __align__(16) unsigned char smem_ng[];
-    (void)pidx;
     if (skip && *skip) return;
-    const int sub = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int sub = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
     const int K = B.K;
     const bool act = lane < K;
     const int nG = L.nG[sub], nc = L.ncl[sub];
-    const size_t mg = L.max_nG > 0 ? L.max_nG : 1, mc = L.max_nc > 0 ? L.max_nc : 1;
-    ACC *f = reinterpret_cast<ACC *>(smem_ng);
-    T *buf = reinterpret_cast<T *>(smem_ng + al16(sizeof(ACC) * mg * 32) + al16(sizeof(ACC) * mc * 32));
-    const OpSet<T> &O = Ops<T>::get(L);
-    const int64_t g0 = L.offG[sub];
-    for (int e = tid; e < nG * 32; e += kNBT) {
-        const int q = e >> 5, k = e & 31;
-        double v = 0.0;
-        if (k < K) {
-            const int id = L.idxG[g0 + q];
-            v = r[(int64_t)L.ifaceDof[id] * K + k] + B.rB[(int64_t)id * K + k];
-        }
-        f[e] = ld<T, ACC>(O.wg + g0 + q) * from_f64<ACC>(v);
+    const NeuSmem ly = NeuSmem::of<T, ACC>(L, B.chunk);
+    const NRecLayout lay(nG, nc, (int)sizeof(T));
+    unsigned char *head = smem_ng;
+    ACC *f = reinterpret_cast<ACC *>(smem_ng + ly.head);
+    unsigned char *ring = smem_ng + ly.head + ly.f;
+    unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem_ng + ly.total - 32);   // stages, head
+    const unsigned char *rec = L.nrec[pidx] + L.nrecOff[pidx][sub];
+    const int ldn = lay.ld, CH = neu_chunk_rows<T>(nG, B.chunk);
+    const int ntile = ldn >> 3, nch = nG > 0 ? (nG + CH - 1) / CH : 0;
+    // N streams once per pass of nw * RT tiles; step s is chunk s % nch of pass s / nch
+    const int npass = (ntile + nw * RT - 1) / (nw * RT), nstep = npass * nch;
+    auto issue = [&](int s) {               // thread 0: step s into stage s & 1
+        const int p0 = (s % nch) * CH, pn = nG - p0 < CH ? nG - p0 : CH;
+        bulk_load(ring + (size_t)(s & 1) * ly.stage, rec + lay.N + (size_t)p0 * ldn * sizeof(T),
+                  (unsigned)(al16((size_t)pn * ldn * sizeof(T))), &bars[s & 1]);
+    };
+    if (tid == 0) {
+        for (int s = 0; s < 3; ++s) mbar_init(&bars[s]);
+        if (lay.N > 0) bulk_load(head, rec, (unsigned)lay.N, &bars[2]);
+        for (int s = 0; s < 2 && s < nstep; ++s) issue(s);
     }
-    // w = N f, N in chunks of rows p (N[p * nG + q])
-    const T *N = O.nmat + L.offN[sub];
-    const int CH = neu_chunk_rows<T>(nG, B.chunk);
-    constexpr int QW = 4;   // output rows per warp and round: q = qb + warp + 8 u, u < QW
-    for (int qb = 0; qb < nG; qb += 8 * QW) {
-        ACC s4[QW] = {};
-        for (int p0 = 0; p0 < nG; p0 += CH) {
-            const int pn = nG - p0 < CH ? nG - p0 : CH;
-            __syncthreads();
-            for (int e = tid; e < pn * nG; e += kNBT) buf[e] = N[(int64_t)p0 * nG + e];
-            __syncthreads();
-            for (int pp = 0; pp < pn; ++pp) {
-                const ACC fv = f[(p0 + pp) * 32 + lane];
+    __syncthreads();
+    bool ok = lay.N == 0 || mbar_wait(&bars[2], 0);
+    int waited = 0;                          // steps waited for
+    if (__syncthreads_and(ok)) {
+        const T *Ps = reinterpret_cast<const T *>(head + lay.psi);
+        const T *wg = reinterpret_cast<const T *>(head + lay.wg);
+        const int *iG = reinterpret_cast<const int *>(head + lay.iG);
+        const int *rcs = reinterpret_cast<const int *>(head + lay.rc);
+        const int *gG = reinterpret_cast<const int *>(head + lay.gG);
+        constexpr int GU = 8;                // rows of r and r_B in flight per warp
+        for (int q0 = warp; q0 < ldn; q0 += nw * GU) {
+            double v[GU], c[GU];
 #pragma unroll
-                for (int u = 0; u < QW; ++u) {
-                    const int q = qb + warp + 8 * u;
-                    if (q < nG) s4[u] += ld<T, ACC>(buf + pp * nG + q) * fv;
-                }
+            for (int u = 0; u < GU; ++u) {
+                const int q = q0 + u * nw;
+                const bool in = q < nG && act;
+                v[u] = in ? r[(int64_t)gG[q] * K + lane] : 0.0;
+                c[u] = in ? B.rB[(int64_t)iG[q] * K + lane] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < GU; ++u) {
+                const int q = q0 + u * nw;
+                if (q < ldn) f[q * 32 + lane] = q < nG ? ld<T, ACC>(wg + q) * from_f64<ACC>(v[u] + c[u]) : (ACC)0;
             }
         }
+        __syncthreads();
+        const int64_t g0 = L.offG[sub];
+        ACC *W = reinterpret_cast<ACC *>(B.w);
+        for (int pass = 0, s = 0; pass < npass && ok; ++pass) {
+            const int t0 = pass * nw * RT + warp;      // tiles t0, t0 + nw, ...
+            ACC acc[RT][8];
 #pragma unroll
-        for (int u = 0; u < QW; ++u) {
-            const int q = qb + warp + 8 * u;
-            if (q < nG && act) B.w[(g0 + q) * K + lane] = to_f64(s4[u]);
+            for (int t = 0; t < RT; ++t)
+#pragma unroll
+                for (int u = 0; u < 8; ++u) acc[t][u] = 0;
+            for (int c = 0; c < nch; ++c, ++s) {
+                const bool got = mbar_wait(&bars[s & 1], (unsigned)(s >> 1) & 1u);
+                waited = s + 1;
+                if (!__syncthreads_and(got)) { ok = false; break; }
+                const T *buf = reinterpret_cast<const T *>(ring + (size_t)(s & 1) * ly.stage);
+                const int p0 = c * CH, pn = nG - p0 < CH ? nG - p0 : CH;
+                if (t0 < ntile) {
+#pragma unroll 2
+                    for (int pp = 0; pp < pn; ++pp) {
+                        const ACC fv = f[(p0 + pp) * 32 + lane];
+#pragma unroll
+                        for (int t = 0; t < RT; ++t) {
+                            if (t0 + t * nw < ntile) {
+                                ACC col[8];
+                                load_vec<T, ACC, 8>(buf + pp * ldn + (t0 + t * nw) * 8, col);
+#pragma unroll
+                                for (int u = 0; u < 8; ++u) acc[t][u] += col[u] * fv;
+                            }
+                        }
+                    }
+                }
+                __syncthreads();                       // the stage is free
+                if (tid == 0 && s + 2 < nstep) issue(s + 2);
+            }
+            if (!ok) break;
+            if (act) {
+#pragma unroll
+                for (int t = 0; t < RT; ++t)
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int q = (t0 + t * nw) * 8 + u;
+                        if (q < nG) W[(g0 + q) * K + lane] = acc[t][u];
+                    }
+            }
+        }
+        if (ok) {
+            // r_c += Psi^T f: a row per warp, eight entries per step
+            for (int k = warp; k < nc; k += nw) {
+                ACC s4[4] = {0, 0, 0, 0};
+                for (int q = 0; q < ldn; q += 8) {
+                    ACC row[8];
+                    load_vec<T, ACC, 8>(Ps + (size_t)k * ldn + q, row);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) s4[u & 3] += row[u] * f[(q + u) * 32 + lane];
+                }
+                if (act) atomicAdd(&B.rcv[(int64_t)rcs[k] * K + lane], to_f64((s4[0] + s4[1]) + (s4[2] + s4[3])));
+            }
+            return;
         }
     }
-    // r_c += Psi^T f (Psi^T[k * nG + q], staged whole)
-    const T *P = O.psit + L.offP[sub];
-    __syncthreads();
-    for (int e = tid; e < nc * nG; e += kNBT) buf[e] = P[e];
-    __syncthreads();
-    for (int k = warp; k < nc; k += 8) {
-        ACC s0 = 0;
-        for (int q = 0; q < nG; ++q) s0 += ld<T, ACC>(buf + (size_t)k * nG + q) * f[q * 32 + lane];
-        if (act) atomicAdd(&B.rcv[(int64_t)L.rc[L.offC[sub] + k] * K + lane], to_f64(s0));
+    // a wait gave up: flag it, and let the copies in flight land (bounded)
+    if (tid == 0) {
+        atomicExch(L.err, 1);
+        if (lay.N > 0) mbar_wait(&bars[2], 0);
+        const int s0 = waited > 0 ? waited - 1 : 0;          // in flight: the step that failed and the next
+        for (int s = s0; s < s0 + 2 && s < nstep; ++s) mbar_wait(&bars[s & 1], (unsigned)(s >> 1) & 1u);
     }
 }
 
-// (9) for K right-hand sides, Psi_i read from global memory (staged whole).
+// (9) for K right-hand sides: u_B += D_i (w_i + Psi_i u_c) on Gamma; clears
+// the r_B and r_c entries it consumed.  Tiles of eight rows per warp as above.
+__host__ __device__ inline size_t avg_head(const DevLevel &L, int esz) {
+    return (size_t)NRecLayout(L.max_nG > 0 ? L.max_nG : 1, L.max_nc > 0 ? L.max_nc : 1, esz).avg_bytes;
+}
+template <class T, class ACC> __host__ inline size_t avg_bg_smem(const DevLevel &L) {
+    return avg_head(L, (int)sizeof(T)) + al16(sizeof(ACC) * (size_t)(L.max_nc > 0 ? L.max_nc : 1) * 32) + 16;
+}
 template <class T, class ACC>
-__global__ void __launch_bounds__(kNBT) k_avg_bg(DevLevel L, BatchLevel B, int pidx, const int *skip) {
+__global__ void __launch_bounds__(32 * kNBW) k_avg_bg(DevLevel L, BatchLevel B, int pidx, const int *skip) {
     extern __shared__ __align__(16) unsigned char smem_ag[];
-    (void)pidx;
     if (skip && *skip) return;
-    const int sub = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int sub = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
     const int K = B.K;
     const bool act = lane < K;
     const int nG = L.nG[sub], nc = L.ncl[sub];
-    const size_t mg = L.max_nG > 0 ? L.max_nG : 1, mc = L.max_nc > 0 ? L.max_nc : 1;
-    ACC *uc = reinterpret_cast<ACC *>(smem_ag + al16(sizeof(ACC) * mg * 32));
-    T *buf = reinterpret_cast<T *>(smem_ag + al16(sizeof(ACC) * mg * 32) + al16(sizeof(ACC) * mc * 32));
-    const OpSet<T> &O = Ops<T>::get(L);
-    const int64_t g0 = L.offG[sub];
-    const int *rcs = L.rc + L.offC[sub];
-    for (int e = tid; e < nc * 32; e += kNBT) {
-        const int k = e >> 5, kk = e & 31;
-        uc[e] = kk < K ? from_f64<ACC>(B.ucv[(int64_t)rcs[k] * K + kk]) : (ACC)0;
+    const NRecLayout lay(nG, nc, (int)sizeof(T));
+    const size_t mh = avg_head(L, (int)sizeof(T));
+    unsigned char *head = smem_ag;
+    ACC *uc = reinterpret_cast<ACC *>(smem_ag + mh);
+    unsigned long long *bar = reinterpret_cast<unsigned long long *>(
+        smem_ag + mh + al16(sizeof(ACC) * (size_t)(L.max_nc > 0 ? L.max_nc : 1) * 32));
+    if (tid == 0) {
+        mbar_init(bar);
+        if (lay.avg_bytes > 0) bulk_load(head, L.nrec[pidx] + L.nrecOff[pidx][sub], (unsigned)lay.avg_bytes, bar);
     }
-    const T *P = O.psit + L.offP[sub];
-    for (int e = tid; e < nc * nG; e += kNBT) buf[e] = P[e];
+    // w of the first tile in flight while the record arrives
+    const int64_t g0 = L.offG[sub];
+    const ACC *W = reinterpret_cast<const ACC *>(B.w);
+    ACC v[8];
+    auto load_w = [&](int t) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int q = t * 8 + u;
+            v[u] = (act && q < nG) ? W[(g0 + q) * K + lane] : (ACC)0;
+        }
+    };
+    const int ntile = lay.ld >> 3;
+    load_w(warp);
     __syncthreads();
-    for (int q = warp; q < nG; q += 8) {
-        ACC v = act ? from_f64<ACC>(B.w[(g0 + q) * K + lane]) : (ACC)0;
-        for (int k = 0; k < nc; ++k) v += ld<T, ACC>(buf + (size_t)k * nG + q) * uc[k * 32 + lane];
+    const bool ok = lay.avg_bytes == 0 || mbar_wait(bar, 0);
+    if (!__syncthreads_and(ok)) {
+        if (tid == 0) {
+            atomicExch(L.err, 1);
+            mbar_wait(bar, 0);               // bounded: the copy lands before the block exits
+        }
+        return;
+    }
+    const T *Ps = reinterpret_cast<const T *>(head + lay.psi);
+    const T *wg = reinterpret_cast<const T *>(head + lay.wg);
+    const int *iG = reinterpret_cast<const int *>(head + lay.iG);
+    const int *rcs = reinterpret_cast<const int *>(head + lay.rc);
+    for (int k = warp; k < nc; k += nw)
+        uc[k * 32 + lane] = act ? from_f64<ACC>(B.ucv[(int64_t)rcs[k] * K + lane]) : (ACC)0;
+    __syncthreads();
+    for (int t = warp; t < ntile; t += nw) {
+        if (t != warp) load_w(t);
+#pragma unroll 2
+        for (int k = 0; k < nc; ++k) {
+            const ACC ucv = uc[k * 32 + lane];
+            ACC row[8];
+            load_vec<T, ACC, 8>(Ps + (size_t)k * lay.ld + t * 8, row);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] += row[u] * ucv;
+        }
         if (act) {
-            const int id = L.idxG[g0 + q];
-            const int64_t e = (int64_t)id * K + lane;
-            atomicAdd(&B.uB[e], to_f64(ld<T, ACC>(O.wg + g0 + q) * v));
-            B.rB[e] = 0.0;            // consumed by the substructure correction
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int q = t * 8 + u;
+                if (q >= nG) break;
+                const int64_t e = (int64_t)iG[q] * K + lane;
+                atomicAdd(&B.uB[e], to_f64(ld<T, ACC>(wg + q) * v[u]));
+                B.rB[e] = 0.0;            // consumed by the substructure correction
+            }
         }
     }
-    __syncthreads();
     if (act)
-        for (int k = warp; k < nc; k += 8) B.rcv[(int64_t)rcs[k] * K + lane] = 0.0;   // consumed
+        for (int k = warp; k < nc; k += nw) B.rcv[(int64_t)rcs[k] * K + lane] = 0.0;   // consumed
 }
 
 // (6)-(8) for K right-hand sides: f = D_i r_B on Gamma, w = N_i f,
@@ -1344,13 +1466,13 @@ __global__ void k_neu_b(DevLevel L, BatchLevel B, int pidx, const double *r, con
         const int nq = nG - q0 < 4 ? nG - q0 : 4;
         for (int pp = 0; pp < nG; ++pp) {
             const ACC fv = f[pp * 32 + lane];
-            const T *Nr = Ns + (size_t)pp * nG + q0;
+            const T *Nr = Ns + (size_t)pp * lay.ld + q0;
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (u < nq) s[u] += ld<T, ACC>(Nr + u) * fv;
         }
         if (act)
-            for (int u = 0; u < nq; ++u) B.w[(g0 + q0 + u) * K + lane] = to_f64(s[u]);
+            for (int u = 0; u < nq; ++u) reinterpret_cast<ACC *>(B.w)[(g0 + q0 + u) * K + lane] = s[u];
     }
     for (int k0 = 0; k0 < nc; k0 += 4) {
         ACC s[4] = {0, 0, 0, 0};
@@ -1359,7 +1481,7 @@ __global__ void k_neu_b(DevLevel L, BatchLevel B, int pidx, const double *r, con
             const ACC fv = f[q * 32 + lane];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (u < nk) s[u] += ld<T, ACC>(Ps + (size_t)(k0 + u) * nG + q) * fv;
+                if (u < nk) s[u] += ld<T, ACC>(Ps + (size_t)(k0 + u) * lay.ld + q) * fv;
         }
         if (act)
             for (int u = 0; u < nk; ++u) atomicAdd(&B.rcv[(int64_t)rcs[k0 + u] * K + lane], to_f64(s[u]));
@@ -1405,10 +1527,10 @@ __global__ void k_avg_b(DevLevel L, BatchLevel B, int pidx, const int *skip, uns
         const int nq = nG - q0 < 4 ? nG - q0 : 4;
         ACC v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = (act && u < nq) ? from_f64<ACC>(B.w[(g0 + q0 + u) * K + lane]) : (ACC)0;
+        for (int u = 0; u < 4; ++u) v[u] = (act && u < nq) ? reinterpret_cast<const ACC *>(B.w)[(g0 + q0 + u) * K + lane] : (ACC)0;
         for (int k = 0; k < nc; ++k) {
             const ACC ucv = uc[k * 32 + lane];
-            const T *Pr = Ps + (size_t)k * nG + q0;
+            const T *Pr = Ps + (size_t)k * lay.ld + q0;
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (u < nq) v[u] += ld<T, ACC>(Pr + u) * ucv;
@@ -1931,6 +2053,27 @@ void avg_b(const DevLevel &L, const BatchLevel &B, int prec, const int *skip, cu
                (unsigned)slice);
 }
 
+// Warps of a block: one per tile of eight rows of the largest interface, at
+// most kNBW; and tiles per warp, so that the interfaces of up to 192 (FP64:
+// 128) DOFs take one pass over N.
+int neu_warps(const DevLevel &L) {
+    const int t = (L.max_nG + 7) / 8;
+    return t < 1 ? 1 : (t > kNBW ? kNBW : t);
+}
+template <class T, class ACC>
+void neu_bg(const DevLevel &L, const BatchLevel &B, int prec, const double *r, const int *skip, cudaStream_t s) {
+    const int nw = neu_warps(L), rt = ((L.max_nG + 7) / 8 + nw - 1) / nw;
+    const size_t sm = neu_bg_smem<T, ACC>(L, B.chunk);
+    const int pi = pidx_b(prec);
+    if (rt <= 1) launch_plain(k_neu_bg<T, ACC, 1>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip);
+    else if (rt == 2 || sizeof(ACC) == 8) launch_plain(k_neu_bg<T, ACC, 2>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip);
+    else launch_plain(k_neu_bg<T, ACC, 3>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip);
+}
+template <class T, class ACC>
+void avg_bg(const DevLevel &L, const BatchLevel &B, int prec, const int *skip, cudaStream_t s) {
+    launch_plain(k_avg_bg<T, ACC>, L.nsub, 32 * neu_warps(L), avg_bg_smem<T, ACC>(L), s, L, B, pidx_b(prec), skip);
+}
+
 template <class T, class ACC> size_t dir_slice_b(const DevLevel &L) {
     if (L.bp == 8) return DirSmemB<T, ACC, 8>::bytes(L);
     if (L.bp == 16) return DirSmemB<T, ACC, 16>::bytes(L);
@@ -1988,7 +2131,7 @@ template <class T, class ACC> BatchRoute route_t(const DevLevel &L, int prec) {
     const int nw_max = ((L.max_b + 1) / 2 + 3) / 4;
     const bool stream = L.bk.n > 0 && L.bperm && nw_max <= kMaxBuckets &&
                         StreamSmemB::of<T, ACC>(L, 32 * nw_max).total <= kSmemMaxB;
-    const bool bg = neu_bg_smem<T, ACC>(L) <= kSmemMaxB;
+    const bool bg = neu_bg_smem<T, ACC>(L) <= kSmemMaxB && avg_bg_smem<T, ACC>(L) <= kSmemMaxB;
     R.dir_stream = !R.dir_staged && stream;
     R.stream_fits = stream;
     R.bg_fits = bg;
@@ -2129,7 +2272,7 @@ void pre_b(const DevLevel &L, const BatchLevel &B, int prec, const double *r, co
     else dir_bs<T, ACC>(L, B, false, r, nullptr, skip, nullptr, s);
     if (ev) cudaEventRecord(ev[1], s);
     if (R.neu_staged) neu_b<T, ACC>(L, B, prec, r, skip, s);
-    else launch_plain(k_neu_bg<T, ACC>, L.nsub, kNBT, neu_bg_smem<T, ACC>(L, B.chunk), s, L, B, pidx_b(prec), r, skip);
+    else neu_bg<T, ACC>(L, B, prec, r, skip, s);
     if (ev) cudaEventRecord(ev[2], s);
 }
 
@@ -2139,7 +2282,7 @@ void post_b(const DevLevel &L, const BatchLevel &B, int prec, const double *r, d
     const BatchRoute R = route_t<T, ACC>(L, prec);
     if (ev) cudaEventRecord(ev[0], s);
     if (R.avg_staged) avg_b<T, ACC>(L, B, prec, skip, s);
-    else launch_plain(k_avg_bg<T, ACC>, L.nsub, kNBT, neu_bg_smem<T, ACC>(L, B.chunk), s, L, B, pidx_b(prec), skip);
+    else avg_bg<T, ACC>(L, B, prec, skip, s);
     if (ev) cudaEventRecord(ev[1], s);
     if (R.post_tc) tc_dir_b(L, B, prec, true, r, z, skip, rz, s);
     else if (R.dir_lane) dir_ls<T, ACC>(L, B, true, r, z, skip, s, rz);
@@ -2249,10 +2392,7 @@ template <class T, class ACC> void tune_t(const DevLevel &L, BatchLevel &B, int 
         for (int c : cand) {
             if (neu_bg_smem<T, ACC>(L, c) > kSmemMaxB) continue;
             B.chunk = c;
-            const double t = time3(s, [&] {
-                launch_plain(k_neu_bg<T, ACC>, L.nsub, kNBT, neu_bg_smem<T, ACC>(L, c), s, L, B, pidx_b(prec), r,
-                             (const int *)nullptr);
-            });
+            const double t = time3(s, [&] { neu_bg<T, ACC>(L, B, prec, r, (const int *)nullptr, s); });
             if (t < best) best = t, pick = c;
         }
         B.chunk = pick;
@@ -2315,8 +2455,12 @@ void prepare_batch_kernels() {
     BDDC_DIR_BS(float, float, false) BDDC_DIR_BS(float, float, true)
     BDDC_DIR_BS(__nv_bfloat16, float, false) BDDC_DIR_BS(__nv_bfloat16, float, true)
 #undef BDDC_DIR_BS
-    BDDC_SMEM_ATTR_B((k_neu_bg<double, double>)); BDDC_SMEM_ATTR_B((k_neu_bg<float, float>));
-    BDDC_SMEM_ATTR_B((k_neu_bg<__nv_bfloat16, float>));
+#define BDDC_NEU_BG(T, A)                                       \
+    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 1>));                      \
+    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 2>));                      \
+    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 3>));
+    BDDC_NEU_BG(double, double) BDDC_NEU_BG(float, float) BDDC_NEU_BG(__nv_bfloat16, float)
+#undef BDDC_NEU_BG
     BDDC_SMEM_ATTR_B((k_avg_bg<double, double>)); BDDC_SMEM_ATTR_B((k_avg_bg<float, float>));
     BDDC_SMEM_ATTR_B((k_avg_bg<__nv_bfloat16, float>));
     BDDC_SMEM_ATTR_B((k_avg_b<double, double>)); BDDC_SMEM_ATTR_B((k_avg_b<float, float>));

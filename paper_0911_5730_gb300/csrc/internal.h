@@ -182,18 +182,23 @@ struct IRecLayout {
         bytes = ow + a16(8LL * nown);
     }
 };
+// ld: row stride of Psi^T and N, nG rounded up to eight entries (zero filled),
+// so that eight consecutive entries of a row are one or two aligned vector
+// reads in every precision.
 struct NRecLayout {
     int64_t psi, wg, iG, rc, gG, N, avg_bytes, bytes;
+    int ld;
     __host__ __device__ NRecLayout(int nG, int nc, int esz) {
         auto a16 = [](int64_t v) { return (v + 15) & ~int64_t(15); };
+        ld = (nG + 7) & ~7;
         psi = 0;
-        wg = a16((int64_t)esz * nc * nG);
+        wg = a16((int64_t)esz * nc * ld);
         iG = wg + a16((int64_t)esz * nG);
         rc = iG + a16(4LL * nG);
         gG = rc + a16(4LL * nc);
         N = gG + a16(4LL * nG);
         avg_bytes = gG;
-        bytes = N + a16((int64_t)esz * nG * nG);
+        bytes = N + a16((int64_t)esz * nG * ld);
     }
 };
 
