@@ -870,7 +870,10 @@ __global__ void k_build_nrec(DevLevel D, OpSet<T> O, unsigned char *rec, const i
         gG[q] = D.ifaceDof[D.idxG[D.offG[sub] + q]];
     }
     for (int k = threadIdx.x; k < nc; k += blockDim.x) rcs[k] = D.rc[D.offC[sub] + k];
-    for (int k = threadIdx.x; k < nG * nG; k += blockDim.x) N[k] = O.nmat[D.offN[sub] + k];
+    for (int k = threadIdx.x; k < nG * ld; k += blockDim.x) {
+        const int row = k / ld, q = k - row * ld;
+        N[k] = q < nG ? O.nmat[D.offN[sub] + (int64_t)row * nG + q] : T(0.0f);
+    }
 }
 
 // y = A x, A dense symmetric n x n row-major with leading dimension ld (a
