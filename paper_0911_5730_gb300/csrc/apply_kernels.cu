@@ -495,17 +495,26 @@ template <int LPR, class ACC> __device__ __forceinline__ ACC lpr_sum(ACC v) {
 // ----------------------------------------------------------------------------
 constexpr int kUI = 8, kUG = 4, kUC = 8, kUO = 4;   // record entries per lane
 constexpr int kChunks = 4;                          // bulk copies per factor
+// Where a wave of substructures does not fit the SMs with whole factors (FP64
+// blocks of 16 rows: 61 KB each, three warps per SM and three waves on the
+// 512^2 channel problem), the factor streams through a ring of kDWRing blocks
+// instead (block j in slot j mod kDWRing, refilled once used; the backward
+// sweep starts from the blocks left in the ring).
+constexpr int kDWRing = 6;
 
-template <class T, class ACC, int BP> struct DirSlice {
+template <class T, class ACC, int BP, int RING> struct DirSlice {
     // every warp's slice starts 16-byte aligned: bulk-copy destinations and
     // mbarriers inside it rely on that
+    __host__ __device__ static size_t fac(const DevLevel &L) {
+        return al16(sizeof(T) * (RING ? (size_t)RING * 2 * BP * BP : (size_t)L.max_fac));
+    }
     static size_t bytes(const DevLevel &L) {
-        return al16(sizeof(T) * (size_t)L.max_fac + al16(sizeof(ACC) * (size_t)L.max_m * BP) +
-                    al16(sizeof(ACC) * (size_t)L.max_nG) + 8 * kChunks + 16);
+        return al16(fac(L) + al16(sizeof(ACC) * (size_t)L.max_m * BP) + al16(sizeof(ACC) * (size_t)L.max_nG) +
+                    8 * (RING ? RING : kChunks) + 16);
     }
 };
 
-template <class T, class ACC, int BP, bool POST>
+template <class T, class ACC, int BP, bool POST, int RING>
 __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip, unsigned slice,
                         RzArgs rz) {
     constexpr int LPR = 32 / BP;
@@ -516,7 +525,7 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     const int sub = blockIdx.x * (blockDim.x >> 5) + warp;
     if (sub >= L.nsub) { pdl_wait(); return; }
     unsigned char *p = smem_w + (size_t)warp * slice;
-    T *fac = reinterpret_cast<T *>(p);      p += al16(sizeof(T) * (size_t)L.max_fac);
+    T *fac = reinterpret_cast<T *>(p);      p += DirSlice<T, ACC, BP, RING>::fac(L);
     ACC *x = reinterpret_cast<ACC *>(p);    p += al16(sizeof(ACC) * (size_t)L.max_m * BP);
     ACC *vG = reinterpret_cast<ACC *>(p);   p += al16(sizeof(ACC) * (size_t)L.max_nG);
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(p);
@@ -524,18 +533,44 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     const int nI = L.nI[sub], nG = L.nG[sub], m = L.nblk[sub];
     const int ncoo = L.ncoo[sub], nown = L.nown[sub];
     const T *F = Ops<T>::get(L).dir + L.offF[sub];
-    const int nch = m < kChunks ? m : kChunks;
+    // copies in flight: whole chunks of the factor, or the ring's first blocks
+    const int nch = RING ? (m < RING ? m : RING) : (m < kChunks ? m : kChunks);
     if (lane == 0)
         for (int c = 0; c < nch; ++c) mbar_init(&bars[c]);
     __syncwarp();
+    constexpr unsigned blk_bytes = 2u * BB * (unsigned)sizeof(T);
     if (lane == 0) {
         for (int c = 0; c < nch; ++c) {
-            const int b0 = c * m / nch, b1 = (c + 1) * m / nch;
-            const unsigned bytes = (unsigned)((size_t)(b1 - b0) * 2 * BB * sizeof(T));
+            const int b0 = RING ? c : c * m / nch, b1 = RING ? c + 1 : (c + 1) * m / nch;
+            const unsigned bytes = (unsigned)(b1 - b0) * blk_bytes;
             mbar_expect(&bars[c], bytes);
             bulk_copy(fac + (size_t)b0 * 2 * BB, F + (size_t)b0 * 2 * BB, bytes, &bars[c]);
         }
     }
+    auto blk = [&](int j) -> const T * { return fac + (size_t)(RING ? j % (RING ? RING : 1) : j) * 2 * BB; };
+    unsigned ph = 0, pend = RING ? (1u << nch) - 1u : 0u;   // ring: parity of a slot's next copy, copies in flight
+    auto wait_slot = [&](int s) -> bool {
+        const bool ok = warp_wait_copy(&bars[s], L.err, lane, (ph >> s) & 1u);
+        ph ^= 1u << s;
+        pend &= ~(1u << s);
+        return ok;
+    };
+    auto refill = [&](int s, int j) {                       // every lane is done with slot s
+        __syncwarp();
+        if (lane == 0) {
+            mbar_expect(&bars[s], blk_bytes);
+            bulk_copy(fac + (size_t)s * 2 * BB, F + (size_t)j * 2 * BB, blk_bytes, &bars[s]);
+        }
+        pend |= 1u << s;
+    };
+    auto drain = [&](int from) {                            // bounded: copies in flight land
+        if (RING) {
+            for (int s = 0; s < nch; ++s)
+                if ((pend >> s) & 1u) mbar_wait(&bars[s], (ph >> s) & 1u);
+        } else {
+            for (int c = from; c < nch; ++c) mbar_wait(&bars[c], 0);
+        }
+    };
     // index record -> registers (coalesced loads, independent of the copies)
     const IRecLayout lay(nI, nG, ncoo, nown);
     const unsigned char *rec = L.irec + L.irecOff[sub];
@@ -569,7 +604,7 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     pdl_wait();
     pdl_trigger();
     if (skip && *skip) {
-        for (int c = 0; c < nch; ++c) mbar_wait(&bars[c], 0);   // bounded: copies land first
+        drain(0);
         return;
     }
     // right-hand side (and u_B on Gamma for the post-correction)
@@ -606,12 +641,16 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     bool ok = true;
     ACC xprev = 0;
     for (int j = 0; j < m; ++j) {
-        while (cw < nch && cw * m / nch <= j) {
-            if (!warp_wait_copy(&bars[cw], L.err, lane)) { ok = false; break; }
-            ++cw;
+        if (RING) {
+            ok = wait_slot(j % (RING ? RING : 1));
+        } else {
+            while (cw < nch && cw * m / nch <= j) {
+                if (!warp_wait_copy(&bars[cw], L.err, lane)) { ok = false; break; }
+                ++cw;
+            }
         }
         if (!ok) break;
-        const T *Li = fac + (size_t)j * 2 * BB;
+        const T *Li = blk(j);
         const T *Ls = Li + BB;
         // t = b_j - L_{j,j-1} x_{j-1}
         ACC a0 = 0, a1 = 0;
@@ -634,18 +673,23 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
         }
         xprev = lpr_sum<LPR>(a0 + a1);
         x[j * BP + rr] = xprev;
+        if (RING && j + RING < m) refill(j % (RING ? RING : 1), j + RING);
     }
     if (!ok) {
-        for (int c = cw; c < nch; ++c) mbar_wait(&bars[c], 0);   // bounded: let copies land
+        drain(cw);
         return;
     }
     ACC znext = 0;
     for (int j = m - 1; j >= 0; --j) {
-        const T *Li = fac + (size_t)j * 2 * BB;
+        if (RING && j < m - RING && !wait_slot(j % (RING ? RING : 1))) {
+            drain(0);
+            return;
+        }
+        const T *Li = blk(j);
         // t = y_j - L_{j+1,j}^T z_{j+1}
         ACC a0 = 0, a1 = 0;
         if (j < m - 1) {
-            const T *Ls1 = fac + (size_t)(j + 1) * 2 * BB + BB;
+            const T *Ls1 = blk(j + 1) + BB;
 #pragma unroll
             for (int i = 0; i < NC; i += 2) {
                 const int c0 = h + LPR * i, c1 = c0 + LPR;
@@ -664,6 +708,8 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
         }
         znext = lpr_sum<LPR>(a0 + a1);
         x[j * BP + rr] = znext;
+        // block j + 1 is used up: its slot takes block j + 1 - RING
+        if (RING && j + 1 < m && j + 1 - RING >= 0) refill((j + 1) % (RING ? RING : 1), j + 1 - RING);
     }
     __syncwarp();
     if (!POST) {
@@ -1382,17 +1428,36 @@ int warps_per_block(int nsub, size_t slice) {
     return w < 1 ? 1 : w;
 }
 
-template <class T, class ACC, int BP>
-void dir_launch(const DevLevel &L, bool post, const double *r, double *z, const int *skip,
-                cudaStream_t s, const RzArgs *rz) {
-    const size_t slice = DirSlice<T, ACC, BP>::bytes(L);
+template <class T, class ACC, int BP, int RING>
+void dir_launch_r(const DevLevel &L, bool post, const double *r, double *z, const int *skip,
+                  cudaStream_t s, const RzArgs *rz) {
+    const size_t slice = DirSlice<T, ACC, BP, RING>::bytes(L);
     const int wpc = warps_per_block(L.nsub, slice);
     const size_t sm = slice * wpc;
     const int grid = (L.nsub + wpc - 1) / wpc;
     const RzArgs none{nullptr, nullptr, nullptr, nullptr};
-    if (!post) launch_pdl(k_dir_w<T, ACC, BP, false>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice, none);
-    else launch_pdl(k_dir_w<T, ACC, BP, true>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice,
+    if (!post) launch_pdl(k_dir_w<T, ACC, BP, false, RING>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice, none);
+    else launch_pdl(k_dir_w<T, ACC, BP, true, RING>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice,
                     rz ? *rz : none);
+}
+// The ring where whole factors would take more waves than it does: with one
+// wave either way, the whole factor saves the second read of its blocks.
+// FP64 apply of the 512^2 channel problem 265 -> 156 us (three waves of three
+// warps per SM, now one of seven), its reduced solve 6.57 -> 4.26 ms.
+template <class T, class ACC, int BP>
+void dir_launch(const DevLevel &L, bool post, const double *r, double *z, const int *skip,
+                cudaStream_t s, const RzArgs *rz) {
+    auto waves = [&](size_t slice) {
+        const int64_t per = (int64_t)num_sms() * (int64_t)(kSmemMax / slice);
+        return per > 0 ? (L.nsub + per - 1) / per : (int64_t)1 << 30;
+    };
+    if constexpr (sizeof(T) == 8) {
+        if (waves(DirSlice<T, ACC, BP, kDWRing>::bytes(L)) < waves(DirSlice<T, ACC, BP, 0>::bytes(L))) {
+            dir_launch_r<T, ACC, BP, kDWRing>(L, post, r, z, skip, s, rz);
+            return;
+        }
+    }
+    dir_launch_r<T, ACC, BP, 0>(L, post, r, z, skip, s, rz);
 }
 
 template <class T, class ACC>
@@ -1445,34 +1510,24 @@ bool warp_path(const DevLevel &L, int prec) {
 void prepare_apply_kernels() {
     const int big = (int)kSmemMax;
 #define BDDC_SMEM_ATTR(k) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, big)
+#define BDDC_DIR_W(T, A, BP, R)                          \
+    BDDC_SMEM_ATTR((k_dir_w<T, A, BP, false, R>));       \
+    BDDC_SMEM_ATTR((k_dir_w<T, A, BP, true, R>));
+    BDDC_DIR_W(double, double, 8, 0) BDDC_DIR_W(double, double, 16, 0) BDDC_DIR_W(double, double, 32, 0)
+    BDDC_DIR_W(double, double, 8, kDWRing) BDDC_DIR_W(double, double, 16, kDWRing) BDDC_DIR_W(double, double, 32, kDWRing)
+    BDDC_DIR_W(float, float, 8, 0) BDDC_DIR_W(float, float, 16, 0) BDDC_DIR_W(float, float, 32, 0)
+    BDDC_DIR_W(__nv_bfloat16, float, 8, 0) BDDC_DIR_W(__nv_bfloat16, float, 16, 0) BDDC_DIR_W(__nv_bfloat16, float, 32, 0)
+#undef BDDC_DIR_W
     BDDC_SMEM_ATTR((k_dir_s<double, double, false>));
     BDDC_SMEM_ATTR((k_dir_s<double, double, true>));
     BDDC_SMEM_ATTR((k_dir_s<float, float, false>));
     BDDC_SMEM_ATTR((k_dir_s<float, float, true>));
     BDDC_SMEM_ATTR((k_dir_s<__nv_bfloat16, float, false>));
     BDDC_SMEM_ATTR((k_dir_s<__nv_bfloat16, float, true>));
-    BDDC_SMEM_ATTR((k_dir_w<double, double, 8, false>));
-    BDDC_SMEM_ATTR((k_dir_w<double, double, 8, true>));
-    BDDC_SMEM_ATTR((k_dir_w<double, double, 16, false>));
-    BDDC_SMEM_ATTR((k_dir_w<double, double, 16, true>));
-    BDDC_SMEM_ATTR((k_dir_w<double, double, 32, false>));
-    BDDC_SMEM_ATTR((k_dir_w<double, double, 32, true>));
     BDDC_SMEM_ATTR((k_neumann_r<double, double>));
     BDDC_SMEM_ATTR((k_average_r<double, double>));
-    BDDC_SMEM_ATTR((k_dir_w<float, float, 8, false>));
-    BDDC_SMEM_ATTR((k_dir_w<float, float, 8, true>));
-    BDDC_SMEM_ATTR((k_dir_w<float, float, 16, false>));
-    BDDC_SMEM_ATTR((k_dir_w<float, float, 16, true>));
-    BDDC_SMEM_ATTR((k_dir_w<float, float, 32, false>));
-    BDDC_SMEM_ATTR((k_dir_w<float, float, 32, true>));
     BDDC_SMEM_ATTR((k_neumann_r<float, float>));
     BDDC_SMEM_ATTR((k_average_r<float, float>));
-    BDDC_SMEM_ATTR((k_dir_w<__nv_bfloat16, float, 8, false>));
-    BDDC_SMEM_ATTR((k_dir_w<__nv_bfloat16, float, 8, true>));
-    BDDC_SMEM_ATTR((k_dir_w<__nv_bfloat16, float, 16, false>));
-    BDDC_SMEM_ATTR((k_dir_w<__nv_bfloat16, float, 16, true>));
-    BDDC_SMEM_ATTR((k_dir_w<__nv_bfloat16, float, 32, false>));
-    BDDC_SMEM_ATTR((k_dir_w<__nv_bfloat16, float, 32, true>));
     BDDC_SMEM_ATTR((k_neumann_r<__nv_bfloat16, float>));
     BDDC_SMEM_ATTR((k_average_r<__nv_bfloat16, float>));
     // the generic kernels: interior vectors and Gamma vectors of any size
