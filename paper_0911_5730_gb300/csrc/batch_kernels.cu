@@ -1821,6 +1821,134 @@ __global__ void k_b_dir_spmv(int nx, int K, const double *__restrict__ w, const 
         }, NoPost{});
 }
 
+// The same first half for more than kMarchMinK right-hand sides, a lane per
+// right-hand side and no tile: each warp marches up a strip of MW columns with
+// three rows of p_new in registers, so nothing meets at a barrier, and the
+// strips are cut into as many equal segments as there are resident warps (one
+// wave).  The FP64 pipe bounds it: per node 9 products, 1 for the dot product
+// and (MW + 2) / MW (and two rows per segment) for p_new, 11.4 in all, as with
+// the tiles; those left a last wave of blocks partly filled and met at the
+// end of their load phases.  Every weight read is in range (a missing
+// neighbour's p_new is zero and reads a finite weight), so the products need
+// no predicates, and their order is the tile kernel's: q is the same bit for
+// bit.
+// 32 right-hand sides: the 1024^2 three-level solve (46 iterations) 101 ->
+// 92 ms, the 512^2 FP64 solve 75.6 -> 72.5 ms, with the update kernel's loads
+// in flight.
+constexpr int MW = 8, kMarchT = 256, kMarchPerSm = 2, kMarchMinK = 16;
+__global__ void __launch_bounds__(kMarchT, kMarchPerSm)
+k_b_dir_march(int nx, int K, const double *__restrict__ w, const double *__restrict__ z, double *p0, double *p1,
+              double *__restrict__ q, double *part, unsigned *counter, BatchScalars *sc, double *alphas, int strips,
+              int rows) {
+    __shared__ double red[kMarchT / 32][32];
+    __shared__ bool last;
+    if (sc->all_done) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n1 = nx - 1;
+    const int64_t n = (int64_t)n1 * n1;
+    const bool odd = sc->step & 1;
+    const double *__restrict__ po = odd ? p1 : p0;
+    double *__restrict__ pn = odd ? p0 : p1;
+    const bool act = lane < K;
+    const int k = act ? lane : 0;
+    const bool live = act && !sc->done[k] && !sc->hold[k];
+    const double bt = sc->beta[k];
+    const int unit = blockIdx.x * (kMarchT / 32) + warp;
+    const int i0 = (unit % strips) * MW, j0 = (unit / strips) * rows;
+    const int j1 = min(n1, j0 + rows);
+    double s = 0.0;
+    if (j0 < n1) {
+        double A[MW + 2], B[MW + 2];
+        auto fetch = [&](int j) {          // p_old and z of row j, zero outside the domain
+#pragma unroll
+            for (int c = 0; c < MW + 2; ++c) {
+                const int i = i0 + c - 1;
+                const bool in = act && j >= 0 && j < n1 && i >= 0 && i < n1;
+                const int64_t g = ((int64_t)j * n1 + i) * K + k;
+                A[c] = in ? po[g] : 0.0;
+                B[c] = in ? z[g] : 0.0;
+            }
+        };
+        auto form = [&](double (&R)[MW + 2]) {
+#pragma unroll
+            for (int c = 0; c < MW + 2; ++c) R[c] = fma(bt, A[c], B[c]);
+        };
+        // row j (C) from the rows below and above (S, N); forms N and fetches row j + 2
+        auto step = [&](int j, const double (&S)[MW + 2], const double (&C)[MW + 2], double (&N)[MW + 2]) {
+            form(N);
+            if (j + 1 < j1) fetch(j + 2);
+            const double *wr = w + (int64_t)j * n1 + i0;
+#pragma unroll
+            for (int c = 0; c < MW; ++c) {
+                if (i0 + c >= n1) break;
+                const double *wc = wr + c;
+                double v = __ldg(wc) * C[c + 1];
+                v = fma(__ldg(wc + n), C[c + 2], v);                    // E
+                v = fma(__ldg(wc + 2 * n), N[c + 1], v);                // N
+                v = fma(__ldg(wc + 3 * n), N[c + 2], v);                // NE
+                v = fma(__ldg(wc + 4 * n), N[c], v);                    // NW
+                v = fma(__ldg(wc + n - 1), C[c], v);                    // W
+                v = fma(__ldg(wc + 2 * n - n1), S[c + 1], v);           // S
+                v = fma(__ldg(wc + 3 * n - n1 - 1), S[c], v);           // SW
+                v = fma(__ldg(wc + 4 * n - n1 + 1), S[c + 2], v);       // SE
+                const int64_t e = ((int64_t)j * n1 + i0 + c) * K + k;
+                if (live) pn[e] = C[c + 1];
+                if (act) q[e] = v;
+                s = fma(v, C[c + 1], s);
+            }
+        };
+        double P0[MW + 2], P1[MW + 2], P2[MW + 2];
+        fetch(j0 - 1);
+        form(P0);
+        fetch(j0);
+        form(P1);
+        fetch(j0 + 1);
+        for (int j = j0; j < j1; j += 3) {
+            step(j, P0, P1, P2);
+            if (j + 1 < j1) step(j + 1, P1, P2, P0);
+            if (j + 2 < j1) step(j + 2, P2, P0, P1);
+        }
+    }
+    // block partials, added over the blocks in a fixed order by the last block
+    red[warp][lane] = s;
+    __syncthreads();
+    constexpr int NWM = kMarchT / 32;
+    if (warp == 0 && act) {
+        double t = 0.0;
+#pragma unroll
+        for (int u = 0; u < NWM; ++u) t += red[u][lane];
+        part[(int64_t)blockIdx.x * K + lane] = t;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double t = 0.0;
+    if (act)
+        for (int b = warp; b < (int)gridDim.x; b += 8 * NWM) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = b + u * NWM < (int)gridDim.x ? __ldcg(&part[(int64_t)(b + u * NWM) * K + lane]) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t += v[u];
+        }
+    red[warp][lane] = t;
+    __syncthreads();
+    if (warp == 0 && act) {
+        double tot = 0.0;
+#pragma unroll
+        for (int u = 0; u < NWM; ++u) tot += red[u][lane];
+        if (!sc->done[lane] && !sc->hold[lane]) {
+            sc->pq[lane] = tot;
+            sc->alpha[lane] = sc->rho[lane] / tot;
+            alphas[(int64_t)sc->it[lane] * K + lane] = sc->alpha[lane];
+        }
+    }
+    if (threadIdx.x == 0) *counter = 0u;
+}
+
 // x += alpha p; r -= alpha q; rr_k; convergence; it_k += 1
 __global__ void k_b_update(int64_t nK, int K, double *__restrict__ x, double *__restrict__ r,
                            const double *p0, const double *p1, const double *__restrict__ q,
@@ -1834,7 +1962,25 @@ __global__ void k_b_update(int64_t nK, int K, double *__restrict__ x, double *__
     const double a = sc->alpha[k];
     double s = 0.0;
     if (live) {
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nK; e += (int64_t)gridDim.x * blockDim.x) {
+        // four entries per round: sixteen independent loads in flight
+        const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+        int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        for (; e + 3 * stride < nK; e += 4 * stride) {
+            double pv[4], qv[4], xv[4], rv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                pv[u] = p[e + u * stride]; qv[u] = q[e + u * stride];
+                xv[u] = x[e + u * stride]; rv[u] = r[e + u * stride];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                x[e + u * stride] = fma(a, pv[u], xv[u]);
+                const double ri = fma(-a, qv[u], rv[u]);
+                r[e + u * stride] = ri;
+                s = fma(ri, ri, s);
+            }
+        }
+        for (; e < nK; e += stride) {
             x[e] = fma(a, p[e], x[e]);
             const double ri = fma(-a, q[e], r[e]);
             r[e] = ri;
@@ -2556,9 +2702,26 @@ template <int TX, int TY> int tile_blocks(int nx) {
     const int n1 = nx - 1;
     return ((n1 + TX - 1) / TX) * ((n1 + TY - 1) / TY);
 }
-int launch_b_dir_spmv_blocks(int nx) {   // the most blocks any tile variant launches
-    return std::max(std::max(tile_blocks<16, 8>(nx), tile_blocks<32, 4>(nx)),
-                    std::max(tile_blocks<32, 8>(nx), tile_blocks<8, 16>(nx)));
+// Strips, rows per segment and blocks of k_b_dir_march: the segments that the
+// resident warps can take at once, at least kMarchRows rows each.
+struct MarchShape { int strips, rows, blocks; };
+MarchShape march_shape(int nx) {
+    constexpr int kMarchRows = 4;
+    const int n1 = nx - 1, warps = kMarchT / 32;
+    MarchShape m;
+    m.strips = (n1 + MW - 1) / MW;
+    int segs = kMarchPerSm * num_sms_b() * warps / m.strips;
+    const int most = (n1 + kMarchRows - 1) / kMarchRows;
+    segs = segs < 1 ? 1 : (segs > most ? most : segs);
+    m.rows = (n1 + segs - 1) / segs;
+    segs = (n1 + m.rows - 1) / m.rows;
+    m.blocks = (m.strips * segs + warps - 1) / warps;
+    return m;
+}
+int launch_b_dir_spmv_blocks(int nx) {   // the most blocks any variant launches
+    return std::max(std::max(std::max(tile_blocks<16, 8>(nx), tile_blocks<32, 4>(nx)),
+                             std::max(tile_blocks<32, 8>(nx), tile_blocks<8, 16>(nx))),
+                    march_shape(nx).blocks);
 }
 template <int TX, int TY>
 void dir_spmv_v(int nx, int K, const double *w, const double *z, double *p0, double *p1, double *q,
@@ -2569,6 +2732,12 @@ void dir_spmv_v(int nx, int K, const double *w, const double *z, double *p0, dou
 void launch_b_dir_spmv(int nx, int K, const double *w, const double *z, double *p0, double *p1,
                        double *q, double *part, unsigned *counter, BatchScalars *sc, double *alphas,
                        cudaStream_t s, int variant) {
+    if (K > kMarchMinK && variant >= 0) {
+        const MarchShape m = march_shape(nx);
+        launch_plain(k_b_dir_march, m.blocks, kMarchT, 0, s, nx, K, w, z, p0, p1, q, part, counter, sc, alphas,
+                     m.strips, m.rows);
+        return;
+    }
     switch (variant) {
     case 1: dir_spmv_v<32, 4>(nx, K, w, z, p0, p1, q, part, counter, sc, alphas, s); break;
     case 2: dir_spmv_v<32, 8>(nx, K, w, z, p0, p1, q, part, counter, sc, alphas, s); break;
