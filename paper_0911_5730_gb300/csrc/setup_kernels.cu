@@ -41,7 +41,7 @@ __device__ bool cta_cholesky(double *A, int n, int lda) {
         const int npairs = m * (m + 1) / 2;
         for (int q = threadIdx.x; q < npairs; q += blockDim.x) {
             // unrank q -> (ii >= kk) in the trailing lower triangle
-            int ii = (int)((sqrt(8.0 * q + 1.0) - 1.0) * 0.5);
+            int ii = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);   // corrected below
             while ((ii + 1) * (ii + 2) / 2 <= q) ++ii;
             while (ii * (ii + 1) / 2 > q) --ii;
             const int kk = q - ii * (ii + 1) / 2;
@@ -51,6 +51,27 @@ __device__ bool cta_cholesky(double *A, int n, int lda) {
         __syncthreads();
     }
     return true;
+}
+
+// The same for a matrix that may be semidefinite to rounding: a pivot that is
+// not positive gives a zero column.
+__device__ void cta_cholesky_semi(double *A, int n, int lda) {
+    for (int j = 0; j < n; ++j) {
+        __syncthreads();
+        const double d = A[(int64_t)j * lda + j];
+        const double l = d > 0.0 ? sqrt(d) : 0.0;
+        __syncthreads();
+        if (threadIdx.x == 0) A[(int64_t)j * lda + j] = l;
+        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x)
+            A[(int64_t)i * lda + j] = l > 0.0 ? A[(int64_t)i * lda + j] / l : 0.0;
+        __syncthreads();
+        const int m = n - j - 1;
+        for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
+            const int i = j + 1 + q / m, k = j + 1 + q % m;
+            if (k <= i) A[(int64_t)i * lda + k] -= A[(int64_t)i * lda + j] * A[(int64_t)k * lda + j];
+        }
+    }
+    __syncthreads();
 }
 
 // Solve L X = B (L lower, n x n), B n x ncols in place; thread per column.
@@ -158,7 +179,7 @@ __global__ void k_band_cholesky(SetupLevel S, int *err) {
         __syncthreads();
         for (int q = threadIdx.x; q < npairs; q += blockDim.x) {
             // pairs 1 <= d1 <= d2 <= bw
-            int d2 = (int)((sqrt(8.0 * q + 1.0) - 1.0) * 0.5);
+            int d2 = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);   // corrected below
             while ((d2 + 1) * (d2 + 2) / 2 <= q) ++d2;
             while (d2 * (d2 + 1) / 2 > q) --d2;
             const int d1 = q - d2 * (d2 + 1) / 2;   // 0..d2
@@ -322,10 +343,11 @@ __device__ void schur_onto(const double *Sfull, int nG, const int *posK, int nk,
 }
 
 // Parallel cyclic Jacobi (round-robin ordering) on a symmetric n x n matrix
-// held in A (row-major, n even after padding).  V receives the eigenvectors.
-__device__ void cta_jacobi(double *A, double *V, int n, double *cs, int *perm) {
+// held in A (row-major, n even after padding), in shared memory where it fits.
+// V receives the eigenvectors.  Step t pairs positions i and n - 1 - i of the
+// order in which index 0 stays and the others have moved t places round.
+__device__ void cta_jacobi(double *A, double *V, int n, double *cs) {
     for (int q = threadIdx.x; q < n * n; q += blockDim.x) V[q] = (q / n == q % n) ? 1.0 : 0.0;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) perm[q] = q;
     __syncthreads();
     __shared__ double offn, totn;
     const int half = n / 2;
@@ -344,9 +366,13 @@ __device__ void cta_jacobi(double *A, double *V, int n, double *cs, int *perm) {
         if (!(offn > 1e-30 * totn) || totn == 0.0) break;
         __syncthreads();
         for (int step = 0; step < n - 1; ++step) {
-            // pairs (perm[i], perm[n-1-i]) for i < half
+            auto at = [&](int pos) {
+                int k = pos - 1 - step;
+                if (k < 0) k += n - 1;
+                return pos == 0 ? 0 : 1 + k;
+            };
             for (int i = threadIdx.x; i < half; i += blockDim.x) {
-                int p = perm[i], q = perm[n - 1 - i];
+                int p = at(i), q = at(n - 1 - i);
                 if (p > q) { int tmp = p; p = q; q = tmp; }
                 const double apq = A[(int64_t)p * n + q];
                 double c = 1.0, s = 0.0;
@@ -384,19 +410,13 @@ __device__ void cta_jacobi(double *A, double *V, int n, double *cs, int *perm) {
                 A[(int64_t)q * n + k] = s * apk + c * aqk;
             }
             __syncthreads();
-            // round-robin rotation of positions 1..n-1
-            if (threadIdx.x == 0) {
-                const int last = perm[n - 1];
-                for (int i = n - 1; i > 1; --i) perm[i] = perm[i - 1];
-                perm[1] = last;
-            }
-            __syncthreads();
         }
     }
 }
 
-__global__ void k_edge_eig(SetupLevel S, EdgeBatch E, double tau, double *work,
-                           int64_t work_stride, int *err) {
+__global__ void __launch_bounds__(128) k_edge_eig(SetupLevel S, EdgeBatch E, double tau, double *work,
+                                                  int64_t work_stride, bool jacobi_smem, int *err) {
+    extern __shared__ double edge_sm[];
     const int e = blockIdx.x;
     const int s = E.s[e], t = E.t[e];
     const int ne = E.ne[e], ncs = E.ncs[e], nk = ne + ncs;
@@ -415,7 +435,7 @@ __global__ void k_edge_eig(SetupLevel S, EdgeBatch E, double tau, double *work,
     double *Sks = w;               w += (int64_t)nk * nk;
     double *Skt = w;               w += (int64_t)nk * nk;
     const int n2 = 2 * ne;
-    const int np = n2 + (n2 & 1);  // Jacobi needs an even size
+    const int np = n2 + (n2 & 1);
     double *Mt = w;                w += (int64_t)n2 * n2;
     double *Xd = w;                w += (int64_t)ne * ne;
     double *Lc = w;                w += (int64_t)nk * nk;
@@ -423,12 +443,16 @@ __global__ void k_edge_eig(SetupLevel S, EdgeBatch E, double tau, double *work,
     double *T = w;                 w += (int64_t)n2 * n2 + (int64_t)nk * n2;
     double *C = w;                 w += (int64_t)np * np;
     double *V = w;                 w += (int64_t)np * np;
+    const int ne2 = ne + (ne & 1);          // the Jacobi sweep needs an even size
+    if (jacobi_smem) {                      // 2 ne2^2 doubles of shared memory
+        C = edge_sm;
+        V = edge_sm + ne2 * ne2;
+    }
     double *cs = w;                w += 4 * (np / 2 + 1);
     double *nv = w;                w += 3 * n2;   // up to three orthonormal null vectors
     double *Wk = w;                w += (int64_t)n2 * n2;
     double *Rw = w;                w += (int64_t)ne * ne;
     double *lamv = w;              w += np;
-    __shared__ int perm[kEdgeMaxN2];
     __shared__ int order[kEdgeMaxN2];
     __shared__ double sh_a;
     __shared__ int sh_nz;
@@ -568,58 +592,75 @@ __global__ void k_edge_eig(SetupLevel S, EdgeBatch E, double tau, double *work,
         if (threadIdx.x == 0) atomicExch(err, 2000000 + e);
         return;
     }
-    // T = L^{-1} X2, X2 = [[Xd, -Xd], [-Xd, Xd]]
-    for (int q = threadIdx.x; q < n2 * n2; q += blockDim.x) {
-        const int i = q / n2, j = q % n2;
-        const double v = Xd[(i % ne) * ne + (j % ne)];
-        T[q] = ((i < ne) == (j < ne)) ? v : -v;
+    // The numerator is B Xd B^T with B = [I; -I], of rank ne at most, so the
+    // nonzero eigenvalues of C = L^-1 B Xd B^T L^-T are those of the ne x ne
+    // matrix K = Lg^T Xd Lg, where G = B^T Y^-1 B = Lg Lg^T: with K u = lam u
+    // and M = L^-1 B, v = M Lg^-T u is a unit eigenvector of C, its jump
+    // d = B^T L^-T v is Lg u and the constraint row Xd d is (Xd Lg) u.  An
+    // eighth of the Jacobi work of the 2 ne x 2 ne problem, in shared memory:
+    // with the top level's factorisation the setup and solve of the 512^2
+    // channel problem took 153 -> 130 ms (22 and 14 ms of it were these two).
+    for (int q = threadIdx.x; q < n2 * ne; q += blockDim.x) {
+        const int i = q / ne, j = q % ne;
+        T[q] = i == j ? 1.0 : (i == ne + j ? -1.0 : 0.0);
     }
     __syncthreads();
-    cta_trsm_lower(Y2, n2, n2, T, n2, n2);
-    // C = L^{-1} T^T  (T^T into C, then solve)
-    for (int q = threadIdx.x; q < np * np; q += blockDim.x) {
-        const int i = q / np, j = q % np;
-        C[q] = (i < n2 && j < n2) ? T[j * n2 + i] : 0.0;
+    cta_trsm_lower(Y2, n2, n2, T, ne, ne);                     // M
+    for (int q = threadIdx.x; q < ne * ne; q += blockDim.x) {  // G, lower triangle
+        const int i = q / ne, j = q % ne;
+        double sum = 0.0;
+        if (j <= i)
+            for (int r = 0; r < n2; ++r) sum += T[r * ne + i] * T[r * ne + j];
+        Wk[q] = sum;
     }
     __syncthreads();
-    cta_trsm_lower(Y2, n2, n2, C, n2, np);
-    for (int q = threadIdx.x; q < n2 * n2; q += blockDim.x) {
-        const int i = q / n2, j = q % n2;
+    cta_cholesky_semi(Wk, ne, ne);
+    for (int q = threadIdx.x; q < ne * ne; q += blockDim.x) {  // P = Xd Lg
+        const int i = q / ne, j = q % ne;
+        double sum = 0.0;
+        for (int r = j; r < ne; ++r) sum += Xd[i * ne + r] * Wk[r * ne + j];
+        T[q] = sum;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < ne2 * ne2; q += blockDim.x) {
+        const int i = q / ne2, j = q % ne2;
+        double sum = 0.0;
+        if (i < ne && j < ne)
+            for (int r = i; r < ne; ++r) sum += Wk[r * ne + i] * T[r * ne + j];
+        C[q] = sum;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < ne2 * ne2; q += blockDim.x) {
+        const int i = q / ne2, j = q % ne2;
         if (j > i) {
-            const double v = 0.5 * (C[i * np + j] + C[j * np + i]);
-            C[i * np + j] = v; C[j * np + i] = v;
+            const double v = 0.5 * (C[i * ne2 + j] + C[j * ne2 + i]);
+            C[i * ne2 + j] = v; C[j * ne2 + i] = v;
         }
     }
     __syncthreads();
-    cta_jacobi(C, V, np, cs, perm);
-    // eigenvalues, sorted descending (padding row gives a zero)
+    cta_jacobi(C, V, ne2, cs);
+    // eigenvalues, sorted descending (a padding row gives a zero); the other
+    // ne of the 2 ne are zero
     if (threadIdx.x == 0) {
-        for (int i = 0; i < np; ++i) { lamv[i] = C[i * np + i]; order[i] = i; }
-        for (int i = 1; i < np; ++i) {
+        for (int i = 0; i < ne2; ++i) { lamv[i] = C[i * ne2 + i]; order[i] = i; }
+        for (int i = 1; i < ne2; ++i) {
             int o = order[i]; double v = lamv[o]; int j = i - 1;
             while (j >= 0 && lamv[order[j]] < v) { order[j + 1] = order[j]; --j; }
             order[j + 1] = o;
         }
         int nsel = 0;
-        while (nsel < np && lamv[order[nsel]] > tau) ++nsel;
+        while (nsel < ne2 && lamv[order[nsel]] > tau) ++nsel;
         if (nsel > ne) nsel = ne;
         E.nsel[e] = nsel;
         for (int i = 0; i < E.max_eigs; ++i)
-            E.lam[(int64_t)e * E.max_eigs + i] = i < n2 ? lamv[order[i]] : 0.0;
+            E.lam[(int64_t)e * E.max_eigs + i] = i < ne ? lamv[order[i]] : 0.0;
     }
     __syncthreads();
     const int nsel = E.nsel[e];
-    // w_k = L^{-T} v_k ; d_k = w_s - w_t ; c_k = Xd d_k
-    for (int q = threadIdx.x; q < n2 * nsel; q += blockDim.x) {
-        const int i = q / nsel, k = q % nsel;
-        Wk[i * nsel + k] = V[i * np + order[k]];
-    }
-    __syncthreads();
-    if (nsel > 0) cta_trsm_lower_t(Y2, n2, n2, Wk, nsel, nsel);
-    for (int q = threadIdx.x; q < nsel * ne; q += blockDim.x) {
+    for (int q = threadIdx.x; q < nsel * ne; q += blockDim.x) {   // c_k = P u_k
         const int k = q / ne, i = q % ne;
         double sum = 0.0;
-        for (int j = 0; j < ne; ++j) sum += Xd[i * ne + j] * (Wk[j * nsel + k] - Wk[(ne + j) * nsel + k]);
+        for (int j = 0; j < ne; ++j) sum += T[i * ne + j] * V[j * ne2 + order[k]];
         Rw[k * ne + i] = sum;
     }
     __syncthreads();
@@ -1013,7 +1054,13 @@ void dense_inverse_from_cholesky(int n, const double *L, double *Ainv, int ld, c
 void launch_edge_eig_work(const SetupLevel &S, const EdgeBatch &E, double tau, double *work,
                           int64_t stride, int *err, cudaStream_t s) {
     if (E.nedge == 0) return;
-    k_edge_eig<<<E.nedge, 128, 0, s>>>(S, E, tau, work, stride, err);
+    // the Jacobi matrices of the longest edge in shared memory (edges of up
+    // to 64 DOFs), else in the work buffer
+    const size_t ne2 = (size_t)E.max_ne + (E.max_ne & 1), sm = 2 * ne2 * ne2 * sizeof(double);
+    const bool in_smem = ne2 <= 64;
+    if (in_smem)
+        cudaFuncSetAttribute(k_edge_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 64 * 64 * (int)sizeof(double));
+    k_edge_eig<<<E.nedge, 128, in_smem ? sm : 0, s>>>(S, E, tau, work, stride, in_smem, err);
 }
 
 }  // namespace bddc
