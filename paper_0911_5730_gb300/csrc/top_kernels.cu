@@ -193,6 +193,138 @@ __global__ void k_band_trinv(int b, const double *L, double *Linv, double *LinvT
     }
 }
 
+// Both of the above for blocks that fit in shared memory: the Cholesky factor
+// of A (to A, upper triangle zero), its inverse and the transpose, by one
+// thread block.  The factorisation's chain over the blocks of A_L waits for
+// this kernel; one SM's FP64 pipe (1.7 multiply-adds per clock) bounds it:
+// b^3 / 3 multiply-adds, 0.12 ms at b = 107.  Panels of kPB columns: the
+// diagonal block by one warp, the rows below by a thread each, the trailing
+// update by all; then the inverse block diagonal by block diagonal.
+// (Unblocked in global memory, the two kernels took 0.35 and 0.32 ms.)
+constexpr int kPB = 16, kPT = 512;
+__host__ __device__ inline int potrf_ld(int b) { return b | 1; }   // odd: column walks free of bank conflicts
+inline size_t potrf_smem(int b, bool inv) {
+    return ((size_t)b * potrf_ld(b) * (inv ? 2 : 1) + kPB * kPB * 16) * sizeof(double);
+}
+__global__ void __launch_bounds__(kPT) k_band_factor(int b, double *A, double *Linv, double *LinvT, bool inv_smem,
+                                                     int *err, int code) {
+    extern __shared__ double sm_f[];
+    const int ld = potrf_ld(b), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int NW = kPT / 32;
+    double *S = sm_f;                                           // L
+    double *T = sm_f + (size_t)b * ld;                          // a kPB x kPB block per warp
+    double *X = inv_smem ? T + kPB * kPB * NW : Linv;           // the inverse
+    const int ldx = inv_smem ? ld : b;
+    __shared__ int bad;
+    if (tid == 0) bad = 0;
+    for (int q = tid; q < b * b; q += kPT) S[(q / b) * ld + q % b] = A[q];
+    __syncthreads();
+    for (int k0 = 0; k0 < b; k0 += kPB) {
+        const int kb = min(kPB, b - k0), k1 = k0 + kb;
+        if (warp == 0) {                                        // the diagonal block
+            for (int j = k0; j < k1; ++j) {
+                const double d = S[j * ld + j];
+                if (!(d > 0.0)) {
+                    if (lane == 0) bad = 1;
+                    break;
+                }
+                const double l = sqrt(d);
+                __syncwarp();
+                if (lane == 0) S[j * ld + j] = l;
+                const int i = j + 1 + lane;
+                if (i < k1) S[i * ld + j] /= l;
+                __syncwarp();
+                const int m = k1 - j - 1;
+                for (int q = lane; q < m * m; q += 32) {
+                    const int ii = j + 1 + q / m, kk = j + 1 + q % m;
+                    if (kk <= ii) S[ii * ld + kk] -= S[ii * ld + j] * S[kk * ld + j];
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        if (bad) {
+            if (tid == 0) atomicExch(err, code);
+            return;
+        }
+        for (int i = k1 + tid; i < b; i += kPT) {               // rows below: x L_kk^T = a
+            double x[kPB];
+#pragma unroll
+            for (int j = 0; j < kPB; ++j) x[j] = j < kb ? S[i * ld + k0 + j] : 0.0;
+#pragma unroll
+            for (int j = 0; j < kPB; ++j) {
+                if (j >= kb) break;
+                x[j] /= S[(k0 + j) * ld + k0 + j];
+                S[i * ld + k0 + j] = x[j];
+#pragma unroll
+                for (int m = j + 1; m < kPB; ++m)
+                    if (m < kb) x[m] = fma(-x[j], S[(k0 + m) * ld + k0 + j], x[m]);
+            }
+        }
+        __syncthreads();
+        // trailing update: a row per warp, a lane per column
+        for (int i = k1 + warp; i < b; i += NW)
+            for (int k = k1 + lane; k <= i; k += 32) {
+                double a0 = 0.0, a1 = 0.0;
+                for (int j = k0; j + 1 < k1; j += 2) {
+                    a0 = fma(S[i * ld + j], S[k * ld + j], a0);
+                    a1 = fma(S[i * ld + j + 1], S[k * ld + j + 1], a1);
+                }
+                if (kb & 1) a0 = fma(S[i * ld + k1 - 1], S[k * ld + k1 - 1], a0);
+                S[i * ld + k] -= a0 + a1;
+            }
+        __syncthreads();
+    }
+    // X = L^-1: the diagonal blocks, a warp each, a lane per column
+    const int nblk = (b + kPB - 1) / kPB;
+    for (int k = warp; k < nblk; k += NW) {
+        const int k0 = k * kPB, kb = min(kPB, b - k0);
+        if (lane < kb) {
+            for (int i = 0; i < kb; ++i) {
+                double s = i == lane ? 1.0 : 0.0;
+                for (int m = lane; m < i; ++m) s -= S[(k0 + i) * ld + k0 + m] * X[(size_t)(k0 + m) * ldx + k0 + lane];
+                X[(size_t)(k0 + i) * ldx + k0 + lane] = i < lane ? 0.0 : s / S[(k0 + i) * ld + k0 + i];
+            }
+        }
+    }
+    __syncthreads();
+    // block (i, i - d) of X = -X_ii sum_k L_ik X_k,i-d, one block per warp
+    double *Tw = T + warp * kPB * kPB;
+    for (int d = 1; d < nblk; ++d) {
+        for (int i = d + warp; i < nblk; i += NW) {
+            const int j = i - d, i0 = i * kPB, j0 = j * kPB, ib = min(kPB, b - i0);
+            for (int q = lane; q < kPB * kPB; q += 32) {        // (block column j is a full one)
+                const int r = q / kPB, c = q % kPB;
+                double a0 = 0.0, a1 = 0.0;
+                if (r < ib)
+                    for (int k = j0; k < i0; k += 2) {
+                        a0 = fma(S[(i0 + r) * ld + k], X[(size_t)k * ldx + j0 + c], a0);
+                        a1 = fma(S[(i0 + r) * ld + k + 1], X[(size_t)(k + 1) * ldx + j0 + c], a1);
+                    }
+                Tw[q] = a0 + a1;
+            }
+            __syncwarp();
+            for (int q = lane; q < kPB * kPB; q += 32) {
+                const int r = q / kPB, c = q % kPB;
+                double s = 0.0;
+                if (r < ib) {
+                    for (int m = 0; m <= r; ++m) s = fma(X[(size_t)(i0 + r) * ldx + i0 + m], Tw[m * kPB + c], s);
+                    X[(size_t)(i0 + r) * ldx + j0 + c] = -s;
+                }
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+    }
+    for (int q = tid; q < b * b; q += kPT) {
+        const int i = q / b, c = q % b;
+        A[q] = c <= i ? S[i * ld + c] : 0.0;
+        const double v = c <= i ? X[(size_t)i * ldx + c] : 0.0;
+        Linv[q] = v;
+        LinvT[(int64_t)c * b + i] = v;
+    }
+}
+
 // C[m x n] = alpha A[m x kk] op(B) + beta C, row-major; op(B)[kk x n] is B
 // (ldb) or, with transB, the transpose of B stored n x kk.
 constexpr int GT = 16;
@@ -227,6 +359,8 @@ void gemm(int m, int n, int kk, double alpha, const double *A, int lda, const do
 }
 
 }  // namespace
+
+constexpr size_t kPotrfSmem = 226 * 1024;   // dynamic shared memory of k_band_factor, beside its static word
 
 bool build_top_band(int n, const std::vector<std::vector<int>> &rc, const std::vector<int64_t> &offAc,
                     const double *ac, int bmin, TopBand &T, DevArena &keep, DevArena &tmp, int *err,
@@ -296,15 +430,26 @@ bool build_top_band(int n, const std::vector<std::vector<int>> &rc, const std::v
             const int bp = (int)bs(k - 1);
             gemm(b, b, bp, -1.0, Mb + offE[k - 1], bp, Mb + offE[k - 1], bp, true, 1.0, Dk, b, st);
         }
-        k_band_potrf<<<1, 512, 0, st>>>(b, Dk, err, 6000000 + k);
-        k_band_trinv<<<1, 256, 0, st>>>(b, Dk, T.Linv + offD[k], T.LinvT + offD[k]);
-        if (k > 0) {   // F_k = Linv_k M_k-1
+        if (potrf_smem(b, false) <= kPotrfSmem) {
+            const bool inv = potrf_smem(b, true) <= kPotrfSmem;
+            k_band_factor<<<1, kPT, potrf_smem(b, inv), st>>>(b, Dk, T.Linv + offD[k], T.LinvT + offD[k], inv, err,
+                                                              6000000 + k);
+        } else {
+            k_band_potrf<<<1, 512, 0, st>>>(b, Dk, err, 6000000 + k);
+            k_band_trinv<<<1, 256, 0, st>>>(b, Dk, T.Linv + offD[k], T.LinvT + offD[k]);
+        }
+        if (k + 1 < nb)   // M_k = E_k Linv_k^T
+            gemm((int)bs(k + 1), b, b, 1.0, E + offE[k], b, T.LinvT + offD[k], b, false, 0.0, Mb + offE[k], b, st);
+    }
+    // F_k = Linv_k M_k-1 and G_k = Linv_k^T M_k^T, off the chain
+    for (int k = 0; k < nb; ++k) {
+        const int b = (int)bs(k);
+        if (k > 0) {
             const int bp = (int)bs(k - 1);
             gemm(b, bp, b, 1.0, T.Linv + offD[k], b, Mb + offE[k - 1], bp, false, 0.0, T.F + offF[k], bp, st);
         }
-        if (k + 1 < nb) {   // M_k = E_k Linv_k^T,  G_k = Linv_k^T M_k^T
+        if (k + 1 < nb) {
             const int bn = (int)bs(k + 1);
-            gemm(bn, b, b, 1.0, E + offE[k], b, T.LinvT + offD[k], b, false, 0.0, Mb + offE[k], b, st);
             gemm(b, bn, b, 1.0, T.LinvT + offD[k], b, Mb + offE[k], b, true, 0.0, T.G + offG[k], bn, st);
         }
     }
@@ -702,6 +847,7 @@ void launch_identity(int n, double *I, cudaStream_t s) {
 }
 
 void prepare_top_kernels() {
+    cudaFuncSetAttribute(k_band_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPotrfSmem);
     const int big = (int)kTopSmemMax;
 #define BDDC_TOP_ATTR(R, F, S) cudaFuncSetAttribute(k_top_chain<R, F, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, big)
     BDDC_TOP_ATTR(1, true, true); BDDC_TOP_ATTR(2, true, true); BDDC_TOP_ATTR(4, true, true);
