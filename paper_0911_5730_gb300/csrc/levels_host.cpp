@@ -8,10 +8,15 @@
 #include "levels_host.h"
 
 #include <algorithm>
+#include <atomic>
+#include <exception>
 #include <map>
+#include <mutex>
 #include <numeric>
 #include <queue>
 #include <stdexcept>
+#include <system_error>
+#include <thread>
 
 namespace bddc {
 
@@ -29,6 +34,39 @@ struct DSU {
         if (a != b) { if (a < b) p[b] = a; else p[a] = b; }
     }
 };
+
+// f(s) for every substructure s < n, shared out to the host's cores (the calls
+// touch disjoint data); few substructures stay on the calling thread.  The
+// first exception is rethrown after all threads have stopped.  (The orderings
+// of the 512^2 channel problem's 1024 substructures were 55 of the 130 ms of
+// its setup and solve.)
+template <class F> void for_each_sub(int n, F &&f) {
+    constexpr int kChunk = 16, kMostThreads = 16;
+    std::atomic<int> next{0};
+    std::exception_ptr first;
+    std::mutex mu;
+    auto work = [&] {
+        try {
+            for (int s0 = next.fetch_add(kChunk); s0 < n; s0 = next.fetch_add(kChunk))
+                for (int s = s0; s < std::min(n, s0 + kChunk); ++s) f(s);
+        } catch (...) {
+            std::lock_guard<std::mutex> lk(mu);
+            if (!first) first = std::current_exception();
+            next = n;
+        }
+    };
+    const int cores = (int)std::thread::hardware_concurrency();
+    const int want = std::min(std::min(cores, kMostThreads), n / (4 * kChunk));
+    std::vector<std::thread> pool;
+    try {
+        for (int t = 1; t < want; ++t) pool.emplace_back(work);
+    } catch (const std::system_error &) {
+        // no more threads to be had: those that started and this one do it
+    }
+    work();
+    for (auto &t : pool) t.join();
+    if (first) std::rethrow_exception(first);
+}
 
 // Bandwidth of an ordering (ord[k] = node) on an undirected graph.
 int bandwidth(const std::vector<std::vector<int>> &adj, const std::vector<int> &ord) {
@@ -121,15 +159,16 @@ void HLevel::build() {
         sub_elems[esub[e]].push_back(e);
     }
     sub_dofs.assign(nsub, {});
-    for (int s = 0; s < nsub; ++s) {
+    for (int s = 0; s < nsub; ++s)
         if (sub_elems[s].empty()) throw Error(BDDC_E_ARG, "empty substructure " + std::to_string(s));
+    for_each_sub(nsub, [&](int s) {
         auto &d = sub_dofs[s];
         for (int e : sub_elems[s])
             for (int64_t k = eptr[e]; k < eptr[e + 1]; ++k)
                 if (eslot[k] >= 0) d.push_back(eslot[k]);
         std::sort(d.begin(), d.end());
         d.erase(std::unique(d.begin(), d.end()), d.end());
-    }
+    });
     subs_ptr.assign(n + 1, 0);
     for (int s = 0; s < nsub; ++s) for (int g : sub_dofs[s]) subs_ptr[g + 1]++;
     for (int g = 0; g < n; ++g) subs_ptr[g + 1] += subs_ptr[g];
@@ -159,14 +198,16 @@ void HLevel::build() {
             for (int64_t b = a + 1; b < eptr[e + 1]; ++b) {
                 const int gb = eslot[b];
                 if (gb < 0 || !is_iface[gb] || is_corner[gb]) continue;
-                if (subs(ga) == subs(gb)) dsu.unite(ga, gb);
+                if (mult(ga) == mult(gb) && std::equal(subs_idx.begin() + subs_ptr[ga], subs_idx.begin() + subs_ptr[ga + 1],
+                                                       subs_idx.begin() + subs_ptr[gb]))
+                    dsu.unite(ga, gb);
             }
         }
     }
     std::map<std::tuple<int, int, int>, std::vector<int>> groups;   // (s, t, root)
     for (int g = 0; g < n; ++g) {
         if (!is_iface[g] || is_corner[g]) continue;
-        auto sv = subs(g);
+        const auto sv = subs_idx.begin() + subs_ptr[g];
         groups[{sv[0], sv[1], dsu.find(g)}].push_back(g);
     }
     edges.clear();
@@ -187,7 +228,8 @@ void HLevel::build() {
     bw.assign(nsub, 0); bsz.assign(nsub, 1); nblk.assign(nsub, 0);
     std::vector<int> loc(n, -1);
     std::vector<std::vector<int>> first_all(nsub);   // lowest coupled position per row
-    for (int s = 0; s < nsub; ++s) {
+    // (loc is set for interior DOFs only, each of which one substructure holds)
+    for_each_sub(nsub, [&](int s) {
         std::vector<int> I;
         for (int g : sub_dofs[s]) (is_iface[g] ? Gord[s] : I).push_back(g);
         for (size_t k = 0; k < I.size(); ++k) loc[I[k]] = (int)k;
@@ -231,7 +273,7 @@ void HLevel::build() {
         bw[s] = std::max(bwn, 0);
         bsz[s] = std::max(bn, 1);
         nblk[s] = I.empty() ? 0 : (int)((I.size() + bsz[s] - 1) / bsz[s]);
-    }
+    });
     // Prefer one power-of-two block size for the whole level (the apply
     // kernels then unroll the block solves completely).
     block_uniform = 0;
