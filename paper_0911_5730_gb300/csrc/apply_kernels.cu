@@ -123,6 +123,8 @@ __device__ void dirichlet_solve(const T *F, int b, int m, bool swz, ACC *x, ACC 
 // (4)-(5): u_I = A_II^{-1} r_I per substructure; r_B on Gamma = r - A_{Gamma I} u_I.
 template <class T, class ACC>
 __global__ void __launch_bounds__(kGT) k_pre(DevLevel L, const double *r, const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     extern __shared__ unsigned char smem_raw[];
     ACC *sm = reinterpret_cast<ACC *>(smem_raw);
@@ -176,6 +178,8 @@ struct StreamSmem {
 
 template <class T, class ACC, bool POST>
 __global__ void __launch_bounds__(kSB) k_dir_s(DevLevel L, const double *r, double *z, const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem_s[];
     const StreamSmem ly = StreamSmem::of<T, ACC>(L);
@@ -320,6 +324,8 @@ __global__ void __launch_bounds__(kSB) k_dir_s(DevLevel L, const double *r, doub
 constexpr int kNRows = 32, kNWarps = 8;
 template <class T, class ACC>
 __global__ void __launch_bounds__(32 * kNWarps) k_neumann(DevLevel L, const double *r, const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     extern __shared__ unsigned char smem_raw[];
     __shared__ ACC part[kNWarps][kNRows];
@@ -369,6 +375,8 @@ __global__ void __launch_bounds__(32 * kNWarps) k_neumann(DevLevel L, const doub
 // (9): u_B = sum_i R_i^T D_i (w_i + Psi_i u_c).
 template <class T, class ACC>
 __global__ void k_average(DevLevel L, const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     extern __shared__ unsigned char smem_raw[];
     ACC *uc = reinterpret_cast<ACC *>(smem_raw);
@@ -391,6 +399,8 @@ __global__ void k_average(DevLevel L, const int *skip) {
 // (10)-(11): interior of u = A_II^{-1}(r_I - A_{I Gamma} u_B), interface of u = u_B.
 template <class T, class ACC>
 __global__ void __launch_bounds__(kGT) k_post(DevLevel L, const double *r, double *z, const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     extern __shared__ unsigned char smem_raw[];
     ACC *sm = reinterpret_cast<ACC *>(smem_raw);
@@ -1098,6 +1108,8 @@ __device__ bool grid_reduce(double local, double *part, unsigned *counter, doubl
 }
 
 __global__ void k_q1_spmv(int nx, const double *w, const double *x, double *y) {
+    pdl_wait();
+    pdl_trigger();
     const int n1 = nx - 1;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= (int64_t)n1 * n1) return;
@@ -1154,15 +1166,20 @@ __global__ void k_pcg_init(int n, const double *b, double *x, double *r, double 
 
 // Iteration `it` of PCG, first half: the new direction p_new = z + beta p_old
 // (into the other buffer, so that p_old stays intact for the halo of other
-// tiles), q = A p_new and alpha = rho / (p_new . q).  The FP64 pipe is the
-// limit here, so p_new is formed once per point of a PT_X x PT_Y tile plus its
-// halo in shared memory, and every thread handles PT_Y / 4 nodes of a column.
-constexpr int PT_X = 64, PT_Y = 16, PT_T = 256;
-__global__ void __launch_bounds__(PT_T)
+// warps), q = A p_new and alpha = rho / (p_new . q).  The FP64 pipe is the
+// limit on large meshes, latency on small ones.  A warp marches up a strip of
+// kDirC columns (a lane each, and one on either side for the neighbours'
+// values, which come by shuffles), three rows of p_new in registers: nothing
+// waits at a barrier, and small meshes spread over as many SMs as there are
+// segments of two rows.
+// (Shared-memory tiles of 64 x 16 nodes by blocks of 256 threads: 522 us per
+// solve of the 32^2 problem, 13.8 ms on 1024^2; now 483 us, with the update
+// spread over more blocks, and 13.05 ms.)
+constexpr int kDirC = 30, kDirT = 128;
+__global__ void __launch_bounds__(kDirT)
 k_pcg_dir_spmv(int nx, const double *__restrict__ w, const double *__restrict__ z, double *p0,
                double *p1, double *__restrict__ q, double *part, unsigned *counter, PcgScalars *sc,
-               double *alphas) {
-    __shared__ double ps[PT_Y + 2][PT_X + 2];
+               double *alphas, int strips, int rows) {
     pdl_wait();
     pdl_trigger();
     if (sc->done) return;
@@ -1378,10 +1395,14 @@ template <class T, class ACC> void pre_t(const DevLevel &L, const double *r, con
     }
     launch_k(false, k_pre<T, ACC>, L.nsub, kGT, generic_smem<ACC>(L), s, L, r, skip);
 }
-template <class T, class ACC> void neumann_t(const DevLevel &L, const double *r, const int *skip, cudaStream_t s) {
+// pdl: beside the warp kernels' programmatic launches; on levels of generic
+// kernels it cost 0.5 ms of the elasticity solve (blocks waiting for their
+// predecessor hold shared memory it could use)
+template <class T, class ACC>
+void neumann_t(const DevLevel &L, const double *r, const int *skip, bool pdl, cudaStream_t s) {
     const int rows = (L.max_nG + kNRows - 1) / kNRows;
     const dim3 grid((unsigned)L.nsub, (unsigned)(rows > 0 ? rows : 1));
-    launch_grid(false, k_neumann<T, ACC>, grid, 32 * kNWarps, sizeof(ACC) * (size_t)(L.max_nG > 0 ? L.max_nG : 1), s, L, r,
+    launch_grid(pdl, k_neumann<T, ACC>, grid, 32 * kNWarps, sizeof(ACC) * (size_t)(L.max_nG > 0 ? L.max_nG : 1), s, L, r,
               skip);
 }
 template <class T, class ACC> void post_t(const DevLevel &L, const double *r, double *z,
@@ -1569,8 +1590,21 @@ void apply_level_dir(const DevLevel &L, int prec, bool post, const double *r, do
     if (rz) launch_pcg_rz((int)L.n, r, z, *rz, s);
 }
 
+// The staged record per warp, unless so few records fit an SM that the
+// substructures take several waves of less than eight warps each: then the
+// generic kernel, which reads the operator from L2 with the whole GPU.
+// (The reduced FP64 solve at 512^2, six records of 33 KB per SM: 4.26 -> 4.00
+// ms, with programmatic launches of its vector kernels.)
+bool neu_few_warps(const DevLevel &L, int prec) {
+    const size_t rec = al16((size_t)L.max_nrec[pidx_of(prec)]) +
+                       al16((prec == BDDC_PREC_FP64 ? 8 : 4) * (size_t)L.max_nG) + 16;
+    const int64_t per = (int64_t)(kSmemMax / al16(rec));
+    return per < 8 && per * num_sms() < L.nsub;
+}
+
 void apply_level_neumann(const DevLevel &L, int prec, const double *r, const int *skip, cudaStream_t s) {
-    if (warp_path(L, prec)) {
+    const bool warp = warp_path(L, prec);
+    if (warp && !neu_few_warps(L, prec)) {
         if (prec == BDDC_PREC_FP64) neu_launch<double, double>(L, prec, r, skip, s);
         else if (prec == BDDC_PREC_FP32) neu_launch<float, float>(L, prec, r, skip, s);
         else neu_launch<__nv_bfloat16, float>(L, prec, r, skip, s);
@@ -1653,7 +1687,7 @@ void launch_q1_weights(int nx, const double *k, double *w, cudaStream_t s) {
 }
 void launch_q1_spmv(int nx, const double *w, const double *x, double *y, cudaStream_t s) {
     const int64_t n = (int64_t)(nx - 1) * (nx - 1);
-    k_q1_spmv<<<(int)((n + 255) / 256), 256, 0, s>>>(nx, w, x, y);
+    launch_pdl(k_q1_spmv, (int)((n + 255) / 256), 256, 0, s, nx, w, x, y);
 }
 void launch_residual(int nx, const double *w, const double *b, const double *x, double *res,
                      cudaStream_t s) {
@@ -1672,17 +1706,15 @@ void launch_pcg_init(int n, const double *b, double *x, double *r, double *p0, d
 void launch_pcg_dir_spmv(int nx, const double *w, const double *z, double *p0, double *p1,
                          double *q, double *part, unsigned *counter, PcgScalars *sc,
                          double *alphas, cudaStream_t s) {
-    const int n1 = nx - 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((n1 + PT_X - 1) / PT_X), (unsigned)((n1 + PT_Y - 1) / PT_Y));
-    cfg.blockDim = dim3(PT_T);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl_enabled() ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, k_pcg_dir_spmv, nx, w, z, p0, p1, q, part, counter, sc, alphas);
+    // about sixteen warps per SM, segments of at least two rows
+    const int n1 = nx - 1, strips = (n1 + kDirC - 1) / kDirC;
+    int segs = 16 * num_sms() / strips;
+    segs = segs < 1 ? 1 : (segs > (n1 + 1) / 2 ? (n1 + 1) / 2 : segs);
+    const int rows = (n1 + segs - 1) / segs;
+    segs = (n1 + rows - 1) / rows;
+    const int wpb = kDirT / 32;
+    launch_pdl(k_pcg_dir_spmv, (strips * segs + wpb - 1) / wpb, kDirT, 0, s, nx, w, z, p0, p1, q, part, counter, sc,
+               alphas, strips, rows);
 }
 void launch_pcg_update(int n, double *x, double *r, const double *p0, const double *p1,
                        const double *q, double *part, unsigned *counter, PcgScalars *sc,

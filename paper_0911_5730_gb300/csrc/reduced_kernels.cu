@@ -69,6 +69,8 @@ __device__ bool red_sum(double v, double *part, unsigned *counter, double *out) 
 __global__ void __launch_bounds__(RT) k_red_init(int ng, const int *ifaceDof, const double *b, const double *qf,
                                                  double *x, double *r, double *p, double *part, unsigned *counter,
                                                  RedScalars *sc, double tol, int maxit) {
+    pdl_wait();
+    pdl_trigger();
     double s = 0.0;
     for (int i = blockIdx.x * RT + threadIdx.x; i < ng; i += gridDim.x * RT) {
         const int g = ifaceDof[i];
@@ -94,6 +96,8 @@ __global__ void __launch_bounds__(RT) k_red_init(int ng, const int *ifaceDof, co
 // rf[ifaceDof[i]] = r[i] (rf: a full-length vector, zero in the interior)
 __global__ void __launch_bounds__(RT) k_red_scatter(int ng, const int *ifaceDof, const double *r, double *rf,
                                                     const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     for (int i = blockIdx.x * RT + threadIdx.x; i < ng; i += gridDim.x * RT) rf[ifaceDof[i]] = r[i];
 }
@@ -101,6 +105,8 @@ __global__ void __launch_bounds__(RT) k_red_scatter(int ng, const int *ifaceDof,
 // rho = r.z (z = u_B), beta = rho / rho_old (0 on a fresh start)
 __global__ void __launch_bounds__(RT) k_red_rz(int ng, const double *r, const double *z, double *part,
                                                unsigned *counter, RedScalars *sc, double *betas, const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     double s = 0.0;
     for (int i = blockIdx.x * RT + threadIdx.x; i < ng; i += gridDim.x * RT) s = fma(r[i], z[i], s);
@@ -117,6 +123,8 @@ __global__ void __launch_bounds__(RT) k_red_rz(int ng, const double *r, const do
 // p = z + beta p, and u_B = p (the input of the next interface product)
 __global__ void __launch_bounds__(RT) k_red_dir(int ng, double *uB, double *p, const RedScalars *sc,
                                                 const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     const double beta = sc->beta;
     for (int i = blockIdx.x * RT + threadIdx.x; i < ng; i += gridDim.x * RT) {
@@ -130,6 +138,8 @@ __global__ void __launch_bounds__(RT) k_red_dir(int ng, double *uB, double *p, c
 __global__ void __launch_bounds__(RT) k_red_pq(int ng, const int *ifaceDof, const double *qf, const double *p,
                                                double *q, double *part, unsigned *counter, RedScalars *sc,
                                                double *alphas, const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     double s = 0.0;
     for (int i = blockIdx.x * RT + threadIdx.x; i < ng; i += gridDim.x * RT) {
@@ -149,6 +159,8 @@ __global__ void __launch_bounds__(RT) k_red_pq(int ng, const int *ifaceDof, cons
 __global__ void __launch_bounds__(RT) k_red_update(int ng, double *x, double *r, const double *p, const double *q,
                                                    double *part, unsigned *counter, RedScalars *sc,
                                                    const int *skip) {
+    pdl_wait();
+    pdl_trigger();
     if (skip && *skip) return;
     const double alpha = sc->alpha;
     double s = 0.0;
@@ -181,27 +193,27 @@ int red_blocks() { return RG; }
 void launch_red_init(int ng, const int *ifaceDof, const double *b, const double *qf, double *x, double *r,
                      double *p, double *part, unsigned *counter, RedScalars *sc, double tol, int maxit,
                      cudaStream_t s) {
-    launch_k(false, k_red_init, red_grid(ng), RT, 0, s, ng, ifaceDof, b, qf, x, r, p, part, counter, sc, tol,
+    launch_k(true, k_red_init, red_grid(ng), RT, 0, s, ng, ifaceDof, b, qf, x, r, p, part, counter, sc, tol,
              maxit);
 }
 void launch_red_scatter(int ng, const int *ifaceDof, const double *r, double *rf, const int *skip,
                         cudaStream_t s) {
-    launch_k(false, k_red_scatter, red_grid(ng), RT, 0, s, ng, ifaceDof, r, rf, skip);
+    launch_k(true, k_red_scatter, red_grid(ng), RT, 0, s, ng, ifaceDof, r, rf, skip);
 }
 void launch_red_rz(int ng, const double *r, const double *z, double *part, unsigned *counter, RedScalars *sc,
                    double *betas, const int *skip, cudaStream_t s) {
-    launch_k(false, k_red_rz, red_grid(ng), RT, 0, s, ng, r, z, part, counter, sc, betas, skip);
+    launch_k(true, k_red_rz, red_grid(ng), RT, 0, s, ng, r, z, part, counter, sc, betas, skip);
 }
 void launch_red_dir(int ng, double *uB, double *p, const RedScalars *sc, const int *skip, cudaStream_t s) {
-    launch_k(false, k_red_dir, red_grid(ng), RT, 0, s, ng, uB, p, sc, skip);
+    launch_k(true, k_red_dir, red_grid(ng), RT, 0, s, ng, uB, p, sc, skip);
 }
 void launch_red_pq(int ng, const int *ifaceDof, const double *qf, const double *p, double *q, double *part,
                    unsigned *counter, RedScalars *sc, double *alphas, const int *skip, cudaStream_t s) {
-    launch_k(false, k_red_pq, red_grid(ng), RT, 0, s, ng, ifaceDof, qf, p, q, part, counter, sc, alphas, skip);
+    launch_k(true, k_red_pq, red_grid(ng), RT, 0, s, ng, ifaceDof, qf, p, q, part, counter, sc, alphas, skip);
 }
 void launch_red_update(int ng, double *x, double *r, const double *p, const double *q, double *part,
                        unsigned *counter, RedScalars *sc, const int *skip, cudaStream_t s) {
-    launch_k(false, k_red_update, red_grid(ng), RT, 0, s, ng, x, r, p, q, part, counter, sc, skip);
+    launch_k(true, k_red_update, red_grid(ng), RT, 0, s, ng, x, r, p, q, part, counter, sc, skip);
 }
 
 }  // namespace bddc
