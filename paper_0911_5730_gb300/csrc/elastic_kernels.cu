@@ -107,11 +107,27 @@ __device__ bool el_grid_sum(double v, double *part, unsigned *counter, double *o
     }
     __syncthreads();
     if (!last) return false;
+    // all threads, eight loads in flight each (with one thread adding the 578
+    // partials of the 384^2 mesh in turn, an FP32 solve there took 5.54 ms,
+    // now 5.07)
+    __threadfence();
+    double t = 0.0;
+    for (unsigned b0 = threadIdx.x; b0 < gridDim.x; b0 += 8 * kET) {
+        double u[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) u[q] = b0 + q * kET < gridDim.x ? __ldcg(&part[b0 + q * kET]) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t += u[q];
+    }
+    t = warp_sum_d(t);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = t;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        double t = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) t += __ldcg(&part[b]);
-        *out = t;
+        double b = 0.0;
+#pragma unroll
+        for (int w = 0; w < kET / 32; ++w) b += ws[w];
+        *out = b;
         *counter = 0u;
     }
     __syncthreads();
@@ -139,10 +155,26 @@ __device__ void el_grid_sum_k(double v, int K, double *part, unsigned *counter, 
     __syncthreads();
     if (!last) return;
     __threadfence();
+    // thread t: column t mod K of blocks t / K, t / K + per, ..., eight loads in flight
+    double t = 0.0;
+    if ((int)threadIdx.x < per * K) {
+        const int kk = threadIdx.x % K;
+        for (int b0 = threadIdx.x / K; b0 < (int)gridDim.x; b0 += 8 * per) {
+            double u[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                u[q] = b0 + q * per < (int)gridDim.x ? __ldcg(&part[(int64_t)(b0 + q * per) * K + kk]) : 0.0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) t += u[q];
+        }
+    }
+    __syncthreads();
+    red[threadIdx.x] = t;
+    __syncthreads();
     if ((int)threadIdx.x < K) {
-        double t = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) t += __ldcg(&part[(int64_t)b * K + threadIdx.x]);
-        fin((int)threadIdx.x, t);
+        double tot = 0.0;
+        for (int u = 0; u < per; ++u) tot += red[u * K + threadIdx.x];
+        fin((int)threadIdx.x, tot);
     }
     __syncthreads();
     if (threadIdx.x == 0) *counter = 0u;
