@@ -1100,7 +1100,12 @@ __device__ bool grid_reduce(double local, double *part, unsigned *counter, doubl
     __syncthreads();
     if (!last) return false;
     double s = 0.0;
-    for (int i = threadIdx.x; i < (int)nb; i += blockDim.x) s += __ldcg(&part[i]);
+    for (int i = threadIdx.x; i < (int)nb; i += 4 * blockDim.x) {   // four loads in flight
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i + u * (int)blockDim.x < (int)nb ? __ldcg(&part[i + u * blockDim.x]) : 0.0;
+        s += (v[0] + v[1]) + (v[2] + v[3]);
+    }
     // in-order across threads is not needed for determinism: fixed partition
     const double tot = block_sum(s);
     if (threadIdx.x == 0) { *out = tot; *counter = 0u; }
@@ -1184,68 +1189,76 @@ k_pcg_dir_spmv(int nx, const double *__restrict__ w, const double *__restrict__ 
     pdl_trigger();
     if (sc->done) return;
     const int n1 = nx - 1;
-    const int n = n1 * n1;
+    const int64_t n = (int64_t)n1 * n1;
     const double bt = sc->beta;
     const bool odd = sc->it & 1;
-    const double *po = odd ? p1 : p0;
-    double *pn = odd ? p0 : p1;
-    const int i0 = blockIdx.x * PT_X, j0 = blockIdx.y * PT_Y;   // 0-based node column / row
-    for (int t = threadIdx.x; t < (PT_Y + 2) * (PT_X + 2); t += PT_T) {
-        const int hy = t / (PT_X + 2), hx = t - hy * (PT_X + 2);
-        const int i = i0 + hx - 1, j = j0 + hy - 1;
-        double v = 0.0;
-        if (i >= 0 && i < n1 && j >= 0 && j < n1) {
-            const int g = j * n1 + i;
-            v = fma(bt, po[g], z[g]);
-        }
-        ps[hy][hx] = v;
-    }
-    __syncthreads();
-    constexpr int NY = PT_Y / (PT_T / PT_X);   // nodes per thread
-    const int tx = threadIdx.x % PT_X, ty = threadIdx.x / PT_X;
-    const int i = i0 + tx;
-    const bool W = i > 0, E = i < n1 - 1;
-    // all weights of the thread's nodes first (independent loads in flight),
-    // then the products from shared memory
-    double wv[NY][9];
-#pragma unroll
-    for (int k = 0; k < NY; ++k) {
-        const int j = j0 + ty + k * (PT_T / PT_X);
-        const bool in = i < n1 && j < n1;
-        const bool S = j > 0, N = j < n1 - 1;
-        const int g = j * n1 + i;
-        wv[k][0] = in ? __ldg(w + g) : 0.0;
-        wv[k][1] = in && E ? __ldg(w + n + g) : 0.0;
-        wv[k][2] = in && N ? __ldg(w + 2 * n + g) : 0.0;
-        wv[k][3] = in && N && E ? __ldg(w + 3 * n + g) : 0.0;
-        wv[k][4] = in && N && W ? __ldg(w + 4 * n + g) : 0.0;
-        wv[k][5] = in && W ? __ldg(w + n + g - 1) : 0.0;
-        wv[k][6] = in && S ? __ldg(w + 2 * n + g - n1) : 0.0;
-        wv[k][7] = in && S && W ? __ldg(w + 3 * n + g - n1 - 1) : 0.0;
-        wv[k][8] = in && S && E ? __ldg(w + 4 * n + g - n1 + 1) : 0.0;
-    }
+    const double *__restrict__ po = odd ? p1 : p0;
+    double *__restrict__ pn = odd ? p0 : p1;
+    const int lane = threadIdx.x & 31;
+    const int unit = blockIdx.x * (kDirT / 32) + (threadIdx.x >> 5);
+    const int j0 = (unit / strips) * rows, j1 = min(n1, j0 + rows);
+    const int i = (unit % strips) * kDirC + lane - 1;       // 0-based node column
+    const bool in = i >= 0 && i < n1;
+    const bool out = in && lane >= 1 && lane <= kDirC;
     double s = 0.0;
+    if (j0 < n1) {
+        double a = 0.0, b = 0.0;                            // p_old and z of the next row
+        auto fetch = [&](int j) {
+            const bool ok = in && j >= 0 && j < n1;
+            const int64_t g = (int64_t)j * n1 + i;
+            a = ok ? po[g] : 0.0;
+            b = ok ? z[g] : 0.0;
+        };
+        // a row of p_new at this column and its two neighbours
+        struct Row { double c, l, r; };
+        auto form = [&]() -> Row {
+            Row R;
+            R.c = fma(bt, a, b);
+            R.l = __shfl_up_sync(0xffffffffu, R.c, 1);
+            R.r = __shfl_down_sync(0xffffffffu, R.c, 1);
+            return R;
+        };
+        fetch(j0 - 1);
+        Row S = form();
+        fetch(j0);
+        Row C = form();
+        fetch(j0 + 1);
+#pragma unroll 2
+        for (int j = j0; j < j1; ++j) {
+            const int64_t g = (int64_t)j * n1 + i;
+            double wv[9];                                   // a missing neighbour's p_new is zero, its weight finite
 #pragma unroll
-    for (int k = 0; k < NY; ++k) {
-        const int ly = ty + k * (PT_T / PT_X);
-        const int j = j0 + ly;
-        if (i >= n1 || j >= n1) continue;
-        const int g = j * n1 + i;
-        const int hy = ly + 1, hx = tx + 1;
-        // neighbours outside the domain hold zero in ps and carry zero weight
-        const double pc = ps[hy][hx];
-        double v = wv[k][0] * pc;
-        v = fma(wv[k][1], ps[hy][hx + 1], v);
-        v = fma(wv[k][2], ps[hy + 1][hx], v);
-        v = fma(wv[k][3], ps[hy + 1][hx + 1], v);
-        v = fma(wv[k][4], ps[hy + 1][hx - 1], v);
-        v = fma(wv[k][5], ps[hy][hx - 1], v);
-        v = fma(wv[k][6], ps[hy - 1][hx], v);
-        v = fma(wv[k][7], ps[hy - 1][hx - 1], v);
-        v = fma(wv[k][8], ps[hy - 1][hx + 1], v);
-        pn[g] = pc;
-        q[g] = v;
-        s = fma(v, pc, s);
+            for (int u = 0; u < 9; ++u) wv[u] = 0.0;
+            if (out) {
+                wv[0] = __ldg(w + g);
+                wv[1] = __ldg(w + n + g);
+                wv[2] = __ldg(w + 2 * n + g);
+                wv[3] = __ldg(w + 3 * n + g);
+                wv[4] = __ldg(w + 4 * n + g);
+                wv[5] = __ldg(w + n + g - 1);
+                wv[6] = __ldg(w + 2 * n + g - n1);
+                wv[7] = __ldg(w + 3 * n + g - n1 - 1);
+                wv[8] = __ldg(w + 4 * n + g - n1 + 1);
+            }
+            const Row N = form();
+            if (j + 1 < j1) fetch(j + 2);
+            double v = wv[0] * C.c;
+            v = fma(wv[1], C.r, v);
+            v = fma(wv[2], N.c, v);
+            v = fma(wv[3], N.r, v);
+            v = fma(wv[4], N.l, v);
+            v = fma(wv[5], C.l, v);
+            v = fma(wv[6], S.c, v);
+            v = fma(wv[7], S.l, v);
+            v = fma(wv[8], S.r, v);
+            if (out) {
+                pn[g] = C.c;
+                q[g] = v;
+                s = fma(v, C.c, s);
+            }
+            S = C;
+            C = N;
+        }
     }
     __shared__ double tot;
     if (grid_reduce(s, part, counter, &tot) && threadIdx.x == 0) {
@@ -1356,9 +1369,12 @@ int grid_for(int64_t n) {
     if (g < 1) g = 1;
     return (int)g;
 }
-// Grid of the FP64 vector kernels of the PCG iteration: about four entries per thread.
+// Grid of the FP64 vector kernels of the PCG iteration: about four entries per
+// thread (a block's reduction costs as much FP64 time as two entries of each
+// of its threads), one where that leaves SMs without a block.
 int vec_grid(int64_t n) {
-    int64_t g = (n + 4 * RB - 1) / (4 * RB);
+    const int per = n >= (int64_t)4 * RB * num_sms() / 2 ? 4 : 1;
+    int64_t g = (n + per * RB - 1) / (per * RB);
     if (g > vec_grid_cap()) g = vec_grid_cap();
     if (g < 1) g = 1;
     return (int)g;
@@ -1610,9 +1626,9 @@ void apply_level_neumann(const DevLevel &L, int prec, const double *r, const int
         else neu_launch<__nv_bfloat16, float>(L, prec, r, skip, s);
         return;
     }
-    if (prec == BDDC_PREC_FP64) neumann_t<double, double>(L, r, skip, s);
-    else if (prec == BDDC_PREC_FP32) neumann_t<float, float>(L, r, skip, s);
-    else neumann_t<__nv_bfloat16, float>(L, r, skip, s);
+    if (prec == BDDC_PREC_FP64) neumann_t<double, double>(L, r, skip, warp, s);
+    else if (prec == BDDC_PREC_FP32) neumann_t<float, float>(L, r, skip, warp, s);
+    else neumann_t<__nv_bfloat16, float>(L, r, skip, warp, s);
 }
 
 void apply_level_average(const DevLevel &L, int prec, const int *skip, cudaStream_t s) {
