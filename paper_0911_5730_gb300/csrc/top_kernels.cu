@@ -479,7 +479,6 @@ namespace {
 
 constexpr int kTopWarps = 8;
 constexpr int kTopThreads = 32 * kTopWarps;
-constexpr int kRowLanes = 8, kRowsPerWarp = 32 / kRowLanes;   // a recurrence's rows
 
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
@@ -603,7 +602,15 @@ __global__ void __launch_bounds__(256) k_top_rows(TopBandArgs a, const double *i
 //
 // STAGED = false (blocks too large for two stages in shared memory): the rows
 // are read from global memory where they are used.
-template <int R, bool FWD, bool STAGED>
+// LN lanes share a row.  The FP64 pipe of an SM takes 19 clocks for a warp's
+// multiply-add, so the step's time is the multiply-adds and the reduction's
+// adds of the busiest warp: sixteen lanes where a CTA's share of every block
+// is at most sixteen rows (every warp then has rows; eight lanes left half of
+// the warps idle), eight for larger blocks.  The two right-hand sides of
+// R = 2 are reduced together: the first exchange leaves each half of the
+// lanes with one of them.  2253 top unknowns, 32
+// right-hand sides: 45 -> 41 us a sweep.
+template <int R, bool FWD, bool STAGED, int LN>
 __global__ void __launch_bounds__(kTopThreads) k_top_chain(TopBandArgs a, const double *in, double *out) {
     if (a.skip && *a.skip) return;          // the same for every CTA of the cluster
     extern __shared__ __align__(16) unsigned char sm_top[];
@@ -686,22 +693,20 @@ __global__ void __launch_bounds__(kTopThreads) k_top_chain(TopBandArgs a, const 
             my_rows(k, r0, r1, bo);
             const int b0 = sboff[k], o0 = FWD ? sboff[k - 1] : sboff[k + 1];
             const double *Mk = staged(k, s);
-            // kRowLanes lanes per row, 32 / kRowLanes rows per warp at once:
-            // the FP64 pipe retires under two lanes per clock per SM here, so
-            // the reduction across lanes (FP64 adds) is kept short
-            const int sub = lane / kRowLanes, l = lane % kRowLanes;
-            for (int i0 = r0 + w * kRowsPerWarp; i0 < r1; i0 += kTopWarps * kRowsPerWarp) {
+            constexpr int RPW = 32 / LN;            // rows of a warp at once
+            const int sub = lane / LN, l = lane % LN;
+            for (int i0 = r0 + w * RPW; i0 < r1; i0 += kTopWarps * RPW) {
                 const int i = i0 + sub;
                 double acc[R] = {}, acc2[R] = {};   // two chains of dependent multiply-adds
                 if (i < r1) {
                     const double *mrow = Mk + (int64_t)(i - r0) * bo;
                     int j = l;
-                    for (; j + kRowLanes < bo; j += 2 * kRowLanes) {
-                        const double m = mrow[j], m2 = mrow[j + kRowLanes];
+                    for (; j + LN < bo; j += 2 * LN) {
+                        const double m = mrow[j], m2 = mrow[j + LN];
 #pragma unroll
                         for (int r = 0; r < R; ++r) {
                             acc[r] = fma(m, vs[(size_t)(o0 + j) * R + r], acc[r]);
-                            acc2[r] = fma(m2, vs[(size_t)(o0 + j + kRowLanes) * R + r], acc2[r]);
+                            acc2[r] = fma(m2, vs[(size_t)(o0 + j + LN) * R + r], acc2[r]);
                         }
                     }
                     if (j < bo) {
@@ -712,16 +717,25 @@ __global__ void __launch_bounds__(kTopThreads) k_top_chain(TopBandArgs a, const 
 #pragma unroll
                     for (int r = 0; r < R; ++r) acc[r] += acc2[r];
                 }
+                double v = acc[0];
+                int rr = l;                         // the right-hand side this lane writes, if < R
+                if constexpr (R == 2) {
+                    const bool up = (l & (LN / 2)) != 0;
+                    v = (up ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[1], LN / 2);
 #pragma unroll
-                for (int r = 0; r < R; ++r)
+                    for (int o = LN / 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    rr = (l & (LN / 2 - 1)) == 0 ? (up ? 1 : 0) : R;
+                } else {
 #pragma unroll
-                    for (int o = kRowLanes / 2; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
-                if (i < r1 && l < R) {
-                    double v = 0.0;
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int o = LN / 2; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
 #pragma unroll
                     for (int r = 0; r < R; ++r)
                         if (l == r) v = acc[r];
-                    double *dst = vs + (size_t)(b0 + i) * R + l;
+                }
+                if (i < r1 && rr < R) {
+                    double *dst = vs + (size_t)(b0 + i) * R + rr;
                     st_async_all(dst, *dst - v, &bars[2 + s]);
                 }
             }
@@ -763,8 +777,12 @@ template <int R, bool FWD> void launch_chain(const TopBandArgs &a, const double 
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const cudaError_t e = staged ? cudaLaunchKernelEx(&cfg, k_top_chain<R, FWD, true>, a, in, out)
-                                 : cudaLaunchKernelEx(&cfg, k_top_chain<R, FWD, false>, a, in, out);
+    const bool wide = (a.bmax + kTopCluster - 1) / kTopCluster <= 2 * kTopWarps;   // two rows a warp with sixteen lanes
+    const cudaError_t e =
+        staged ? (wide ? cudaLaunchKernelEx(&cfg, k_top_chain<R, FWD, true, 16>, a, in, out)
+                       : cudaLaunchKernelEx(&cfg, k_top_chain<R, FWD, true, 8>, a, in, out))
+               : (wide ? cudaLaunchKernelEx(&cfg, k_top_chain<R, FWD, false, 16>, a, in, out)
+                       : cudaLaunchKernelEx(&cfg, k_top_chain<R, FWD, false, 8>, a, in, out));
     if (e != cudaSuccess)
         throw Error(BDDC_E_CUDA, std::string("launch of the top-level recurrence: ") + cudaGetErrorString(e));
 }
@@ -849,7 +867,9 @@ void launch_identity(int n, double *I, cudaStream_t s) {
 void prepare_top_kernels() {
     cudaFuncSetAttribute(k_band_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPotrfSmem);
     const int big = (int)kTopSmemMax;
-#define BDDC_TOP_ATTR(R, F, S) cudaFuncSetAttribute(k_top_chain<R, F, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, big)
+#define BDDC_TOP_ATTR(R, F, S)                                                                     \
+    cudaFuncSetAttribute(k_top_chain<R, F, S, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, big); \
+    cudaFuncSetAttribute(k_top_chain<R, F, S, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, big)
     BDDC_TOP_ATTR(1, true, true); BDDC_TOP_ATTR(2, true, true); BDDC_TOP_ATTR(4, true, true);
     BDDC_TOP_ATTR(1, false, true); BDDC_TOP_ATTR(2, false, true); BDDC_TOP_ATTR(4, false, true);
     BDDC_TOP_ATTR(1, true, false); BDDC_TOP_ATTR(2, true, false); BDDC_TOP_ATTR(4, true, false);
