@@ -445,7 +445,7 @@ __device__ __forceinline__ void finish_rz(double tot, PcgScalars *sc, double *be
 }
 // The block's warps meet once (warps past the last substructure have left),
 // warp 0 adds their partials, and the block that finishes last adds the
-// blocks', eight loads in flight per lane.  One fence, one atomic and one
+// blocks', sixteen loads in flight per lane.  One fence, one atomic and one
 // partial per block: with one of each per substructure, the 16384
 // substructures of the 1024^2 three-level problem ended in a serial chain of
 // 512 loads and adds (a solve of 45 iterations 14.88 ms, now 13.80).
@@ -469,11 +469,12 @@ __device__ __forceinline__ void block_rz(double acc, const RzArgs &rz, unsigned 
     __threadfence();
     t = 0.0;
     const int nb = (int)gridDim.x;
-    for (int k = lane; k < nb; k += 8 * 32) {
-        double v[8];
+    for (int k = lane; k < nb; k += 16 * 32) {
+        double v[16];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = k + 32 * u < nb ? __ldcg(&rz.part[k + 32 * u]) : 0.0;
-        t += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        for (int u = 0; u < 16; ++u) v[u] = k + 32 * u < nb ? __ldcg(&rz.part[k + 32 * u]) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 16; u += 4) t += (v[u] + v[u + 1]) + (v[u + 2] + v[u + 3]);
     }
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if (lane == 0) {
@@ -503,7 +504,22 @@ template <int LPR, class ACC> __device__ __forceinline__ ACC lpr_sum(ACC v) {
 // record (interior / interface ids, coupling A_{Gamma I}, owned entries) is
 // held in registers: nI <= 256, nG <= 128, coupling entries <= 256.
 // ----------------------------------------------------------------------------
-constexpr int kUI = 8, kUG = 4, kUC = 8, kUO = 4;   // record entries per lane
+constexpr int kUI = 8, kUG = 4, kUC = 8, kUO = 4;   // record entries per lane, at most
+// Record entries per lane by size class: the registers they take limit the
+// warps of an SM (80 a thread for the largest, 16 warps; 1024^2 three-level FP32 solve
+// 13.05 -> 8.6 ms together with the blocks of eight warps, k_dir_w 101 + 46 ->
+// 41 + 34 us an iteration over both levels).
+__host__ __device__ constexpr int ui_of(int cls) { return cls == 0 ? 2 : kUI; }
+__host__ __device__ constexpr int ug_of(int cls) { return cls == 0 ? 1 : (cls == 1 ? 2 : kUG); }
+__host__ __device__ constexpr int uc_of(int cls) { return cls == 0 ? 4 : kUC; }
+__host__ __device__ constexpr int uo_of(int cls) { return cls == 2 ? kUO : 1; }
+inline int dir_class(const DevLevel &L) {
+    for (int c = 0; c < 2; ++c)
+        if (L.max_m * L.max_b <= 32 * ui_of(c) && L.max_nG <= 32 * ug_of(c) && L.max_coo <= 32 * uc_of(c) &&
+            L.max_own <= 32 * uo_of(c))
+            return c;
+    return 2;
+}
 constexpr int kChunks = 4;                          // bulk copies per factor
 // Where a wave of substructures does not fit the SMs with whole factors (FP64
 // blocks of 16 rows: 61 KB each, three warps per SM and three waves on the
@@ -524,10 +540,11 @@ template <class T, class ACC, int BP, int RING> struct DirSlice {
     }
 };
 
-template <class T, class ACC, int BP, bool POST, int RING>
+template <class T, class ACC, int BP, bool POST, int RING, int CLS>
 __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip, unsigned slice,
                         RzArgs rz) {
     constexpr int LPR = 32 / BP;
+    constexpr int UI = ui_of(CLS), UG = ug_of(CLS), UC = uc_of(CLS), UO = uo_of(CLS);
     constexpr int NC = BP / LPR;
     constexpr int BB = BP * BP;
     extern __shared__ __align__(16) unsigned char smem_w[];
@@ -589,21 +606,21 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     const int *gP = reinterpret_cast<const int *>(rec + lay.pr);
     const double *gC = reinterpret_cast<const double *>(rec + lay.cv);
     const int *gO = reinterpret_cast<const int *>(rec + lay.ow);
-    int ii[kUI], ig[kUG], pr[kUC], owp[kUO], owd[kUO];
-    ACC cv[kUC];
+    int ii[UI], ig[UG], pr[UC], owp[UO], owd[UO];
+    ACC cv[UC];
 #pragma unroll
-    for (int u = 0; u < kUI; ++u) { const int i = u * 32 + lane; ii[u] = i < nI ? gI[i] : -1; }
+    for (int u = 0; u < UI; ++u) { const int i = u * 32 + lane; ii[u] = i < nI ? gI[i] : -1; }
 #pragma unroll
-    for (int u = 0; u < kUG; ++u) { const int q = u * 32 + lane; ig[u] = q < nG ? gGi[q] : -1; }
+    for (int u = 0; u < UG; ++u) { const int q = u * 32 + lane; ig[u] = q < nG ? gGi[q] : -1; }
 #pragma unroll
-    for (int u = 0; u < kUC; ++u) {
+    for (int u = 0; u < UC; ++u) {
         const int k = u * 32 + lane;
         pr[u] = k < ncoo ? gP[k] : -1;
-        cv[u] = k < ncoo ? (ACC)gC[k] : (ACC)0;
+        cv[u] = k < ncoo ? from_f64<ACC>(gC[k]) : (ACC)0;
     }
     if (POST) {
 #pragma unroll
-        for (int u = 0; u < kUO; ++u) {
+        for (int u = 0; u < UO; ++u) {
             const int k = u * 32 + lane;
             owp[u] = k < nown ? gO[2 * k] : -1;
             owd[u] = k < nown ? gO[2 * k + 1] : -1;
@@ -618,27 +635,27 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
         return;
     }
     // right-hand side (and u_B on Gamma for the post-correction)
-    double rv[kUI];
+    double rv[UI];
 #pragma unroll
-    for (int u = 0; u < kUI; ++u) rv[u] = ii[u] >= 0 ? r[ii[u]] : 0.0;
+    for (int u = 0; u < UI; ++u) rv[u] = ii[u] >= 0 ? r[ii[u]] : 0.0;
 #pragma unroll
-    for (int u = 0; u < kUI; ++u) {
+    for (int u = 0; u < UI; ++u) {
         const int i = u * 32 + lane;
-        if (i < m * BP) x[i] = (ACC)rv[u];
+        if (i < m * BP) x[i] = from_f64<ACC>(rv[u]);
     }
     if (POST) {
-        double uv[kUG];
+        double uv[UG];
 #pragma unroll
-        for (int u = 0; u < kUG; ++u) uv[u] = ig[u] >= 0 ? L.uB[ig[u]] : 0.0;
+        for (int u = 0; u < UG; ++u) uv[u] = ig[u] >= 0 ? L.uB[ig[u]] : 0.0;
 #pragma unroll
-        for (int u = 0; u < kUG; ++u) if (ig[u] >= 0) vG[u * 32 + lane] = (ACC)uv[u];
+        for (int u = 0; u < UG; ++u) if (ig[u] >= 0) vG[u * 32 + lane] = from_f64<ACC>(uv[u]);
         __syncwarp();
 #pragma unroll
-        for (int u = 0; u < kUC; ++u)
+        for (int u = 0; u < UC; ++u)
             if (pr[u] >= 0) atomicAdd(&x[pr[u] & 0xffff], -cv[u] * vG[pr[u] >> 16]);
     } else {
 #pragma unroll
-        for (int u = 0; u < kUG; ++u) {
+        for (int u = 0; u < UG; ++u) {
             if (ig[u] >= 0) {
                 vG[u * 32 + lane] = 0;
                 L.uB[ig[u]] = 0.0;   // consumed by the previous post-correction
@@ -724,30 +741,30 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     __syncwarp();
     if (!POST) {
 #pragma unroll
-        for (int u = 0; u < kUC; ++u)
+        for (int u = 0; u < UC; ++u)
             if (pr[u] >= 0) atomicAdd(&vG[pr[u] >> 16], cv[u] * x[pr[u] & 0xffff]);
         __syncwarp();
 #pragma unroll
-        for (int u = 0; u < kUG; ++u) {
+        for (int u = 0; u < UG; ++u) {
             if (ig[u] >= 0) {
                 const ACC v = vG[u * 32 + lane];
-                if (v != (ACC)0) atomicAdd(&L.rB[ig[u]], -(double)v);
+                if (v != (ACC)0) atomicAdd(&L.rB[ig[u]], -to_f64(v));
             }
         }
     } else {
         double acc = 0.0;
 #pragma unroll
-        for (int u = 0; u < kUI; ++u) {
+        for (int u = 0; u < UI; ++u) {
             if (ii[u] >= 0) {
-                const double zv = (double)x[u * 32 + lane];
+                const double zv = to_f64(x[u * 32 + lane]);
                 z[ii[u]] = zv;
                 acc = fma(rv[u], zv, acc);
             }
         }
 #pragma unroll
-        for (int u = 0; u < kUO; ++u) {
+        for (int u = 0; u < UO; ++u) {
             if (owp[u] >= 0) {
-                const double zv = (double)vG[owp[u]];
+                const double zv = to_f64(vG[owp[u]]);
                 z[owd[u]] = zv;
                 if (rz.sc) acc = fma(r[owd[u]], zv, acc);
             }
@@ -805,7 +822,7 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int q = q0 + u * 32 + lane;
-            if (q < nG) f[q] = ld<T, ACC>(wg + q) * (ACC)v[u];
+            if (q < nG) f[q] = ld<T, ACC>(wg + q) * from_f64<ACC>(v[u]);
         }
     }
     __syncwarp();
@@ -818,7 +835,7 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
             s1 += ld<T, ACC>(Ns + (size_t)(pp + 1) * lay.ld + q) * f[pp + 1];
         }
         if (pp < nG) s0 += ld<T, ACC>(Ns + (size_t)pp * lay.ld + q) * f[pp];
-        L.w[g0 + q] = (double)(s0 + s1);
+        L.w[g0 + q] = to_f64(s0 + s1);
     }
     // coarse right-hand side: lane k sums row k of Psi^T, staggered to avoid bank conflicts
     for (int k = lane; k < nc; k += 32) {
@@ -827,7 +844,7 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
             const int q = (t + k) % nG;
             s0 += ld<T, ACC>(Ps + (size_t)k * lay.ld + q) * f[q];
         }
-        atomicAdd(&L.rcv[rcs[k]], (double)s0);
+        atomicAdd(&L.rcv[rcs[k]], to_f64(s0));
     }
 }
 
@@ -868,12 +885,12 @@ __global__ void k_average_r(DevLevel L, int pidx, const int *skip, unsigned slic
     const T *wg = reinterpret_cast<const T *>(rec + lay.wg);
     const int *iG = reinterpret_cast<const int *>(rec + lay.iG);
     const int *rcs = reinterpret_cast<const int *>(rec + lay.rc);
-    for (int k = lane; k < nc; k += 32) uc[k] = (ACC)L.ucv[rcs[k]];
+    for (int k = lane; k < nc; k += 32) uc[k] = from_f64<ACC>(L.ucv[rcs[k]]);
     __syncwarp();
     for (int q = lane; q < nG; q += 32) {
-        ACC v = (q < 128) ? (ACC)wv[q >> 5] : (ACC)L.w[g0 + q];
+        ACC v = from_f64<ACC>((q < 128) ? wv[q >> 5] : L.w[g0 + q]);
         for (int k = 0; k < nc; ++k) v += ld<T, ACC>(Ps + (size_t)k * lay.ld + q) * uc[k];
-        atomicAdd(&L.uB[iG[q]], (double)(ld<T, ACC>(wg + q) * v));
+        atomicAdd(&L.uB[iG[q]], to_f64(ld<T, ACC>(wg + q) * v));
         L.rB[iG[q]] = 0.0;            // consumed by the substructure correction
     }
     for (int k = lane; k < nc; k += 32) L.rcv[rcs[k]] = 0.0;   // consumed by the coarse solve
@@ -1455,27 +1472,38 @@ constexpr size_t kSmemBudget = kSmemMax;
 int num_sms() { return device_sms(); }
 
 // Warps (substructures) per block: as many as needed for one wave over the
-// SMs, limited by the shared-memory slices that fit in one block.
+// SMs, limited by the shared-memory slices that fit in one block; eight where
+// that takes several waves (three blocks of them share an SM's registers,
+// where one block of sixteen leaves almost half unused, and they end one by
+// one).
 int warps_per_block(int nsub, size_t slice) {
     const int fit = (int)(kSmemMax / slice);
     int want = (nsub + num_sms() - 1) / num_sms();
     if (want < 4) want = 4;
+    if (want > 16) want = 8;
     int w = want < fit ? want : fit;
-    if (w > 16) w = 16;
     return w < 1 ? 1 : w;
 }
 
-template <class T, class ACC, int BP, int RING>
-void dir_launch_r(const DevLevel &L, bool post, const double *r, double *z, const int *skip,
+template <class T, class ACC, int BP, int RING, int CLS>
+void dir_launch_c(const DevLevel &L, bool post, const double *r, double *z, const int *skip,
                   cudaStream_t s, const RzArgs *rz) {
     const size_t slice = DirSlice<T, ACC, BP, RING>::bytes(L);
     const int wpc = warps_per_block(L.nsub, slice);
     const size_t sm = slice * wpc;
     const int grid = (L.nsub + wpc - 1) / wpc;
     const RzArgs none{nullptr, nullptr, nullptr, nullptr};
-    if (!post) launch_pdl(k_dir_w<T, ACC, BP, false, RING>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice, none);
-    else launch_pdl(k_dir_w<T, ACC, BP, true, RING>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice,
+    if (!post) launch_pdl(k_dir_w<T, ACC, BP, false, RING, CLS>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice, none);
+    else launch_pdl(k_dir_w<T, ACC, BP, true, RING, CLS>, grid, 32 * wpc, sm, s, L, r, z, skip, (unsigned)slice,
                     rz ? *rz : none);
+}
+template <class T, class ACC, int BP, int RING>
+void dir_launch_r(const DevLevel &L, bool post, const double *r, double *z, const int *skip,
+                  cudaStream_t s, const RzArgs *rz) {
+    const int cls = dir_class(L);
+    if (cls == 0) dir_launch_c<T, ACC, BP, RING, 0>(L, post, r, z, skip, s, rz);
+    else if (cls == 1) dir_launch_c<T, ACC, BP, RING, 1>(L, post, r, z, skip, s, rz);
+    else dir_launch_c<T, ACC, BP, RING, 2>(L, post, r, z, skip, s, rz);
 }
 // The ring where whole factors would take more waves than it does: with one
 // wave either way, the whole factor saves the second read of its blocks.
@@ -1547,14 +1575,16 @@ bool warp_path(const DevLevel &L, int prec) {
 void prepare_apply_kernels() {
     const int big = (int)kSmemMax;
 #define BDDC_SMEM_ATTR(k) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, big)
-#define BDDC_DIR_W(T, A, BP, R)                          \
-    BDDC_SMEM_ATTR((k_dir_w<T, A, BP, false, R>));       \
-    BDDC_SMEM_ATTR((k_dir_w<T, A, BP, true, R>));
+#define BDDC_DIR_WC(T, A, BP, R, C)                      \
+    BDDC_SMEM_ATTR((k_dir_w<T, A, BP, false, R, C>));    \
+    BDDC_SMEM_ATTR((k_dir_w<T, A, BP, true, R, C>));
+#define BDDC_DIR_W(T, A, BP, R) BDDC_DIR_WC(T, A, BP, R, 0) BDDC_DIR_WC(T, A, BP, R, 1) BDDC_DIR_WC(T, A, BP, R, 2)
     BDDC_DIR_W(double, double, 8, 0) BDDC_DIR_W(double, double, 16, 0) BDDC_DIR_W(double, double, 32, 0)
     BDDC_DIR_W(double, double, 8, kDWRing) BDDC_DIR_W(double, double, 16, kDWRing) BDDC_DIR_W(double, double, 32, kDWRing)
     BDDC_DIR_W(float, float, 8, 0) BDDC_DIR_W(float, float, 16, 0) BDDC_DIR_W(float, float, 32, 0)
     BDDC_DIR_W(__nv_bfloat16, float, 8, 0) BDDC_DIR_W(__nv_bfloat16, float, 16, 0) BDDC_DIR_W(__nv_bfloat16, float, 32, 0)
 #undef BDDC_DIR_W
+#undef BDDC_DIR_WC
     BDDC_SMEM_ATTR((k_dir_s<double, double, false>));
     BDDC_SMEM_ATTR((k_dir_s<double, double, true>));
     BDDC_SMEM_ATTR((k_dir_s<float, float, false>));
