@@ -150,163 +150,179 @@ __global__ void __launch_bounds__(kGT) k_pre(DevLevel L, const double *r, const 
 }
 
 // Dirichlet solves of large or irregular substructures (no block size the
-// warp kernels take): one block of kSB threads per substructure streams the
-// factor blocks [Linv_j | L_{j,j-1}] through a ring of kNS shared-memory
-// stages with bulk copies (block i always in stage i % kNS), so the copies of
-// the next blocks overlap the solve of the current one.  The forward sweep
-// refills a stage as soon as its block is used; the backward sweep starts
-// from the kNS blocks the forward sweep left in the ring and refills the
-// stage of block j+1 after step j (the last step that needs L_{j+1,j}).
-// kTPR threads share a row of a block solve (column-strided partial sums,
-// shuffle-reduced).  Every wait is bounded; a block whose wait gives up
-// flags *L.err, lets its copies land (bounded) and leaves.
-constexpr int kSB = 256, kNS = 3, kTPR = 4;
+// warp kernels take): one block per substructure streams the factor through a
+// ring of shared-memory slots with bulk copies.  The unit is half a block: the
+// forward sweep uses Linv_0, Lsub_1, Linv_1, Lsub_2, ... and the backward
+// sweep the same sequence in reverse, so half s sits in slot s mod ring, is
+// replaced by half s + ring (s - ring on the way back) as soon as it is used,
+// and the sweeps turn round on the halves left in the ring.  Two slots are
+// enough to run, so blocks of up to about 160 rows in FP32 fit; four are used
+// where they do.  kTPR threads share a row of a block solve (column-strided
+// partial sums, shuffle-reduced).  Every wait is bounded; a thread whose wait
+// gives up waits no more, the block flags *L.err, lets its copies land
+// (bounded) and leaves.
+// Nine level-2 substructures of the 384^2 elasticity problem: 30 + 30 -> 23 + 19 us.
+constexpr int kSB = 256, kSBWide = 512, kNS = 4, kTPR = 4;
 
 struct StreamSmem {
     size_t stage, x, tmp, vg, total;
-    template <class T, class ACC> __host__ __device__ static StreamSmem of(const DevLevel &L) {
+    template <class T, class ACC> __host__ __device__ static StreamSmem of(const DevLevel &L, int ring) {
         StreamSmem m;
         const size_t mb = L.max_b > 0 ? L.max_b : 1, mld = L.max_ld > 0 ? L.max_ld : 1;
-        m.stage = al16(2 * mb * mld * sizeof(T) + 32);       // plus slack to align each copy
+        m.stage = al16(mb * mld * sizeof(T) + 32);       // plus slack to align each copy
         m.x = al16(sizeof(ACC) * (size_t)(L.max_m > 0 ? L.max_m : 1) * mb);
         m.tmp = al16(sizeof(ACC) * mb);
         m.vg = al16(sizeof(ACC) * (size_t)(L.max_nG > 0 ? L.max_nG : 1));
-        m.total = kNS * m.stage + m.x + m.tmp + m.vg + 8 * kNS + 16;
+        m.total = ring * m.stage + m.x + m.tmp + m.vg + 8 * kNS + 16;
         return m;
     }
 };
 
 template <class T, class ACC, bool POST>
-__global__ void __launch_bounds__(kSB) k_dir_s(DevLevel L, const double *r, double *z, const int *skip) {
+__global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, double *z, const int *skip,
+                                                   int ring) {
     pdl_wait();
     pdl_trigger();
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem_s[];
-    const StreamSmem ly = StreamSmem::of<T, ACC>(L);
-    unsigned char *ring = smem_s;
-    ACC *x = reinterpret_cast<ACC *>(smem_s + kNS * ly.stage);
+    const StreamSmem ly = StreamSmem::of<T, ACC>(L, ring);
+    ACC *x = reinterpret_cast<ACC *>(smem_s + ring * ly.stage);
     ACC *tmp = reinterpret_cast<ACC *>(reinterpret_cast<unsigned char *>(x) + ly.x);
     ACC *vG = reinterpret_cast<ACC *>(reinterpret_cast<unsigned char *>(tmp) + ly.tmp);
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(vG) + ly.vg);
-    const int sub = blockIdx.x, tid = threadIdx.x;
+    const int sub = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
     const int nI = L.nI[sub], nG = L.nG[sub], b = L.bsz[sub], m = nI > 0 ? L.nblk[sub] : 0;
     const bool swz = L.bp != 0;
     const OpSet<T> &O = Ops<T>::get(L);
     const T *F = O.dir + L.offF[sub];
     const int ldb = fld(b, swz);
-    const size_t bb2 = 2 * (size_t)b * ldb;
-    // block i: its bytes rounded out to 16-byte boundaries, and where it starts in its stage
-    auto issue = [&](int i) {
-        const uintptr_t a = reinterpret_cast<uintptr_t>(F + (size_t)i * bb2);
+    const size_t bsq = (size_t)b * ldb;
+    const int ns = 2 * m - 1;
+    unsigned par = 0, pend = 0;           // bit q: parity of slot q's next phase; a copy in flight (thread 0)
+    bool ok = true;
+    // half s (2 j: Linv_j, 2 j - 1: Lsub_j): its bytes rounded out to 16-byte
+    // boundaries, and where it starts in its slot
+    auto half_of = [&](int s) { return F + ((size_t)(s + 1) / 2 * 2 + (s & 1)) * bsq; };
+    auto issue = [&](int s) {
+        const int q = s % ring;
+        const uintptr_t a = reinterpret_cast<uintptr_t>(half_of(s));
         const uintptr_t al = a & ~uintptr_t(15);
-        const uintptr_t ae = (a + bb2 * sizeof(T) + 15) & ~uintptr_t(15);
-        mbar_expect(&bars[i % kNS], (unsigned)(ae - al));
-        bulk_copy(ring + (size_t)(i % kNS) * ly.stage, reinterpret_cast<const void *>(al), (unsigned)(ae - al),
-                  &bars[i % kNS]);
+        const uintptr_t ae = (a + bsq * sizeof(T) + 15) & ~uintptr_t(15);
+        mbar_expect(&bars[q], (unsigned)(ae - al));
+        bulk_copy(smem_s + (size_t)q * ly.stage, reinterpret_cast<const void *>(al), (unsigned)(ae - al), &bars[q]);
+        pend |= 1u << q;
     };
-    auto blk = [&](int i) {
-        const uintptr_t a = reinterpret_cast<uintptr_t>(F + (size_t)i * bb2);
-        return reinterpret_cast<const T *>(ring + (size_t)(i % kNS) * ly.stage + (a & 15));
+    auto slot = [&](int s) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(half_of(s));
+        return reinterpret_cast<const T *>(smem_s + (size_t)(s % ring) * ly.stage + (a & 15));
+    };
+    auto wait_half = [&](int s) {         // every thread sees the copy's completion itself
+        const int q = s % ring;
+        if (ok) {
+            ok = mbar_wait(&bars[q], (par >> q) & 1u);
+            if (ok) pend &= ~(1u << q);
+        }
+        par ^= 1u << q;
     };
     if (tid == 0) {
-        for (int s = 0; s < kNS; ++s) mbar_init(&bars[s]);
-        for (int i = 0; i < kNS && i < m; ++i) issue(i);
+        for (int q = 0; q < ring; ++q) mbar_init(&bars[q]);
+        for (int s = 0; s < ring && s < ns; ++s) issue(s);
     }
     const int *iI = L.idxI + L.offI[sub];
     const int *iG = L.idxG + L.offG[sub];
-    for (int i = tid; i < m * b; i += kSB) x[i] = i < nI ? (ACC)r[iI[i]] : (ACC)0;
+    for (int i = tid; i < m * b; i += nt) x[i] = i < nI ? from_f64<ACC>(r[iI[i]]) : (ACC)0;
     if (POST) {
-        for (int q = tid; q < nG; q += kSB) vG[q] = (ACC)L.uB[iG[q]];
+        for (int q = tid; q < nG; q += nt) vG[q] = from_f64<ACC>(L.uB[iG[q]]);
         __syncthreads();
-        for (int64_t k = L.offCOO[sub] + tid; k < L.offCOO[sub + 1]; k += kSB)
+        for (int64_t k = L.offCOO[sub] + tid; k < L.offCOO[sub + 1]; k += nt)
             atomicAdd(&x[L.cooI[k]], -ld<T, ACC>(O.aig + k) * vG[L.cooG[k]]);
     } else {
-        for (int q = tid; q < nG; q += kSB) vG[q] = 0;
+        for (int q = tid; q < nG; q += nt) vG[q] = 0;
     }
     __syncthreads();
-    unsigned par = 0;                     // bit s: parity of the next phase of stage s
-    const int part = tid % kTPR, r0 = tid / kTPR;
-    constexpr int RPP = kSB / kTPR;       // rows per pass
-    bool ok = true;
-    auto wait_block = [&](int i) {
-        const int s = i % kNS;
-        const bool got = mbar_wait(&bars[s], (par >> s) & 1u);
-        par ^= 1u << s;
-        return __syncthreads_and(got) != 0;
-    };
-    for (int j = 0; j < m && ok; ++j) {
-        if (!wait_block(j)) { ok = false; break; }
-        const T *Li = blk(j), *Ls = Li + (size_t)b * ldb;
+    const int part = tid % kTPR, r0 = tid / kTPR, RPP = nt / kTPR;   // rows per pass
+    // row sums of M v (TR: of its transpose) over the columns [c0(row), c1(row))
+    auto rows = [&](auto &&entry, const ACC *v, auto &&lo, auto &&hi, auto &&put) {
         for (int pass = 0; pass * RPP < b; ++pass) {      // the same passes in every thread
             const int rr = r0 + pass * RPP;
-            ACC a = 0;
-            if (rr < b && j > 0)
-                for (int c = part; c < b; c += kTPR)
-                    a += ld<T, ACC>(Ls + fpos(rr, c, ldb, swz)) * x[(j - 1) * b + c];
-#pragma unroll
-            for (int o = kTPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (rr < b && part == 0) tmp[rr] = x[j * b + rr] - a;
-        }
-        __syncthreads();
-        for (int pass = 0; pass * RPP < b; ++pass) {
-            const int rr = r0 + pass * RPP;
-            ACC a = 0;
-            if (rr < b)
-                for (int c = part; c <= rr; c += kTPR) a += ld<T, ACC>(Li + fpos(rr, c, ldb, swz)) * tmp[c];
-#pragma unroll
-            for (int o = kTPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (rr < b && part == 0) x[j * b + rr] = a;
-        }
-        __syncthreads();
-        if (tid == 0 && j + kNS < m) issue(j + kNS);
-    }
-    for (int j = m - 1; j >= 0 && ok; --j) {
-        if (j < m - kNS && !wait_block(j)) { ok = false; break; }
-        const T *Li = blk(j);
-        for (int pass = 0; pass * RPP < b; ++pass) {
-            const int rr = r0 + pass * RPP;
-            ACC a = 0;
-            if (rr < b && j < m - 1) {
-                const T *Ls1 = blk(j + 1) + (size_t)b * ldb;     // L_{j+1,j}^T: entry (rr, c) is (c, rr)
-                for (int c = part; c < b; c += kTPR)
-                    a += ld<T, ACC>(Ls1 + fpos(c, rr, ldb, swz)) * x[(j + 1) * b + c];
+            ACC a = 0, a2 = 0;
+            if (rr < b) {
+                const int c1 = hi(rr);
+                int c = lo(rr) + part;
+                for (; c + kTPR < c1; c += 2 * kTPR) {
+                    a += entry(rr, c) * v[c];
+                    a2 += entry(rr, c + kTPR) * v[c + kTPR];
+                }
+                if (c < c1) a += entry(rr, c) * v[c];
             }
+            a += a2;
 #pragma unroll
             for (int o = kTPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (rr < b && part == 0) tmp[rr] = x[j * b + rr] - a;
+            if (rr < b && part == 0) put(rr, a);
         }
-        __syncthreads();
-        for (int pass = 0; pass * RPP < b; ++pass) {
-            const int rr = r0 + pass * RPP;
-            ACC a = 0;
-            if (rr < b)
-                for (int c = rr + part; c < b; c += kTPR) a += ld<T, ACC>(Li + fpos(c, rr, ldb, swz)) * tmp[c];
-#pragma unroll
-            for (int o = kTPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (rr < b && part == 0) x[j * b + rr] = a;
+    };
+    auto zero = [](int) { return 0; };
+    auto all = [&](int) { return b; };
+    auto self = [](int rr) { return rr; };
+    auto next = [](int rr) { return rr + 1; };
+    for (int j = 0; j < m; ++j) {
+        ACC *xj = x + j * b;
+        if (j > 0) {
+            wait_half(2 * j - 1);
+            const T *Ls = slot(2 * j - 1);
+            rows([&](int rr, int c) { return ld<T, ACC>(Ls + fpos(rr, c, ldb, swz)); }, xj - b, zero, all,
+                 [&](int rr, ACC a) { tmp[rr] = xj[rr] - a; });
+        } else {
+            for (int rr = tid; rr < b; rr += nt) tmp[rr] = xj[rr];
         }
+        wait_half(2 * j);
         __syncthreads();
-        // block j+1 is no longer needed: its stage takes block j+1-kNS
-        if (tid == 0 && j + 1 < m && j + 1 - kNS >= 0 && j + 1 - kNS < m - kNS) issue(j + 1 - kNS);
+        if (tid == 0 && ok && j > 0 && 2 * j - 1 + ring < ns) issue(2 * j - 1 + ring);
+        const T *Li = slot(2 * j);
+        rows([&](int rr, int c) { return ld<T, ACC>(Li + fpos(rr, c, ldb, swz)); }, tmp, zero, next,
+             [&](int rr, ACC a) { xj[rr] = a; });
+        __syncthreads();
+        if (tid == 0 && ok && 2 * j + ring < ns) issue(2 * j + ring);
     }
-    if (!ok) {
+    for (int j = m - 1; j >= 0; --j) {
+        ACC *xj = x + j * b;
+        if (j < m - 1) {
+            const int s = 2 * j + 1;                      // L_{j+1,j}^T: entry (rr, c) is (c, rr)
+            if (s < ns - ring) wait_half(s);
+            const T *Ls1 = slot(s);
+            rows([&](int rr, int c) { return ld<T, ACC>(Ls1 + fpos(c, rr, ldb, swz)); }, xj + b, zero, all,
+                 [&](int rr, ACC a) { tmp[rr] = xj[rr] - a; });
+        } else {
+            for (int rr = tid; rr < b; rr += nt) tmp[rr] = xj[rr];
+        }
+        if (2 * j < ns - ring) wait_half(2 * j);
+        __syncthreads();
+        if (tid == 0 && ok && j < m - 1 && 2 * j + 1 - ring >= 0) issue(2 * j + 1 - ring);
+        const T *Li = slot(2 * j);
+        rows([&](int rr, int c) { return ld<T, ACC>(Li + fpos(c, rr, ldb, swz)); }, tmp, self, all,
+             [&](int rr, ACC a) { xj[rr] = a; });
+        __syncthreads();
+        if (tid == 0 && ok && 2 * j - ring >= 0) issue(2 * j - ring);
+    }
+    if (!__syncthreads_and(ok)) {
         if (tid == 0) {
             atomicExch(L.err, 1);
-            for (int s = 0; s < kNS; ++s) mbar_wait(&bars[s], (par >> s) & 1u);   // bounded
+            for (int q = 0; q < ring; ++q)                // bounded: copies in flight land first
+                if ((pend >> q) & 1u) mbar_wait(&bars[q], (par >> q) & 1u);
         }
         return;
     }
     if (!POST) {
-        for (int64_t k = L.offCOO[sub] + tid; k < L.offCOO[sub + 1]; k += kSB)
+        for (int64_t k = L.offCOO[sub] + tid; k < L.offCOO[sub + 1]; k += nt)
             atomicAdd(&vG[L.cooG[k]], ld<T, ACC>(O.aig + k) * x[L.cooI[k]]);
         __syncthreads();
-        for (int q = tid; q < nG; q += kSB) {
-            if (vG[q] != (ACC)0) atomicAdd(&L.rB[iG[q]], -(double)vG[q]);
+        for (int q = tid; q < nG; q += nt) {
+            if (vG[q] != (ACC)0) atomicAdd(&L.rB[iG[q]], -to_f64(vG[q]));
             L.uB[iG[q]] = 0.0;   // consumed by the previous post-correction
         }
     } else {
-        for (int i = tid; i < nI; i += kSB) z[iI[i]] = (double)x[i];
-        for (int64_t k = L.offOwn[sub] + tid; k < L.offOwn[sub + 1]; k += kSB) {
+        for (int i = tid; i < nI; i += nt) z[iI[i]] = to_f64(x[i]);
+        for (int64_t k = L.offOwn[sub] + tid; k < L.offOwn[sub + 1]; k += nt) {
             const int id = L.own[k];
             z[L.ifaceDof[id]] = L.uB[id];
         }
@@ -372,9 +388,11 @@ __global__ void __launch_bounds__(32 * kNWarps) k_neumann(DevLevel L, const doub
     }
 }
 
-// (9): u_B = sum_i R_i^T D_i (w_i + Psi_i u_c).
+// (9): u_B = sum_i R_i^T D_i (w_i + Psi_i u_c).  A block takes kARows interface
+// rows of one substructure (blockIdx.y), a thread per row.
+constexpr int kARows = 128;
 template <class T, class ACC>
-__global__ void k_average(DevLevel L, const int *skip) {
+__global__ void __launch_bounds__(kARows) k_average(DevLevel L, const int *skip) {
     pdl_wait();
     pdl_trigger();
     if (skip && *skip) return;
@@ -384,16 +402,20 @@ __global__ void k_average(DevLevel L, const int *skip) {
     const int nG = L.nG[sub], nc = L.ncl[sub];
     const OpSet<T> &O = Ops<T>::get(L);
     const int64_t g0 = L.offG[sub];
-    for (int k = threadIdx.x; k < nc; k += blockDim.x) uc[k] = (ACC)L.ucv[L.rc[L.offC[sub] + k]];
+    if (blockIdx.y > 0 && (int)(blockIdx.y * kARows) >= nG) return;
+    for (int k = threadIdx.x; k < nc; k += blockDim.x) uc[k] = from_f64<ACC>(L.ucv[L.rc[L.offC[sub] + k]]);
     __syncthreads();
     const T *P = O.psit + L.offP[sub];
-    for (int q = threadIdx.x; q < nG; q += blockDim.x) {
-        ACC v = (ACC)L.w[g0 + q];
+    const int q = blockIdx.y * kARows + threadIdx.x;
+    if (q < nG) {
+        ACC v = from_f64<ACC>(L.w[g0 + q]);
+#pragma unroll 4
         for (int k = 0; k < nc; ++k) v += ld<T, ACC>(P + (int64_t)k * nG + q) * uc[k];
-        atomicAdd(&L.uB[L.idxG[g0 + q]], (double)(ld<T, ACC>(O.wg + g0 + q) * v));
+        atomicAdd(&L.uB[L.idxG[g0 + q]], to_f64(ld<T, ACC>(O.wg + g0 + q) * v));
         L.rB[L.idxG[g0 + q]] = 0.0;
     }
-    for (int k = threadIdx.x; k < nc; k += blockDim.x) L.rcv[L.rc[L.offC[sub] + k]] = 0.0;
+    if (blockIdx.y == 0)
+        for (int k = threadIdx.x; k < nc; k += blockDim.x) L.rcv[L.rc[L.offC[sub] + k]] = 0.0;
 }
 
 // (10)-(11): interior of u = A_II^{-1}(r_I - A_{I Gamma} u_B), interface of u = u_B.
@@ -616,7 +638,7 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     for (int u = 0; u < UC; ++u) {
         const int k = u * 32 + lane;
         pr[u] = k < ncoo ? gP[k] : -1;
-        cv[u] = k < ncoo ? from_f64<ACC>(gC[k]) : (ACC)0;
+        cv[u] = k < ncoo ? (ACC)(gC[k]) : (ACC)0;
     }
     if (POST) {
 #pragma unroll
@@ -641,14 +663,14 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
 #pragma unroll
     for (int u = 0; u < UI; ++u) {
         const int i = u * 32 + lane;
-        if (i < m * BP) x[i] = from_f64<ACC>(rv[u]);
+        if (i < m * BP) x[i] = (ACC)(rv[u]);
     }
     if (POST) {
         double uv[UG];
 #pragma unroll
         for (int u = 0; u < UG; ++u) uv[u] = ig[u] >= 0 ? L.uB[ig[u]] : 0.0;
 #pragma unroll
-        for (int u = 0; u < UG; ++u) if (ig[u] >= 0) vG[u * 32 + lane] = from_f64<ACC>(uv[u]);
+        for (int u = 0; u < UG; ++u) if (ig[u] >= 0) vG[u * 32 + lane] = (ACC)(uv[u]);
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < UC; ++u)
@@ -748,7 +770,7 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
         for (int u = 0; u < UG; ++u) {
             if (ig[u] >= 0) {
                 const ACC v = vG[u * 32 + lane];
-                if (v != (ACC)0) atomicAdd(&L.rB[ig[u]], -to_f64(v));
+                if (v != (ACC)0) atomicAdd(&L.rB[ig[u]], -(double)(v));
             }
         }
     } else {
@@ -756,7 +778,7 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
 #pragma unroll
         for (int u = 0; u < UI; ++u) {
             if (ii[u] >= 0) {
-                const double zv = to_f64(x[u * 32 + lane]);
+                const double zv = (double)(x[u * 32 + lane]);
                 z[ii[u]] = zv;
                 acc = fma(rv[u], zv, acc);
             }
@@ -764,7 +786,7 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
 #pragma unroll
         for (int u = 0; u < UO; ++u) {
             if (owp[u] >= 0) {
-                const double zv = to_f64(vG[owp[u]]);
+                const double zv = (double)(vG[owp[u]]);
                 z[owd[u]] = zv;
                 if (rz.sc) acc = fma(r[owd[u]], zv, acc);
             }
@@ -822,7 +844,7 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int q = q0 + u * 32 + lane;
-            if (q < nG) f[q] = ld<T, ACC>(wg + q) * from_f64<ACC>(v[u]);
+            if (q < nG) f[q] = ld<T, ACC>(wg + q) * (ACC)(v[u]);
         }
     }
     __syncwarp();
@@ -835,7 +857,7 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
             s1 += ld<T, ACC>(Ns + (size_t)(pp + 1) * lay.ld + q) * f[pp + 1];
         }
         if (pp < nG) s0 += ld<T, ACC>(Ns + (size_t)pp * lay.ld + q) * f[pp];
-        L.w[g0 + q] = to_f64(s0 + s1);
+        L.w[g0 + q] = (double)(s0 + s1);
     }
     // coarse right-hand side: lane k sums row k of Psi^T, staggered to avoid bank conflicts
     for (int k = lane; k < nc; k += 32) {
@@ -844,7 +866,7 @@ __global__ void k_neumann_r(DevLevel L, int pidx, const double *r, const int *sk
             const int q = (t + k) % nG;
             s0 += ld<T, ACC>(Ps + (size_t)k * lay.ld + q) * f[q];
         }
-        atomicAdd(&L.rcv[rcs[k]], to_f64(s0));
+        atomicAdd(&L.rcv[rcs[k]], (double)(s0));
     }
 }
 
@@ -885,12 +907,12 @@ __global__ void k_average_r(DevLevel L, int pidx, const int *skip, unsigned slic
     const T *wg = reinterpret_cast<const T *>(rec + lay.wg);
     const int *iG = reinterpret_cast<const int *>(rec + lay.iG);
     const int *rcs = reinterpret_cast<const int *>(rec + lay.rc);
-    for (int k = lane; k < nc; k += 32) uc[k] = from_f64<ACC>(L.ucv[rcs[k]]);
+    for (int k = lane; k < nc; k += 32) uc[k] = (ACC)(L.ucv[rcs[k]]);
     __syncwarp();
     for (int q = lane; q < nG; q += 32) {
-        ACC v = from_f64<ACC>((q < 128) ? wv[q >> 5] : L.w[g0 + q]);
+        ACC v = (ACC)((q < 128) ? wv[q >> 5] : L.w[g0 + q]);
         for (int k = 0; k < nc; ++k) v += ld<T, ACC>(Ps + (size_t)k * lay.ld + q) * uc[k];
-        atomicAdd(&L.uB[iG[q]], to_f64(ld<T, ACC>(wg + q) * v));
+        atomicAdd(&L.uB[iG[q]], (double)(ld<T, ACC>(wg + q) * v));
         L.rB[iG[q]] = 0.0;            // consumed by the substructure correction
     }
     for (int k = lane; k < nc; k += 32) L.rcv[rcs[k]] = 0.0;   // consumed by the coarse solve
@@ -1406,9 +1428,16 @@ bool force_generic_dir() {
     const char *e = std::getenv("BDDC_GENERIC_DIR");
     return e && e[0] == '1';
 }
-template <class T, class ACC> bool stream_fits(const DevLevel &L) {
-    return !force_generic_dir() && StreamSmem::of<T, ACC>(L).total <= 227 * 1024;
+// Slots of the streaming kernel's ring, 2 to kNS; 0: not even two fit.
+template <class T, class ACC> int stream_ring(const DevLevel &L) {
+    if (force_generic_dir()) return 0;
+    for (int n = kNS; n >= 2; --n)
+        if (StreamSmem::of<T, ACC>(L, n).total <= 227 * 1024) return n;
+    return 0;
 }
+// Threads of its blocks: a pass of kSB / kTPR rows where that covers a block's
+// rows, else twice as many.
+int stream_threads(const DevLevel &L) { return L.max_b <= kSB / kTPR ? kSB : kSBWide; }
 // Shared memory of the generic interior kernels (the whole interior vector of
 // the largest substructure); a level beyond one block's shared memory has no
 // kernel to run on and is refused.
@@ -1421,9 +1450,9 @@ template <class ACC> size_t generic_smem(const DevLevel &L) {
 }
 template <class T, class ACC> void pre_t(const DevLevel &L, const double *r, const int *skip,
                                          cudaStream_t s) {
-    if (stream_fits<T, ACC>(L)) {
-        launch_k(false, k_dir_s<T, ACC, false>, L.nsub, kSB, StreamSmem::of<T, ACC>(L).total, s, L, r,
-                 (double *)nullptr, skip);
+    if (const int ring = stream_ring<T, ACC>(L)) {
+        launch_k(false, k_dir_s<T, ACC, false>, L.nsub, stream_threads(L), StreamSmem::of<T, ACC>(L, ring).total, s, L,
+                 r, (double *)nullptr, skip, ring);
         return;
     }
     launch_k(false, k_pre<T, ACC>, L.nsub, kGT, generic_smem<ACC>(L), s, L, r, skip);
@@ -1440,8 +1469,9 @@ void neumann_t(const DevLevel &L, const double *r, const int *skip, bool pdl, cu
 }
 template <class T, class ACC> void post_t(const DevLevel &L, const double *r, double *z,
                                           const int *skip, cudaStream_t s) {
-    if (stream_fits<T, ACC>(L)) {
-        launch_k(false, k_dir_s<T, ACC, true>, L.nsub, kSB, StreamSmem::of<T, ACC>(L).total, s, L, r, z, skip);
+    if (const int ring = stream_ring<T, ACC>(L)) {
+        launch_k(false, k_dir_s<T, ACC, true>, L.nsub, stream_threads(L), StreamSmem::of<T, ACC>(L, ring).total, s, L, r,
+                 z, skip, ring);
         return;
     }
     launch_k(false, k_post<T, ACC>, L.nsub, kGT, generic_smem<ACC>(L), s, L, r, z, skip);
@@ -1669,9 +1699,11 @@ void apply_level_average(const DevLevel &L, int prec, const int *skip, cudaStrea
         return;
     }
     const size_t smn = sizeof(double) * (size_t)(L.max_nc > 0 ? L.max_nc : 1);
-    if (prec == BDDC_PREC_FP64) launch_k(false, k_average<double, double>, L.nsub, 128, smn, s, L, skip);
-    else if (prec == BDDC_PREC_FP32) launch_k(false, k_average<float, float>, L.nsub, 128, smn, s, L, skip);
-    else launch_k(false, k_average<__nv_bfloat16, float>, L.nsub, 128, smn, s, L, skip);
+    const int rows = (L.max_nG + kARows - 1) / kARows;
+    const dim3 grid((unsigned)L.nsub, (unsigned)(rows > 0 ? rows : 1));
+    if (prec == BDDC_PREC_FP64) launch_grid(false, k_average<double, double>, grid, kARows, smn, s, L, skip);
+    else if (prec == BDDC_PREC_FP32) launch_grid(false, k_average<float, float>, grid, kARows, smn, s, L, skip);
+    else launch_grid(false, k_average<__nv_bfloat16, float>, grid, kARows, smn, s, L, skip);
 }
 
 void apply_level_pre(const DevLevel &L, int prec, const double *r, const int *skip, cudaStream_t s,
