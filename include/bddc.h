@@ -183,8 +183,8 @@ typedef struct {
     int32_t tuned_route[3];
     /* the launch shape of the single right-hand-side product with the dense
      * top-level inverse, timed on that inverse at setup (0: 4 warps per row,
-     * 2 rows per block; 1: 8 and 1; 2: 2 and 4; 3: 4 and 4); -1 without a
-     * dense inverse */
+     * 2 rows per block; 1: 8 and 1; 2: 2 and 4; 3: four rows per warp,
+     * four warps sharing their columns); -1 without a dense inverse */
     int32_t tuned_symv;
 } bddc_info;
 

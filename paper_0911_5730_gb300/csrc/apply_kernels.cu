@@ -534,13 +534,16 @@ constexpr int kUI = 8, kUG = 4, kUC = 8, kUO = 4;   // record entries per lane, 
 __host__ __device__ constexpr int ui_of(int cls) { return cls == 0 ? 2 : kUI; }
 __host__ __device__ constexpr int ug_of(int cls) { return cls == 0 ? 1 : (cls == 1 ? 2 : kUG); }
 __host__ __device__ constexpr int uc_of(int cls) { return cls == 0 ? 4 : kUC; }
-__host__ __device__ constexpr int uo_of(int cls) { return cls == 2 ? kUO : 1; }
+__host__ __device__ constexpr int uo_of(int cls) { return cls >= 2 ? kUO : 1; }
+// Class 3: records of any size, read where they are used in rounds of 32 kUB
+// entries (the interiors of 16 x 16 elasticity substructures hold 450 DOFs).
+constexpr int kUB = 8;
 inline int dir_class(const DevLevel &L) {
-    for (int c = 0; c < 2; ++c)
+    for (int c = 0; c < 3; ++c)
         if (L.max_m * L.max_b <= 32 * ui_of(c) && L.max_nG <= 32 * ug_of(c) && L.max_coo <= 32 * uc_of(c) &&
             L.max_own <= 32 * uo_of(c))
             return c;
-    return 2;
+    return 3;
 }
 constexpr int kChunks = 4;                          // bulk copies per factor
 // Where a wave of substructures does not fit the SMs with whole factors (FP64
@@ -549,6 +552,7 @@ constexpr int kChunks = 4;                          // bulk copies per factor
 // instead (block j in slot j mod kDWRing, refilled once used; the backward
 // sweep starts from the blocks left in the ring).
 constexpr int kDWRing = 6;
+constexpr int kDWRingL = 4;   // class 3 (large interiors in FP32 / BF16)
 
 template <class T, class ACC, int BP, int RING> struct DirSlice {
     // every warp's slice starts 16-byte aligned: bulk-copy destinations and
@@ -630,17 +634,18 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     const int *gO = reinterpret_cast<const int *>(rec + lay.ow);
     int ii[UI], ig[UG], pr[UC], owp[UO], owd[UO];
     ACC cv[UC];
+    constexpr bool REG = CLS < 3;         // the record in registers
 #pragma unroll
-    for (int u = 0; u < UI; ++u) { const int i = u * 32 + lane; ii[u] = i < nI ? gI[i] : -1; }
+    for (int u = 0; u < UI && REG; ++u) { const int i = u * 32 + lane; ii[u] = i < nI ? gI[i] : -1; }
 #pragma unroll
-    for (int u = 0; u < UG; ++u) { const int q = u * 32 + lane; ig[u] = q < nG ? gGi[q] : -1; }
+    for (int u = 0; u < UG && REG; ++u) { const int q = u * 32 + lane; ig[u] = q < nG ? gGi[q] : -1; }
 #pragma unroll
-    for (int u = 0; u < UC; ++u) {
+    for (int u = 0; u < UC && REG; ++u) {
         const int k = u * 32 + lane;
         pr[u] = k < ncoo ? gP[k] : -1;
         cv[u] = k < ncoo ? (ACC)(gC[k]) : (ACC)0;
     }
-    if (POST) {
+    if (POST && REG) {
 #pragma unroll
         for (int u = 0; u < UO; ++u) {
             const int k = u * 32 + lane;
@@ -658,33 +663,73 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
     }
     // right-hand side (and u_B on Gamma for the post-correction)
     double rv[UI];
+    if constexpr (REG) {
 #pragma unroll
-    for (int u = 0; u < UI; ++u) rv[u] = ii[u] >= 0 ? r[ii[u]] : 0.0;
+        for (int u = 0; u < UI; ++u) rv[u] = ii[u] >= 0 ? r[ii[u]] : 0.0;
 #pragma unroll
-    for (int u = 0; u < UI; ++u) {
-        const int i = u * 32 + lane;
-        if (i < m * BP) x[i] = (ACC)(rv[u]);
-    }
-    if (POST) {
-        double uv[UG];
+        for (int u = 0; u < UI; ++u) {
+            const int i = u * 32 + lane;
+            if (i < m * BP) x[i] = (ACC)(rv[u]);
+        }
+        if (POST) {
+            double uv[UG];
 #pragma unroll
-        for (int u = 0; u < UG; ++u) uv[u] = ig[u] >= 0 ? L.uB[ig[u]] : 0.0;
+            for (int u = 0; u < UG; ++u) uv[u] = ig[u] >= 0 ? L.uB[ig[u]] : 0.0;
 #pragma unroll
-        for (int u = 0; u < UG; ++u) if (ig[u] >= 0) vG[u * 32 + lane] = (ACC)(uv[u]);
-        __syncwarp();
+            for (int u = 0; u < UG; ++u) if (ig[u] >= 0) vG[u * 32 + lane] = (ACC)(uv[u]);
+            __syncwarp();
 #pragma unroll
-        for (int u = 0; u < UC; ++u)
-            if (pr[u] >= 0) atomicAdd(&x[pr[u] & 0xffff], -cv[u] * vG[pr[u] >> 16]);
-    } else {
+            for (int u = 0; u < UC; ++u)
+                if (pr[u] >= 0) atomicAdd(&x[pr[u] & 0xffff], -cv[u] * vG[pr[u] >> 16]);
+        } else {
 #pragma unroll
-        for (int u = 0; u < UG; ++u) {
-            if (ig[u] >= 0) {
-                vG[u * 32 + lane] = 0;
-                L.uB[ig[u]] = 0.0;   // consumed by the previous post-correction
+            for (int u = 0; u < UG; ++u) {
+                if (ig[u] >= 0) {
+                    vG[u * 32 + lane] = 0;
+                    L.uB[ig[u]] = 0.0;   // consumed by the previous post-correction
+                }
             }
         }
+        __syncwarp();
+    } else {
+        for (int i0 = lane; i0 < m * BP; i0 += 32 * kUB) {
+            double v[kUB];
+#pragma unroll
+            for (int u = 0; u < kUB; ++u) v[u] = i0 + 32 * u < nI ? r[gI[i0 + 32 * u]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < kUB; ++u)
+                if (i0 + 32 * u < m * BP) x[i0 + 32 * u] = (ACC)v[u];
+        }
+        for (int q0 = lane; q0 < nG; q0 += 32 * kUB) {
+            double v[kUB];
+#pragma unroll
+            for (int u = 0; u < kUB; ++u) {
+                const int q = q0 + 32 * u;
+                v[u] = POST && q < nG ? L.uB[gGi[q]] : 0.0;
+                if (!POST && q < nG) L.uB[gGi[q]] = 0.0;   // consumed by the previous post-correction
+            }
+#pragma unroll
+            for (int u = 0; u < kUB; ++u)
+                if (q0 + 32 * u < nG) vG[q0 + 32 * u] = (ACC)v[u];
+        }
+        if (POST) {
+            __syncwarp();
+            for (int k0 = lane; k0 < ncoo; k0 += 32 * kUB) {
+                int e[kUB];
+                double c[kUB];
+#pragma unroll
+                for (int u = 0; u < kUB; ++u) {
+                    const int k = k0 + 32 * u;
+                    e[u] = k < ncoo ? gP[k] : -1;
+                    c[u] = k < ncoo ? gC[k] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < kUB; ++u)
+                    if (e[u] >= 0) atomicAdd(&x[e[u] & 0xffff], -(ACC)c[u] * vG[e[u] >> 16]);
+            }
+        }
+        __syncwarp();
     }
-    __syncwarp();
     const int rr = lane / LPR, h = lane % LPR;
     int cw = 0;   // next chunk to wait for
     bool ok = true;
@@ -761,6 +806,56 @@ __global__ void k_dir_w(DevLevel L, const double *r, double *z, const int *skip,
         if (RING && j + 1 < m && j + 1 - RING >= 0) refill((j + 1) % (RING ? RING : 1), j + 1 - RING);
     }
     __syncwarp();
+    if constexpr (!REG) {
+        if (!POST) {
+            for (int k0 = lane; k0 < ncoo; k0 += 32 * kUB) {
+                int e[kUB];
+                double c[kUB];
+#pragma unroll
+                for (int u = 0; u < kUB; ++u) {
+                    const int k = k0 + 32 * u;
+                    e[u] = k < ncoo ? gP[k] : -1;
+                    c[u] = k < ncoo ? gC[k] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < kUB; ++u)
+                    if (e[u] >= 0) atomicAdd(&vG[e[u] >> 16], (ACC)c[u] * x[e[u] & 0xffff]);
+            }
+            __syncwarp();
+            for (int q = lane; q < nG; q += 32) {
+                const ACC v = vG[q];
+                if (v != (ACC)0) atomicAdd(&L.rB[gGi[q]], -(double)v);
+            }
+        } else {
+            double acc = 0.0;
+            for (int i0 = lane; i0 < nI; i0 += 32 * kUB) {
+                int id[kUB];
+                double rn[kUB];
+#pragma unroll
+                for (int u = 0; u < kUB; ++u) id[u] = i0 + 32 * u < nI ? gI[i0 + 32 * u] : -1;
+#pragma unroll
+                for (int u = 0; u < kUB; ++u) rn[u] = rz.sc && id[u] >= 0 ? r[id[u]] : 0.0;
+#pragma unroll
+                for (int u = 0; u < kUB; ++u)
+                    if (id[u] >= 0) {
+                        const double zv = (double)x[i0 + 32 * u];
+                        z[id[u]] = zv;
+                        acc = fma(rn[u], zv, acc);
+                    }
+            }
+            for (int k = lane; k < nown; k += 32) {
+                const double zv = (double)vG[gO[2 * k]];
+                z[gO[2 * k + 1]] = zv;
+                if (rz.sc) acc = fma(r[gO[2 * k + 1]], zv, acc);
+            }
+            if (rz.sc) {
+                const int w0 = (int)(blockIdx.x * (blockDim.x >> 5));
+                const int nw = min((int)(blockDim.x >> 5), L.nsub - w0);
+                block_rz(acc, rz, smem_w, slice, nw, warp, lane);
+            }
+        }
+        return;
+    }
     if (!POST) {
 #pragma unroll
         for (int u = 0; u < UC; ++u)
@@ -1040,6 +1135,77 @@ k_dense_symv(int n, int ld, const double *A, const double *x, double *y, const i
             for (int k = 0; k < WR; ++k) t += part[threadIdx.x][k];
             y[rr] = t;
         }
+    }
+}
+
+// The same product with four rows to a warp: a vector load of x serves four
+// rows, and the four sums of a warp are reduced together (the first two
+// exchanges leave a quarter of the lanes with each row), six FP64 adds instead
+// of five per row.  One row per warp spends up to 40 adds on the 70
+// multiply-adds of a row of 2253 entries, and every one of them takes the FP64
+// pipe as long.  Four warps share the columns of a group of rows, two groups to
+// a block.  2253 rows: 10.7 -> 9.8 us; 1500 rows: 5.1 and 5.3, the setup's
+// timing picks.
+constexpr int kSvW = 4, kSvG = 2;
+__global__ void __launch_bounds__(32 * kSvW * kSvG)
+k_dense_symv4(int n, int ld, const double *A, const double *x, double *y, const int *skip) {
+    __shared__ double part[kSvG][kSvW][4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gr = warp / kSvW, ws = warp % kSvW;
+    const int row0 = (blockIdx.x * kSvG + gr) * 4;
+    constexpr int step = 64 * kSvW, PRE = 2;
+    const int c0 = 64 * ws + 2 * lane;
+    const double *a[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = A + (int64_t)(row0 + i < n ? row0 + i : n - 1) * ld;
+    double2 pre[PRE][4];                    // setup data: before the previous kernel's end
+#pragma unroll
+    for (int u = 0; u < PRE; ++u)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int c = c0 + u * step;
+            pre[u][i] = c < ld ? *reinterpret_cast<const double2 *>(a[i] + c) : make_double2(0.0, 0.0);
+        }
+    pdl_wait();
+    pdl_trigger();
+    if (skip && *skip) return;
+    double s[4] = {0.0, 0.0, 0.0, 0.0}, t[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) {
+        const int c = c0 + u * step;
+        if (c < ld) {
+            const double2 xv = *reinterpret_cast<const double2 *>(x + c);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                s[i] = fma(pre[u][i].x, xv.x, s[i]);
+                t[i] = fma(pre[u][i].y, xv.y, t[i]);
+            }
+        }
+    }
+#pragma unroll 2
+    for (int c = c0 + PRE * step; c < ld; c += step) {
+        const double2 xv = *reinterpret_cast<const double2 *>(x + c);
+        double2 av[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const double2 *>(a[i] + c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            s[i] = fma(av[i].x, xv.x, s[i]);
+            t[i] = fma(av[i].y, xv.y, t[i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] += t[i];
+    const bool h = lane & 16, q = lane & 8;
+    double b0 = (h ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, h ? s[0] : s[2], 16);
+    double b1 = (h ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, h ? s[1] : s[3], 16);
+    double v = (q ? b1 : b0) + __shfl_xor_sync(0xffffffffu, q ? b0 : b1, 8);
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 7) == 0) part[gr][ws][(h ? 2 : 0) + (q ? 1 : 0)] = v;
+    __syncthreads();
+    if (threadIdx.x < 4 * kSvG) {
+        const int g = threadIdx.x >> 2, i = threadIdx.x & 3, row = (blockIdx.x * kSvG + g) * 4 + i;
+        if (row < n) y[row] = (part[g][0][i] + part[g][1][i]) + (part[g][2][i] + part[g][3][i]);
     }
 }
 
@@ -1530,10 +1696,14 @@ void dir_launch_c(const DevLevel &L, bool post, const double *r, double *z, cons
 template <class T, class ACC, int BP, int RING>
 void dir_launch_r(const DevLevel &L, bool post, const double *r, double *z, const int *skip,
                   cudaStream_t s, const RzArgs *rz) {
-    const int cls = dir_class(L);
-    if (cls == 0) dir_launch_c<T, ACC, BP, RING, 0>(L, post, r, z, skip, s, rz);
-    else if (cls == 1) dir_launch_c<T, ACC, BP, RING, 1>(L, post, r, z, skip, s, rz);
-    else dir_launch_c<T, ACC, BP, RING, 2>(L, post, r, z, skip, s, rz);
+    if constexpr (RING == kDWRingL) {
+        dir_launch_c<T, ACC, BP, RING, 3>(L, post, r, z, skip, s, rz);
+    } else {
+        const int cls = dir_class(L);
+        if (cls == 0) dir_launch_c<T, ACC, BP, RING, 0>(L, post, r, z, skip, s, rz);
+        else if (cls == 1) dir_launch_c<T, ACC, BP, RING, 1>(L, post, r, z, skip, s, rz);
+        else dir_launch_c<T, ACC, BP, RING, 2>(L, post, r, z, skip, s, rz);
+    }
 }
 // The ring where whole factors would take more waves than it does: with one
 // wave either way, the whole factor saves the second read of its blocks.
@@ -1549,6 +1719,12 @@ void dir_launch(const DevLevel &L, bool post, const double *r, double *z, const 
     if constexpr (sizeof(T) == 8) {
         if (waves(DirSlice<T, ACC, BP, kDWRing>::bytes(L)) < waves(DirSlice<T, ACC, BP, 0>::bytes(L))) {
             dir_launch_r<T, ACC, BP, kDWRing>(L, post, r, z, skip, s, rz);
+            return;
+        }
+    }
+    if constexpr (sizeof(T) < 8) {
+        if (dir_class(L) == 3) {
+            dir_launch_r<T, ACC, BP, kDWRingL>(L, post, r, z, skip, s, rz);
             return;
         }
     }
@@ -1584,6 +1760,21 @@ void avg_launch(const DevLevel &L, int prec, const int *skip, cudaStream_t s) {
                (unsigned)slice);
 }
 
+// Interiors beyond the records of warp_path in FP32 / BF16 with a power-of-two
+// block size: the warp Dirichlet kernel in class 3 where there are warps for
+// every SM and a wave of them fits; the block-per-substructure kernels
+// (k_dir_s) otherwise.  576 elasticity substructures of 450 interior
+// DOFs: 28 + 24 us, where k_dir_s took 40 + 35; a handful of substructures runs
+// faster with a block each.
+bool warp_dir_large(const DevLevel &L, int prec) {
+    if (prec == BDDC_PREC_FP64 || force_generic_dir()) return false;
+    if (!(L.bp == 8 || L.bp == 16 || L.bp == 32) || !L.irec || dir_class(L) != 3 || L.max_m * L.bp > 65535) return false;
+    const size_t e = prec == BDDC_PREC_FP32 ? 4 : 2;
+    const size_t slice = al16(al16(e * kDWRingL * 2 * L.bp * L.bp) + al16(4 * (size_t)L.max_m * L.bp) +
+                              al16(4 * (size_t)L.max_nG) + 8 * kDWRingL + 16);
+    return L.nsub >= num_sms() && (int64_t)num_sms() * (int64_t)(kSmemMax / slice) >= L.nsub;
+}
+
 // The warp kernels need a power-of-two block size, the records and their
 // shared slices within one block.
 bool warp_path(const DevLevel &L, int prec) {
@@ -1613,6 +1804,10 @@ void prepare_apply_kernels() {
     BDDC_DIR_W(double, double, 8, kDWRing) BDDC_DIR_W(double, double, 16, kDWRing) BDDC_DIR_W(double, double, 32, kDWRing)
     BDDC_DIR_W(float, float, 8, 0) BDDC_DIR_W(float, float, 16, 0) BDDC_DIR_W(float, float, 32, 0)
     BDDC_DIR_W(__nv_bfloat16, float, 8, 0) BDDC_DIR_W(__nv_bfloat16, float, 16, 0) BDDC_DIR_W(__nv_bfloat16, float, 32, 0)
+    BDDC_DIR_WC(float, float, 8, kDWRingL, 3) BDDC_DIR_WC(float, float, 16, kDWRingL, 3)
+    BDDC_DIR_WC(float, float, 32, kDWRingL, 3)
+    BDDC_DIR_WC(__nv_bfloat16, float, 8, kDWRingL, 3) BDDC_DIR_WC(__nv_bfloat16, float, 16, kDWRingL, 3)
+    BDDC_DIR_WC(__nv_bfloat16, float, 32, kDWRingL, 3)
 #undef BDDC_DIR_W
 #undef BDDC_DIR_WC
     BDDC_SMEM_ATTR((k_dir_s<double, double, false>));
@@ -1644,11 +1839,11 @@ void build_records(DevLevel &D, const int *ownPos, const int *ownDof, cudaStream
     k_build_nrec<__nv_bfloat16><<<D.nsub, 128, 0, s>>>(D, D.b16, D.nrec[2], D.nrecOff[2]);
 }
 
-bool apply_fuses_rz(const DevLevel &L, int prec) { return warp_path(L, prec); }
+bool apply_fuses_rz(const DevLevel &L, int prec) { return warp_path(L, prec) || warp_dir_large(L, prec); }
 
 void apply_level_dir(const DevLevel &L, int prec, bool post, const double *r, double *z, const int *skip,
                      cudaStream_t s, const RzArgs *rz) {
-    if (warp_path(L, prec)) {
+    if (warp_path(L, prec) || warp_dir_large(L, prec)) {
         if (prec == BDDC_PREC_FP64) dir_dispatch<double, double>(L, post, r, z, skip, s, rz);
         else if (prec == BDDC_PREC_FP32) dir_dispatch<float, float>(L, post, r, z, skip, s, rz);
         else dir_dispatch<__nv_bfloat16, float>(L, post, r, z, skip, s, rz);
@@ -1730,7 +1925,9 @@ void launch_dense_symv(int n, int ld, const double *A, const double *x, double *
     switch (variant) {   // (warps per row, rows per block)
         case 1: launch_pdl(k_dense_symv<8, 1>, n, 256, 0, s, n, ld, A, x, y, skip); break;
         case 2: launch_pdl(k_dense_symv<2, 4>, (n + 3) / 4, 256, 0, s, n, ld, A, x, y, skip); break;
-        case 3: launch_pdl(k_dense_symv<4, 4>, (n + 3) / 4, 512, 0, s, n, ld, A, x, y, skip); break;
+        case 3:
+            launch_pdl(k_dense_symv4, (n + 4 * kSvG - 1) / (4 * kSvG), 32 * kSvW * kSvG, 0, s, n, ld, A, x, y, skip);
+            break;
         default: launch_pdl(k_dense_symv<4, 2>, (n + 1) / 2, 256, 0, s, n, ld, A, x, y, skip); break;
     }
 }
