@@ -821,35 +821,42 @@ __global__ void __launch_bounds__(32 * kLSW) k_dir_ls(DevLevel L, BatchLevel B, 
 // shared memory (large or irregular cells).  Persistent blocks, one launch
 // per size bucket (the substructures whose blocks take the same number of
 // warps), each block taking the bucket's substructures largest first; per
-// substructure all 32 right-hand-side columns go in one pass, so the factor
-// is streamed once, block by block, through a ring of SBN stages as in the
-// single right-hand-side streaming kernel (block i in stage i % SBN; the
-// backward sweep starts from the blocks left in the ring and refills the
-// stage of block j+1 after step j).  Thread t of a substructure with block
-// size b owns column group g = t / h (columns 4g..4g+3) and rows k and k + h
-// (k = t mod h, h = ceil(b/2)) of every block: a 2-row x 4-column register
-// tile, so a factor entry read from shared memory feeds four FMAs and a
-// broadcast 4-column vector eight, with four factor columns in flight.  Rows
-// of a block are ld apart (odd unless swizzled), so the transposed walks of
-// the backward sweep are free of bank conflicts too.  The block results of
-// the forward sweep (y_j) and of the backward sweep (x_j) go to a global
-// scratch [8][rows][4] per substructure, which stays in L2; each thread
-// reads back only what it wrote, one step ahead.
-constexpr int SBN = 3, kSBMaxT = 32 * kMaxBuckets;   // ring stages, largest block
-
-// doubles of the reduction area: four per thread, and the 8 x 32 of the
-// final r.z sum
-__host__ __device__ inline size_t red_doubles(int nt) { return 4 * (size_t)nt > 256 ? 4 * (size_t)nt : 256; }
+// substructure all 32 right-hand-side columns go in one pass, so each sweep
+// streams the factor once.  The unit of the stream is half a block: the
+// forward sweep uses Linv_0, Lsub_1, Linv_1, Lsub_2, ... and the backward
+// sweep the same sequence in reverse, so a ring of SBN halves (half s in slot
+// s mod SBN, refilled SBN halves ahead as soon as it is used) needs no more
+// than what is in use and in flight, and turns round on the halves left in
+// it.  Thread t of a substructure with block size b owns column group
+// g = t / h (columns 4g..4g+3) and rows k and k + h (k = t mod h,
+// h = ceil(b/2)) of every block: a 2-row x 4-column register tile, so a
+// factor entry read from shared memory feeds four FMAs and a broadcast
+// 4-column vector eight, with four factor columns in flight.  Rows of a block
+// are ld apart (odd unless swizzled), so the transposed walks of the backward
+// sweep are free of bank conflicts too.  The sweeps touch global memory only
+// through the factor's copies and a scratch [8][rows][4] per substructure in
+// L2 (each thread its own entries, one step ahead): a first pass of the block,
+// a lane per column, gathers the right-hand side (with the post-correction's
+// A_IG u_B terms) into it, and a last one writes z and sums r.z.  With those
+// gathers inside the sweeps a warp waited on chains of dependent loads at
+// every step (ncu: long scoreboard 2.4 of 5.6 cycles per instruction).
+// 1024 Voronoi cells of 1000 DOFs, 21
+// right-hand sides: solve 145.8 -> 133.3 ms; 1024 cells of 225 DOFs in FP64, 32
+// right-hand sides: 600 and 667 us before, 617 and 684 with whole products, 535
+// and 594 with the zeros of Lsub left out (which took the Voronoi solve from 130
+// to 124 ms).
+constexpr int SBN = 4, kSBMaxT = 32 * kMaxBuckets;   // ring slots, largest block
+constexpr int kSBSmallT = 192;                       // the common block sizes: more blocks per SM
 
 struct StreamSmemB {
     size_t stage, ring, vec, red, total;
-    template <class T, class ACC> __host__ __device__ static StreamSmemB of(const DevLevel &L, int nt) {
+    template <class T, class ACC> __host__ __device__ static StreamSmemB of(const DevLevel &L) {
         StreamSmemB m;
         const size_t mb = L.max_b > 0 ? L.max_b : 1, mld = L.max_ld > 0 ? L.max_ld : 1;
-        m.stage = al16(2 * mb * mld * sizeof(T) + 32);
+        m.stage = al16(mb * mld * sizeof(T) + 32);
         m.ring = SBN * m.stage;
         m.vec = al16(sizeof(ACC) * mb * kMaxBatch);   // [8][b][4]
-        m.red = al16(8 * red_doubles(nt) + 16);       // four doubles per thread (at least 256), a flag
+        m.red = al16(8 * 32 * kMaxBuckets + 16);      // r.z partials per warp and column, a flag
         m.total = m.ring + 2 * m.vec + m.red + 8 * SBN + 16;
         return m;
     }
@@ -913,106 +920,136 @@ __device__ __forceinline__ void prod2(ACC (&a0)[4], ACC (&a1)[4], const T *M, in
     }
 }
 
-template <class T, class ACC, bool SWZ, bool POST>
-__global__ void __launch_bounds__(kSBMaxT, 1) k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z,
-                                                    const int *skip, RzBatch rz, const int *perm, int count) {
+template <class T, class ACC, bool SWZ, bool POST, int NT>
+__global__ void __launch_bounds__(NT, NT == kSBSmallT ? 4 : 1)
+k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, RzBatch rz, const int *perm,
+         int count) {
     extern __shared__ __align__(16) unsigned char smem_bs[];
     if (skip && *skip) return;
     const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = nt >> 5;
-    const StreamSmemB ly = StreamSmemB::of<T, ACC>(L, nt);
+    const StreamSmemB ly = StreamSmemB::of<T, ACC>(L);
     unsigned char *ring = smem_bs;
     ACC *ybuf = reinterpret_cast<ACC *>(smem_bs + ly.ring);
     ACC *tbuf = reinterpret_cast<ACC *>(smem_bs + ly.ring + ly.vec);
     double *red = reinterpret_cast<double *>(smem_bs + ly.ring + 2 * ly.vec);
-    int *flag = reinterpret_cast<int *>(red + red_doubles(nt));
+    int *flag = reinterpret_cast<int *>(red + 32 * kMaxBuckets);
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem_bs + ly.ring + 2 * ly.vec + ly.red);
     const int K = B.K;
+    const bool lact = lane < K;
     const OpSet<T> &O = Ops<T>::get(L);
     if (tid == 0)
         for (int s2 = 0; s2 < SBN; ++s2) mbar_init(&bars[s2]);
     __syncthreads();
-    unsigned par = 0;                     // bit s: parity of the next phase of stage s
-    bool ok = true;
-    auto wait_block = [&](int i) {
-        const int s2 = i % SBN;
-        const bool got = mbar_wait(&bars[s2], (par >> s2) & 1u);
-        par ^= 1u << s2;
-        return __syncthreads_and(got) != 0;
-    };
-    for (int ti = blockIdx.x; ti < count && ok; ti += gridDim.x) {
+    unsigned par = 0, pend = 0;           // bit s: parity of slot s's next phase; a copy in flight (thread 0)
+    bool ok = true;                       // false once a wait of this thread gave up: it waits no more
+    for (int ti = blockIdx.x; ti < count; ti += gridDim.x) {
         const int sub = perm[ti];
         const int nI = L.nI[sub], nG = L.nG[sub], b = L.bsz[sub], m = nI > 0 ? L.nblk[sub] : 0;
         const int mb = m * b, ldb = fld(b, SWZ), h = (b + 1) >> 1;
         const T *F = O.dir + L.offF[sub];
-        const size_t bsq = (size_t)b * ldb, bb2 = 2 * bsq;
+        const size_t bsq = (size_t)b * ldb;
         const int *iI = L.idxI + L.offI[sub];
         const int *iG = L.idxG + L.offG[sub];
         ACC *Ysub = reinterpret_cast<ACC *>(B.ys) + L.offY[sub] * kMaxBatch;   // [8][mb][4]
+        ACC *Yl = Ysub + (size_t)(lane >> 2) * mb * 4 + (lane & 3);            // this lane's column: row i at 4 i
         const bool act = tid < 8 * h;
         const int cg = act ? tid / h : 0, k = act ? tid - cg * h : 0;
         const int r0 = k, r1 = k + h, r1c = r1 < b ? r1 : b - 1;   // r1 == b for odd b: computed, not kept
         const bool colact = act && 4 * cg < K;
         ACC *Yg = Ysub + (size_t)cg * mb * 4;
         ACC *yb = ybuf + (size_t)cg * b * 4, *tb = tbuf + (size_t)cg * b * 4;
-        auto issue = [&](int i) {
-            const uintptr_t a = reinterpret_cast<uintptr_t>(F + (size_t)i * bb2);
+        // half s of the sequence Linv_0, Lsub_1, Linv_1, ...: s = 2 j: Linv_j, s = 2 j - 1: Lsub_j
+        const int ns = 2 * m - 1;
+        auto half_of = [&](int s) { return F + ((size_t)(s + 1) / 2 * 2 + (s & 1)) * bsq; };
+        auto issue = [&](int s) {         // thread 0: half s, its bytes rounded out to 16-byte boundaries
+            const uintptr_t a = reinterpret_cast<uintptr_t>(half_of(s));
             const uintptr_t al = a & ~uintptr_t(15);
-            const uintptr_t ae = (a + bb2 * sizeof(T) + 15) & ~uintptr_t(15);
-            mbar_expect(&bars[i % SBN], (unsigned)(ae - al));
-            bulk_copy(ring + (size_t)(i % SBN) * ly.stage, reinterpret_cast<const void *>(al),
-                      (unsigned)(ae - al), &bars[i % SBN]);
+            const uintptr_t ae = (a + bsq * sizeof(T) + 15) & ~uintptr_t(15);
+            mbar_expect(&bars[s % SBN], (unsigned)(ae - al));
+            bulk_copy(ring + (size_t)(s % SBN) * ly.stage, reinterpret_cast<const void *>(al),
+                      (unsigned)(ae - al), &bars[s % SBN]);
+            pend |= 1u << (s % SBN);
         };
-        auto blk = [&](int i) {
-            const uintptr_t a = reinterpret_cast<uintptr_t>(F + (size_t)i * bb2);
-            return reinterpret_cast<const T *>(ring + (size_t)(i % SBN) * ly.stage + (a & 15));
+        auto slot = [&](int s) {
+            const uintptr_t a = reinterpret_cast<uintptr_t>(half_of(s));
+            return reinterpret_cast<const T *>(ring + (size_t)(s % SBN) * ly.stage + (a & 15));
         };
-        if (tid == 0)
-            for (int i = 0; i < SBN && i < m; ++i) issue(i);
-        // interior row i of the right-hand side in this thread's four columns,
-        // minus its A_{I Gamma} u_B terms in the post-correction (the row's
-        // coupling entries in increasing order); padding rows are zero
-        const int64_t i0 = L.offI[sub];
-        auto load_row = [&](int i, ACC (&v)[4]) {
+        auto wait_half = [&](int s) {     // every thread sees the copy's completion itself
+            const int q = s % SBN;
+            if (ok) {
+                ok = mbar_wait(&bars[q], (par >> q) & 1u);
+                if (ok) pend &= ~(1u << q);
+            }
+            par ^= 1u << q;
+        };
+        if (tid == 0 && ok)
+            for (int s = 0; s < SBN && s < ns; ++s) issue(s);
+        {
+            // the right-hand side into the scratch, a lane per column, four
+            // rows in flight: interior rows of r, minus their A_{I Gamma} u_B
+            // terms in the post-correction (the row's coupling entries in
+            // increasing order); padding rows and columns are zero
+            const int64_t i0 = L.offI[sub];
+            constexpr int PU = 4;
+            for (int q0 = w * PU; q0 < mb; q0 += nw * PU) {
+                double v[PU];
+                int e0[PU], e1[PU];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = 0;
-            if (i >= nI) return;
-            const double *ri = r + (int64_t)iI[i] * K;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (4 * cg + q < K) v[q] = from_f64<ACC>(ri[4 * cg + q]);
-            if (POST)
-                for (int64_t p = L.cooRptr[i0 + i]; p < L.cooRptr[i0 + i + 1]; ++p) {
-                    const ACC a = ld<T, ACC>(O.aig + L.cooRowE[p]);
-                    const double *u = B.uB + (int64_t)L.cooRowId[p] * K;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (4 * cg + q < K) v[q] -= a * from_f64<ACC>(u[4 * cg + q]);
+                for (int u = 0; u < PU; ++u) {
+                    const int i = q0 + u;
+                    v[u] = (i < nI && lact) ? r[(int64_t)iI[i] * K + lane] : 0.0;
+                    e0[u] = e1[u] = 0;
+                    if (POST && i < nI) {
+                        e0[u] = (int)L.cooRptr[i0 + i];
+                        e1[u] = (int)L.cooRptr[i0 + i + 1];
+                    }
                 }
-        };
-        double rzs[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+                for (int u = 0; u < PU; ++u) {
+                    if (q0 + u >= mb) break;
+                    ACC x = from_f64<ACC>(v[u]);
+                    if (POST && lact)
+                        for (int p = e0[u]; p < e1[u]; ++p)
+                            x -= ld<T, ACC>(O.aig + L.cooRowE[p]) *
+                                 from_f64<ACC>(B.uB[(int64_t)L.cooRowId[p] * K + lane]);
+                    Yl[(size_t)(q0 + u) * 4] = x;
+                }
+            }
+        }
+        __syncthreads();
         ACC n0[4], n1[4];                 // the next step's rows, loaded a step ahead
-        if (colact && m > 0) { load_row(r0, n0); load_row(r1c, n1); }
+        if (colact && m > 0) {
+            ld4(Yg + (size_t)r0 * 4, n0);
+            ld4(Yg + (size_t)r1c * 4, n1);
+        }
         // forward: y_j = Linv_j (rhs_j - Lsub_j y_{j-1})
         for (int j = 0; j < m; ++j) {
-            if (!wait_block(j)) { ok = false; break; }
-            const T *Li = blk(j), *Ls = Li + bsq;
+            ACC a0[4], a1[4];
             if (colact) {
-                ACC a0[4], a1[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) { a0[q] = n0[q]; a1[q] = n1[q]; }
                 if (j + 1 < m) {
-                    load_row((j + 1) * b + r0, n0);
-                    load_row((j + 1) * b + r1c, n1);
+                    ld4(Yg + ((size_t)(j + 1) * b + r0) * 4, n0);
+                    ld4(Yg + ((size_t)(j + 1) * b + r1c) * 4, n1);
                 }
-                if (j > 0) prod2<T, ACC, true, true, true, SWZ>(a0, a1, Ls, ldb, yb, 0, b, r0, r1c);
+            }
+            if (j > 0) {
+                wait_half(2 * j - 1);
+                if (colact) prod2<T, ACC, true, true, true, SWZ>(a0, a1, slot(2 * j - 1), ldb, yb, 0, b, r0, r1c);
+            }
+            if (colact) {
                 st4(tb + r0 * 4, a0);
                 if (r1 < b) st4(tb + r1 * 4, a1);
             }
+            wait_half(2 * j);
             __syncthreads();
+            if (tid == 0 && ok && j > 0 && 2 * j - 1 + SBN < ns) issue(2 * j - 1 + SBN);
             if (colact) {
                 // Linv_j lower triangular (zeros stored above): row k needs
                 // columns < h only, row k + h all of them
-                ACC a0[4] = {0, 0, 0, 0}, a1[4] = {0, 0, 0, 0};
+                const T *Li = slot(2 * j);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a0[q] = a1[q] = 0;
                 prod2<T, ACC, false, true, true, SWZ>(a0, a1, Li, ldb, tb, 0, h, r0, r1c);
                 prod2<T, ACC, false, false, true, SWZ>(a1, a1, Li, ldb, tb, h, b, r1c, r1c);
                 st4(yb + r0 * 4, a0);
@@ -1026,99 +1063,117 @@ __global__ void __launch_bounds__(kSBMaxT, 1) k_dir_bs(DevLevel L, BatchLevel B,
                     for (int q = 0; q < 4; ++q) { n0[q] = a0[q]; n1[q] = a1[q]; }   // y_{m-1}
             }
             __syncthreads();
-            if (tid == 0 && j + SBN < m) issue(j + SBN);
+            if (tid == 0 && ok && 2 * j + SBN < ns) issue(2 * j + SBN);
         }
-        // backward: x_j = Linv_j^T (y_j - Lsub_{j+1}^T x_{j+1})
-        for (int j = m - 1; j >= 0 && ok; --j) {
-            if (j < m - SBN && !wait_block(j)) { ok = false; break; }
-            const T *Li = blk(j);
+        // backward: x_j = Linv_j^T (y_j - Lsub_{j+1}^T x_{j+1}); halves ns-1 ..
+        // ns-SBN are still in the ring
+        for (int j = m - 1; j >= 0; --j) {
+            ACC a0[4], a1[4];
             if (colact) {
-                ACC a0[4], a1[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) { a0[q] = n0[q]; a1[q] = n1[q]; }
                 if (j > 0) {
                     ld4(Yg + ((size_t)(j - 1) * b + r0) * 4, n0);
                     ld4(Yg + ((size_t)(j - 1) * b + r1c) * 4, n1);
                 }
-                if (j < m - 1) prod2<T, ACC, true, true, false, SWZ>(a0, a1, blk(j + 1) + bsq, ldb, yb, 0, b, r0, r1c);
+            }
+            if (j < m - 1) {
+                const int s = 2 * j + 1;
+                if (s < ns - SBN) wait_half(s);
+                if (colact) prod2<T, ACC, true, true, false, SWZ>(a0, a1, slot(s), ldb, yb, 0, b, r0, r1c);
+            }
+            if (colact) {
                 st4(tb + r0 * 4, a0);
                 if (r1 < b) st4(tb + r1 * 4, a1);
             }
+            if (2 * j < ns - SBN) wait_half(2 * j);
             __syncthreads();
+            if (tid == 0 && ok && j < m - 1 && 2 * j + 1 - SBN >= 0) issue(2 * j + 1 - SBN);
             if (colact) {
                 // Linv_j^T upper triangular: row k needs all columns, row k + h
                 // columns >= h only
-                ACC a0[4] = {0, 0, 0, 0}, a1[4] = {0, 0, 0, 0};
+                const T *Li = slot(2 * j);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a0[q] = a1[q] = 0;
                 prod2<T, ACC, false, false, false, SWZ>(a0, a0, Li, ldb, tb, 0, h, r0, r0);
                 prod2<T, ACC, false, true, false, SWZ>(a0, a1, Li, ldb, tb, h, b, r0, r1c);
-#pragma unroll
-                for (int rw = 0; rw < 2; ++rw) {
-                    const int row = rw ? r1 : r0;
-                    if (row >= b) break;
-                    const ACC (&a)[4] = rw ? a1 : a0;
-                    st4(yb + row * 4, a);
-                    if (!POST) {
-                        st4(Yg + ((size_t)j * b + row) * 4, a);
-                    } else if (j * b + row < nI) {
-                        const int64_t o = (int64_t)iI[j * b + row] * K;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int kk = 4 * cg + q;
-                            if (kk >= K) break;
-                            const double zv = to_f64(a[q]);
-                            z[o + kk] = zv;
-                            if (rz.sc) rzs[q] = fma(r[o + kk], zv, rzs[q]);
-                        }
-                    }
+                st4(yb + r0 * 4, a0);
+                st4(Yg + ((size_t)j * b + r0) * 4, a0);
+                if (r1 < b) {
+                    st4(yb + r1 * 4, a1);
+                    st4(Yg + ((size_t)j * b + r1) * 4, a1);
                 }
             }
             __syncthreads();
-            if (tid == 0 && j + 1 < m && j + 1 - SBN >= 0) issue(j + 1 - SBN);
+            if (tid == 0 && ok && 2 * j - SBN >= 0) issue(2 * j - SBN);
         }
-        if (!ok) break;
-        // every issued block has been waited for: the ring is idle from here
+        if (!__syncthreads_and(ok)) break;
+        // every issued half has been waited for: the ring is idle from here
         if (!POST) {
             // r_B -= A_{Gamma I} x (Gamma entry q: warp q mod nw, lane: column;
             // the entry's couplings in order); u_B was consumed by the previous
             // post-correction
             const int64_t g0 = L.offG[sub];
-            if (lane < K)
+            if (lact)
                 for (int q = w; q < nG; q += nw) {
                     ACC acc = 0;
                     for (int64_t e = L.cooGptr[g0 + q]; e < L.cooGptr[g0 + q + 1]; ++e)
-                        acc += ld<T, ACC>(O.aig + e) *
-                               Ysub[((size_t)(lane >> 2) * mb + L.cooI[e]) * 4 + (lane & 3)];
+                        acc += ld<T, ACC>(O.aig + e) * Yl[(size_t)L.cooI[e] * 4];
                     const int64_t o = (int64_t)iG[q] * K + lane;
                     if (acc != (ACC)0) atomicAdd(&B.rB[o], -to_f64(acc));
                     B.uB[o] = 0.0;
                 }
+            __syncthreads();              // the scratch and the buffers are free for the next substructure
             continue;
         }
-        // interface entries of z (owned by this substructure): u_B
-        if (colact)
-            for (int64_t e = L.offOwn[sub] + k; e < L.offOwn[sub + 1]; e += h) {
-                const int id = L.own[e];
-                const int64_t o = (int64_t)L.ifaceDof[id] * K;
+        // z: the interior rows from the scratch and the owned interface
+        // entries (u_B), a lane per column; r.z over what is written
+        double rzs = 0.0;
+        constexpr int PU = 4;
+        for (int q0 = w * PU; q0 < nI; q0 += nw * PU) {
+            double zv[PU], rv[PU];
+            int o[PU];                    // DOF
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int kk = 4 * cg + q;
-                    if (kk >= K) break;
-                    const double zv = B.uB[(int64_t)id * K + kk];
-                    z[o + kk] = zv;
-                    if (rz.sc) rzs[q] = fma(r[o + kk], zv, rzs[q]);
-                }
+            for (int u = 0; u < PU; ++u) {
+                const int i = q0 + u;
+                const bool in = i < nI && lact;
+                o[u] = in ? iI[i] : 0;
+                zv[u] = in ? to_f64(Yl[(size_t)i * 4]) : 0.0;
+                rv[u] = in && rz.sc ? r[(int64_t)o[u] * K + lane] : 0.0;
             }
-        if (!rz.sc) continue;
-        // r.z per column: the h threads of its group in order, then the
-        // substructures by the block that finishes the last one, in order
 #pragma unroll
-        for (int q = 0; q < 4; ++q) red[tid * 4 + q] = rzs[q];
+            for (int u = 0; u < PU; ++u) {
+                if (q0 + u < nI && lact) z[(int64_t)o[u] * K + lane] = zv[u];
+                rzs = fma(rv[u], zv[u], rzs);
+            }
+        }
+        for (int64_t q0 = L.offOwn[sub] + w * PU; q0 < L.offOwn[sub + 1]; q0 += nw * PU) {
+            double zv[PU], rv[PU];
+            int o[PU];                    // DOF
+#pragma unroll
+            for (int u = 0; u < PU; ++u) {
+                const bool in = q0 + u < L.offOwn[sub + 1] && lact;
+                const int id = in ? L.own[q0 + u] : 0;
+                o[u] = in ? L.ifaceDof[id] : 0;
+                zv[u] = in ? B.uB[(int64_t)id * K + lane] : 0.0;
+                rv[u] = in && rz.sc ? r[(int64_t)o[u] * K + lane] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < PU; ++u) {
+                if (q0 + u < L.offOwn[sub + 1] && lact) z[(int64_t)o[u] * K + lane] = zv[u];
+                rzs = fma(rv[u], zv[u], rzs);
+            }
+        }
+        __syncthreads();                  // the scratch is free for the next substructure
+        if (!rz.sc) continue;
+        // r.z per column: the warps in order, then the substructures by the
+        // block that finishes the last one, in order
+        red[w * 32 + lane] = rzs;
         __syncthreads();
-        if (tid < K) {
-            const int g = tid >> 2, q = tid & 3;
+        if (w == 0 && lact) {
             double t = 0.0;
-            for (int u = g * h; u < g * h + h; ++u) t += red[u * 4 + q];
-            rz.part[(int64_t)sub * K + tid] = t;
+            for (int u = 0; u < nw; ++u) t += red[u * 32 + lane];
+            rz.part[(int64_t)sub * K + lane] = t;
         }
         __threadfence();
         __syncthreads();
@@ -1130,7 +1185,7 @@ __global__ void __launch_bounds__(kSBMaxT, 1) k_dir_bs(DevLevel L, BatchLevel B,
             // bucket of the finishing block: the same order in every run
             for (int g = w; g < 8; g += nw) {
                 double t = 0.0;
-                if (lane < K) {
+                if (lact) {
                     // sixteen loads in flight (one at a time, this tail took
                     // 25 us more at 1024 substructures)
                     for (int sb = g; sb < L.nsub; sb += 8 * 16) {
@@ -1145,7 +1200,7 @@ __global__ void __launch_bounds__(kSBMaxT, 1) k_dir_bs(DevLevel L, BatchLevel B,
                 red[g * 32 + lane] = t;
             }
             __syncthreads();
-            if (w == 0 && lane < K) {
+            if (w == 0 && lact) {
                 double tot = 0.0;
                 for (int v = 0; v < 8; ++v) tot += red[v * 32 + lane];
                 BatchScalars *sc = rz.sc;
@@ -1162,10 +1217,10 @@ __global__ void __launch_bounds__(kSBMaxT, 1) k_dir_bs(DevLevel L, BatchLevel B,
         }
         __syncthreads();                  // red is free for the next substructure
     }
-    if (!ok && tid == 0) {
-        atomicExch(L.err, 1);
-        for (int s2 = 0; s2 < SBN; ++s2) mbar_wait(&bars[s2], (par >> s2) & 1u);   // bounded
-    }
+    if (!ok) atomicExch(L.err, 1);
+    if (tid == 0)                         // bounded: copies in flight land before the block exits
+        for (int s2 = 0; s2 < SBN; ++s2)
+            if ((pend >> s2) & 1u) mbar_wait(&bars[s2], (par >> s2) & 1u);
 }
 
 // (6)-(9) for K right-hand sides, a block of up to kNBW warps per
@@ -2276,7 +2331,7 @@ template <class T, class ACC> BatchRoute route_t(const DevLevel &L, int prec) {
     // the largest bucket's layout bounds every bucket's
     const int nw_max = ((L.max_b + 1) / 2 + 3) / 4;
     const bool stream = L.bk.n > 0 && L.bperm && nw_max <= kMaxBuckets &&
-                        StreamSmemB::of<T, ACC>(L, 32 * nw_max).total <= kSmemMaxB;
+                        StreamSmemB::of<T, ACC>(L).total <= kSmemMaxB;
     const bool bg = neu_bg_smem<T, ACC>(L) <= kSmemMaxB && avg_bg_smem<T, ACC>(L) <= kSmemMaxB;
     R.dir_stream = !R.dir_staged && stream;
     R.stream_fits = stream;
@@ -2362,8 +2417,11 @@ void dir_bs_buckets(const DevLevel &L, const BatchLevel &B, const double *r, dou
         Lb.max_ld = L.bk.max_ld[i];
         Lb.max_nG = L.bk.max_nG[i];
         const int nt = 32 * L.bk.nw[i];
-        const size_t sm = StreamSmemB::of<T, ACC>(Lb, nt).total;
-        const int per = resident_blocks(reinterpret_cast<const void *>(k_dir_bs<T, ACC, SWZ, POST>), nt, sm, s);
+        const size_t sm = StreamSmemB::of<T, ACC>(Lb).total;
+        auto kern = k_dir_bs<T, ACC, SWZ, POST, kSBMaxT>;
+        if constexpr (sizeof(ACC) == 4)       // (FP64 wants the 128 registers)
+            if (nt <= kSBSmallT) kern = k_dir_bs<T, ACC, SWZ, POST, kSBSmallT>;
+        const int per = resident_blocks(reinterpret_cast<const void *>(kern), nt, sm, s);
         if (!launch) continue;
         const int grid = std::min(L.bk.count[i], per * num_sms_b());
         cudaStream_t si = s;
@@ -2371,7 +2429,7 @@ void dir_bs_buckets(const DevLevel &L, const BatchLevel &B, const double *r, dou
             si = F->st[i - 1];
             BDDC_CUDA_TRY(cudaStreamWaitEvent(si, F->fork, 0));
         }
-        launch_plain(k_dir_bs<T, ACC, SWZ, POST>, grid, nt, sm, si, Lb, B, r, z, skip, rz,
+        launch_plain(kern, grid, nt, sm, si, Lb, B, r, z, skip, rz,
                      (const int *)(L.bperm + L.bk.first[i]), L.bk.count[i]);
         if (F && i > 0) BDDC_CUDA_TRY(cudaEventRecord(F->join[i - 1], si));
     }
@@ -2595,11 +2653,17 @@ void prepare_batch_kernels() {
     cudaFuncSetAttribute(k_gemm_b<4, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(GM_S * gm_stage(32)));
     cudaFuncSetAttribute(k_gemm_b<1, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(GM_S * gm_stage(16)));
 #define BDDC_DIR_BS(T, A, SW)                                   \
-    BDDC_SMEM_ATTR_B((k_dir_bs<T, A, SW, false>));              \
-    BDDC_SMEM_ATTR_B((k_dir_bs<T, A, SW, true>));
+    BDDC_SMEM_ATTR_B((k_dir_bs<T, A, SW, false, kSBMaxT>));     \
+    BDDC_SMEM_ATTR_B((k_dir_bs<T, A, SW, true, kSBMaxT>));
+#define BDDC_DIR_BS_SMALL(T, SW)                                    \
+    BDDC_SMEM_ATTR_B((k_dir_bs<T, float, SW, false, kSBSmallT>));   \
+    BDDC_SMEM_ATTR_B((k_dir_bs<T, float, SW, true, kSBSmallT>));
     BDDC_DIR_BS(double, double, false) BDDC_DIR_BS(double, double, true)
     BDDC_DIR_BS(float, float, false) BDDC_DIR_BS(float, float, true)
     BDDC_DIR_BS(__nv_bfloat16, float, false) BDDC_DIR_BS(__nv_bfloat16, float, true)
+    BDDC_DIR_BS_SMALL(float, false) BDDC_DIR_BS_SMALL(float, true)
+    BDDC_DIR_BS_SMALL(__nv_bfloat16, false) BDDC_DIR_BS_SMALL(__nv_bfloat16, true)
+#undef BDDC_DIR_BS_SMALL
 #undef BDDC_DIR_BS
 #define BDDC_NEU_BG(T, A)                                       \
     BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 1>));                      \
