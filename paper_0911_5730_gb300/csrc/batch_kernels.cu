@@ -428,6 +428,12 @@ __global__ void __launch_bounds__(32 * lanes_per_rhs<BP>()) k_dir_b(DevLevel L, 
 // the block of their interior row at the start (a stable counting sort by
 // ballots), so each step applies only its own.
 constexpr int kLSW = 4, kLSRing = 4;
+// Rows of u_B (and half as many of r and z) in flight outside the sweeps, and
+// blocks per SM: with blocks of 8 rows the registers of 32 rows in flight
+// (166 a thread) left twelve warps per SM.  With half of them 24 warps: 16384
+// substructures, post 291 -> 279 us, 1024^2 FP32 solve of 32 91.7 -> 84.5 ms.
+__host__ __device__ constexpr int ls_rows(int bp) { return bp == 8 ? 16 : 32; }
+__host__ __device__ constexpr int ls_blocks(int bp) { return bp == 8 ? 6 : 0; }
 
 template <class T, int BP> struct LaneSmem {
     size_t slot, ring, bsm, vg, rec, srt, bst, bars, warp, total;
@@ -448,7 +454,7 @@ template <class T, int BP> struct LaneSmem {
 };
 
 template <class T, int BP, bool POST>
-__global__ void __launch_bounds__(32 * kLSW) k_dir_ls(DevLevel L, BatchLevel B, const double *r, double *z,
+__global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L, BatchLevel B, const double *r, double *z,
                                                      const int *skip, RzBatch rz) {
     using ACC = float;
     constexpr int BB = BP * BP;
@@ -504,11 +510,12 @@ __global__ void __launch_bounds__(32 * kLSW) k_dir_ls(DevLevel L, BatchLevel B, 
         const int *gP = reinterpret_cast<const int *>(rec + lay.pr);
         const int *gO = reinterpret_cast<const int *>(rec + lay.ow);
         float *ys = reinterpret_cast<float *>(B.ys) + L.offY[sub] * 32;
-        // post: the first 32 rows of u_B in flight while the entries are sorted
-        double uv[32];
+        // post: the first UV rows of u_B in flight while the entries are sorted
+        constexpr int UV = ls_rows(BP);
+        double uv[UV];
         if (POST) {
 #pragma unroll
-            for (int u = 0; u < 32; ++u) uv[u] = (u < nG && act) ? B.uB[(int64_t)gGi[u] * K + lane] : 0.0;
+            for (int u = 0; u < UV; ++u) uv[u] = (u < nG && act) ? B.uB[(int64_t)gGi[u] * K + lane] : 0.0;
         }
         // the coupling values narrowed in place: entry e's binary32 in the
         // first half of its binary64 slot (read and written by one lane)
@@ -553,14 +560,14 @@ __global__ void __launch_bounds__(32 * kLSW) k_dir_ls(DevLevel L, BatchLevel B, 
             }
         }
         if (POST) {
-            for (int q0 = 0; q0 < nG; q0 += 32) {
+            for (int q0 = 0; q0 < nG; q0 += UV) {
 #pragma unroll
-                for (int u = 0; u < 32; ++u)
+                for (int u = 0; u < UV; ++u)
                     if (q0 + u < nG) vG[(q0 + u) * 32 + lane] = from_f64<ACC>(uv[u]);
-                if (q0 + 32 < nG) {
+                if (q0 + UV < nG) {
 #pragma unroll
-                    for (int u = 0; u < 32; ++u) {
-                        const int q = q0 + 32 + u;
+                    for (int u = 0; u < UV; ++u) {
+                        const int q = q0 + UV + u;
                         uv[u] = (q < nG && act) ? B.uB[(int64_t)gGi[q] * K + lane] : 0.0;
                     }
                 }
@@ -722,17 +729,18 @@ __global__ void __launch_bounds__(32 * kLSW) k_dir_ls(DevLevel L, BatchLevel B, 
             // r.z over the interior entries just written (read back by the
             // lane that wrote them), in four partial sums
             double a4[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int i0 = 0; i0 < nI; i0 += 32) {
-                double rv[32], zv[32];
+            constexpr int RU = ls_rows(BP) / 2 * (BP == 8 ? 1 : 2);
+            for (int i0 = 0; i0 < nI; i0 += RU) {
+                double rv[RU], zv[RU];
 #pragma unroll
-                for (int u = 0; u < 32; ++u) {
+                for (int u = 0; u < RU; ++u) {
                     const bool in = i0 + u < nI;
                     const int64_t e = in ? (int64_t)gI[i0 + u] * K + lane : 0;
                     rv[u] = in ? r[e] : 0.0;
                     zv[u] = in ? z[e] : 0.0;
                 }
 #pragma unroll
-                for (int u = 0; u < 32; ++u) a4[u & 3] = fma(rv[u], zv[u], a4[u & 3]);
+                for (int u = 0; u < RU; ++u) a4[u & 3] = fma(rv[u], zv[u], a4[u & 3]);
             }
             acc = (a4[0] + a4[1]) + (a4[2] + a4[3]);
         }
