@@ -836,10 +836,10 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
 // s mod SBN, refilled SBN halves ahead as soon as it is used) needs no more
 // than what is in use and in flight, and turns round on the halves left in
 // it.  Thread t of a substructure with block size b owns column group
-// g = t / h (columns 4g..4g+3) and rows k and k + h (k = t mod h,
-// h = ceil(b/2)) of every block: a 2-row x 4-column register tile, so a
-// factor entry read from shared memory feeds four FMAs and a broadcast
-// 4-column vector eight, with four factor columns in flight.  Rows of a block
+// g = t / h (columns 4g..4g+3) and the R rows k, k + h, ... (k = t mod h,
+// h = ceil(b/R), R = bs_rows) of every block: an R-row x 4-column register
+// tile, so a factor entry read from shared memory feeds four FMAs and a
+// broadcast 4-column vector 4 R, with four factor columns in flight.  Rows of a block
 // are ld apart (odd unless swizzled), so the transposed walks of the backward
 // sweep are free of bank conflicts too.  The sweeps touch global memory only
 // through the factor's copies and a scratch [8][rows][4] per substructure in
@@ -853,18 +853,25 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
 // right-hand sides: 600 and 667 us before, 617 and 684 with whole products, 535
 // and 594 with the zeros of Lsub left out (which took the Voronoi solve from 130
 // to 124 ms).
-constexpr int SBN = 4, kSBMaxT = 32 * kMaxBuckets;   // ring slots, largest block
-constexpr int kSBSmallT = 192;                       // the common block sizes: more blocks per SM
+constexpr int kSBMaxT = 32 * kMaxBuckets;            // largest block
+constexpr int kSBSmallT = 96;                        // the common block sizes: more blocks per SM
+// Rows of a thread: four in the FP32 accumulator, so that a 4-column vector
+// feeds sixteen multiply-adds; two in FP64, whose pipe is the limit anyway.
+template <class ACC> __host__ __device__ constexpr int bs_rows() { return sizeof(ACC) == 4 ? 4 : 2; }
+// Slots of the ring: three where shared memory limits the blocks of an SM.
+template <class ACC> __host__ __device__ constexpr int bs_ring() { return sizeof(ACC) == 4 ? 3 : 4; }
 
+__host__ __device__ inline size_t red_doubles(int nt) { return nt > 256 ? (size_t)nt : 256; }
 struct StreamSmemB {
     size_t stage, ring, vec, red, total;
-    template <class T, class ACC> __host__ __device__ static StreamSmemB of(const DevLevel &L) {
+    template <class T, class ACC> __host__ __device__ static StreamSmemB of(const DevLevel &L, int nt) {
+        constexpr int SBN = bs_ring<ACC>();
         StreamSmemB m;
         const size_t mb = L.max_b > 0 ? L.max_b : 1, mld = L.max_ld > 0 ? L.max_ld : 1;
         m.stage = al16(mb * mld * sizeof(T) + 32);
         m.ring = SBN * m.stage;
         m.vec = al16(sizeof(ACC) * mb * kMaxBatch);   // [8][b][4]
-        m.red = al16(8 * 32 * kMaxBuckets + 16);      // r.z partials per warp and column, a flag
+        m.red = al16(8 * red_doubles(nt) + 16);       // r.z partials per warp and column, a flag
         m.total = m.ring + 2 * m.vec + m.red + 8 * SBN + 16;
         return m;
     }
@@ -886,61 +893,70 @@ __device__ __forceinline__ void st4(double *p, const double (&v)[4]) {
     reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
 }
 
-// a0 (row r0) and, with TWO, a1 (row r1) -= (SUB) or += sum over c in
-// [c0, c1) of M(r, c) v[c] for four columns.  COL: M(r, c) is the stored
-// entry (r, c) (a column walk); else the stored entry (c, r) (a row walk,
-// the transposed block).
-template <class T, class ACC, bool SUB, bool TWO, bool COL, bool SWZ>
-__device__ __forceinline__ void prod2(ACC (&a0)[4], ACC (&a1)[4], const T *M, int ldm, const ACC *v, int c0,
-                                      int c1, int r0, int r1) {
+// a[i] (row rw[i], F <= i < E) -= (SUB) or += sum over c in [c0, c1) of
+// M(row, c) v[c] for four columns.  COL: M(r, c) is the stored entry (r, c) (a
+// column walk); else the stored entry (c, r) (a row walk, the transposed block).
+template <class T, class ACC, bool SUB, bool COL, bool SWZ, int F, int E, int R>
+__device__ __forceinline__ void prod(ACC (&a)[R][4], const T *M, int ldm, const ACC *v, int c0, int c1,
+                                     const int (&rw)[R]) {
     auto at = [&](int r, int c) -> const T * {
         if (COL) return M + c * ldm + (SWZ ? (r ^ c) : r);
         return M + r * ldm + (SWZ ? (c ^ r) : c);
     };
-    auto fma4 = [&](ACC (&a)[4], ACC l, const ACC (&x)[4]) {
+    auto fma4 = [&](ACC (&y)[4], ACC l, const ACC (&x)[4]) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            if (SUB) a[q] -= l * x[q];
-            else a[q] += l * x[q];
+            if (SUB) y[q] -= l * x[q];
+            else y[q] += l * x[q];
         }
     };
     int c = c0;
     for (; c + 4 <= c1; c += 4) {
-        ACC x[4][4], l0[4], l1[4];
+        ACC x[4][4], l[4][R];
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) ld4(v + (c + cc) * 4, x[cc]);
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-            l0[cc] = ld<T, ACC>(at(r0, c + cc));
-            if (TWO) l1[cc] = ld<T, ACC>(at(r1, c + cc));
-        }
+        for (int cc = 0; cc < 4; ++cc)
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-            fma4(a0, l0[cc], x[cc]);
-            if (TWO) fma4(a1, l1[cc], x[cc]);
-        }
+            for (int i = F; i < E; ++i) l[cc][i] = ld<T, ACC>(at(rw[i], c + cc));
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+            for (int i = F; i < E; ++i) fma4(a[i], l[cc][i], x[cc]);
     }
     for (; c < c1; ++c) {
         ACC x[4];
         ld4(v + c * 4, x);
-        fma4(a0, ld<T, ACC>(at(r0, c)), x);
-        if (TWO) fma4(a1, ld<T, ACC>(at(r1, c)), x);
+#pragma unroll
+        for (int i = F; i < E; ++i) fma4(a[i], ld<T, ACC>(at(rw[i], c)), x);
     }
+}
+// a = Linv v (lower triangular, zeros stored above) or, with COL false, its
+// transpose: rows k, k + h, ...; row i of them has its columns in [0, (i + 1) h)
+// (transposed: [i h, b)), taken in segments of h columns
+template <class T, class ACC, bool COL, bool SWZ, int R, int SEG = 0>
+__device__ __forceinline__ void prod_tri(ACC (&a)[R][4], const T *M, int ldm, const ACC *v, int h, int b,
+                                         const int (&rw)[R]) {
+    const int c1 = (SEG + 1) * h < b ? (SEG + 1) * h : b;
+    if constexpr (COL) prod<T, ACC, false, true, SWZ, SEG, R, R>(a, M, ldm, v, SEG * h, c1, rw);
+    else prod<T, ACC, false, false, SWZ, 0, SEG + 1, R>(a, M, ldm, v, SEG * h, c1, rw);
+    if constexpr (SEG + 1 < R) prod_tri<T, ACC, COL, SWZ, R, SEG + 1>(a, M, ldm, v, h, b, rw);
 }
 
 template <class T, class ACC, bool SWZ, bool POST, int NT>
-__global__ void __launch_bounds__(NT, NT == kSBSmallT ? 4 : 1)
+__global__ void __launch_bounds__(NT, NT == kSBSmallT ? 6 : 1)
 k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, RzBatch rz, const int *perm,
          int count) {
+    constexpr int R = bs_rows<ACC>(), SBN = bs_ring<ACC>();   // rows of a thread, slots
     extern __shared__ __align__(16) unsigned char smem_bs[];
     if (skip && *skip) return;
     const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = nt >> 5;
-    const StreamSmemB ly = StreamSmemB::of<T, ACC>(L);
+    const StreamSmemB ly = StreamSmemB::of<T, ACC>(L, nt);
     unsigned char *ring = smem_bs;
     ACC *ybuf = reinterpret_cast<ACC *>(smem_bs + ly.ring);
     ACC *tbuf = reinterpret_cast<ACC *>(smem_bs + ly.ring + ly.vec);
     double *red = reinterpret_cast<double *>(smem_bs + ly.ring + 2 * ly.vec);
-    int *flag = reinterpret_cast<int *>(red + 32 * kMaxBuckets);
+    int *flag = reinterpret_cast<int *>(red + red_doubles(nt));
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem_bs + ly.ring + 2 * ly.vec + ly.red);
     const int K = B.K;
     const bool lact = lane < K;
@@ -953,7 +969,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
     for (int ti = blockIdx.x; ti < count; ti += gridDim.x) {
         const int sub = perm[ti];
         const int nI = L.nI[sub], nG = L.nG[sub], b = L.bsz[sub], m = nI > 0 ? L.nblk[sub] : 0;
-        const int mb = m * b, ldb = fld(b, SWZ), h = (b + 1) >> 1;
+        const int mb = m * b, ldb = fld(b, SWZ), h = (b + R - 1) / R;
         const T *F = O.dir + L.offF[sub];
         const size_t bsq = (size_t)b * ldb;
         const int *iI = L.idxI + L.offI[sub];
@@ -962,7 +978,10 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
         ACC *Yl = Ysub + (size_t)(lane >> 2) * mb * 4 + (lane & 3);            // this lane's column: row i at 4 i
         const bool act = tid < 8 * h;
         const int cg = act ? tid / h : 0, k = act ? tid - cg * h : 0;
-        const int r0 = k, r1 = k + h, r1c = r1 < b ? r1 : b - 1;   // r1 == b for odd b: computed, not kept
+        int rw[R];                        // its rows; beyond the block: computed on the last one, not kept
+#pragma unroll
+        for (int i = 0; i < R; ++i) rw[i] = k + i * h < b ? k + i * h : b - 1;
+        auto kept = [&](int i) { return k + i * h < b; };
         const bool colact = act && 4 * cg < K;
         ACC *Yg = Ysub + (size_t)cg * mb * 4;
         ACC *yb = ybuf + (size_t)cg * b * 4, *tb = tbuf + (size_t)cg * b * 4;
@@ -1025,50 +1044,49 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
             }
         }
         __syncthreads();
-        ACC n0[4], n1[4];                 // the next step's rows, loaded a step ahead
-        if (colact && m > 0) {
-            ld4(Yg + (size_t)r0 * 4, n0);
-            ld4(Yg + (size_t)r1c * 4, n1);
-        }
+        ACC nx[R][4];                     // the next step's rows, loaded a step ahead
+        if (colact && m > 0)
+#pragma unroll
+            for (int i = 0; i < R; ++i) ld4(Yg + (size_t)rw[i] * 4, nx[i]);
         // forward: y_j = Linv_j (rhs_j - Lsub_j y_{j-1})
         for (int j = 0; j < m; ++j) {
-            ACC a0[4], a1[4];
+            ACC a[R][4];
             if (colact) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) { a0[q] = n0[q]; a1[q] = n1[q]; }
-                if (j + 1 < m) {
-                    ld4(Yg + ((size_t)(j + 1) * b + r0) * 4, n0);
-                    ld4(Yg + ((size_t)(j + 1) * b + r1c) * 4, n1);
+                for (int i = 0; i < R; ++i) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[i][q] = nx[i][q];
+                    if (j + 1 < m) ld4(Yg + ((size_t)(j + 1) * b + rw[i]) * 4, nx[i]);
                 }
             }
             if (j > 0) {
                 wait_half(2 * j - 1);
-                if (colact) prod2<T, ACC, true, true, true, SWZ>(a0, a1, slot(2 * j - 1), ldb, yb, 0, b, r0, r1c);
+                if (colact) prod<T, ACC, true, true, SWZ, 0, R, R>(a, slot(2 * j - 1), ldb, yb, 0, b, rw);
             }
             if (colact) {
-                st4(tb + r0 * 4, a0);
-                if (r1 < b) st4(tb + r1 * 4, a1);
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+                    if (kept(i)) st4(tb + rw[i] * 4, a[i]);
             }
             wait_half(2 * j);
             __syncthreads();
             if (tid == 0 && ok && j > 0 && 2 * j - 1 + SBN < ns) issue(2 * j - 1 + SBN);
             if (colact) {
-                // Linv_j lower triangular (zeros stored above): row k needs
-                // columns < h only, row k + h all of them
-                const T *Li = slot(2 * j);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) a0[q] = a1[q] = 0;
-                prod2<T, ACC, false, true, true, SWZ>(a0, a1, Li, ldb, tb, 0, h, r0, r1c);
-                prod2<T, ACC, false, false, true, SWZ>(a1, a1, Li, ldb, tb, h, b, r1c, r1c);
-                st4(yb + r0 * 4, a0);
-                st4(Yg + ((size_t)j * b + r0) * 4, a0);
-                if (r1 < b) {
-                    st4(yb + r1 * 4, a1);
-                    st4(Yg + ((size_t)j * b + r1) * 4, a1);
+                for (int i = 0; i < R; ++i)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[i][q] = 0;
+                prod_tri<T, ACC, true, SWZ, R>(a, slot(2 * j), ldb, tb, h, b, rw);
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    if (kept(i)) {
+                        st4(yb + rw[i] * 4, a[i]);
+                        st4(Yg + ((size_t)j * b + rw[i]) * 4, a[i]);
+                    }
+                    if (j + 1 == m)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) nx[i][q] = a[i][q];   // y_{m-1}
                 }
-                if (j + 1 == m)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) { n0[q] = a0[q]; n1[q] = a1[q]; }   // y_{m-1}
             }
             __syncthreads();
             if (tid == 0 && ok && 2 * j + SBN < ns) issue(2 * j + SBN);
@@ -1076,41 +1094,40 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
         // backward: x_j = Linv_j^T (y_j - Lsub_{j+1}^T x_{j+1}); halves ns-1 ..
         // ns-SBN are still in the ring
         for (int j = m - 1; j >= 0; --j) {
-            ACC a0[4], a1[4];
+            ACC a[R][4];
             if (colact) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) { a0[q] = n0[q]; a1[q] = n1[q]; }
-                if (j > 0) {
-                    ld4(Yg + ((size_t)(j - 1) * b + r0) * 4, n0);
-                    ld4(Yg + ((size_t)(j - 1) * b + r1c) * 4, n1);
+                for (int i = 0; i < R; ++i) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[i][q] = nx[i][q];
+                    if (j > 0) ld4(Yg + ((size_t)(j - 1) * b + rw[i]) * 4, nx[i]);
                 }
             }
             if (j < m - 1) {
                 const int s = 2 * j + 1;
                 if (s < ns - SBN) wait_half(s);
-                if (colact) prod2<T, ACC, true, true, false, SWZ>(a0, a1, slot(s), ldb, yb, 0, b, r0, r1c);
+                if (colact) prod<T, ACC, true, false, SWZ, 0, R, R>(a, slot(s), ldb, yb, 0, b, rw);
             }
             if (colact) {
-                st4(tb + r0 * 4, a0);
-                if (r1 < b) st4(tb + r1 * 4, a1);
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+                    if (kept(i)) st4(tb + rw[i] * 4, a[i]);
             }
             if (2 * j < ns - SBN) wait_half(2 * j);
             __syncthreads();
             if (tid == 0 && ok && j < m - 1 && 2 * j + 1 - SBN >= 0) issue(2 * j + 1 - SBN);
             if (colact) {
-                // Linv_j^T upper triangular: row k needs all columns, row k + h
-                // columns >= h only
-                const T *Li = slot(2 * j);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) a0[q] = a1[q] = 0;
-                prod2<T, ACC, false, false, false, SWZ>(a0, a0, Li, ldb, tb, 0, h, r0, r0);
-                prod2<T, ACC, false, true, false, SWZ>(a0, a1, Li, ldb, tb, h, b, r0, r1c);
-                st4(yb + r0 * 4, a0);
-                st4(Yg + ((size_t)j * b + r0) * 4, a0);
-                if (r1 < b) {
-                    st4(yb + r1 * 4, a1);
-                    st4(Yg + ((size_t)j * b + r1) * 4, a1);
-                }
+                for (int i = 0; i < R; ++i)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[i][q] = 0;
+                prod_tri<T, ACC, false, SWZ, R>(a, slot(2 * j), ldb, tb, h, b, rw);
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+                    if (kept(i)) {
+                        st4(yb + rw[i] * 4, a[i]);
+                        st4(Yg + ((size_t)j * b + rw[i]) * 4, a[i]);
+                    }
             }
             __syncthreads();
             if (tid == 0 && ok && 2 * j - SBN >= 0) issue(2 * j - SBN);
@@ -1736,21 +1753,20 @@ __device__ void grid_reduce_k(double v, int K, double *part, unsigned *counter, 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // thread t sums blocks b = t / K, t / K + per, ... of right-hand side t % K
-    // (four independent partial sums, added in a fixed order)
+    // thread t sums blocks b = t / K, t / K + per, ... of right-hand side t % K,
+    // sixteen loads in flight (with four, the 1216 blocks of a vector kernel
+    // took 38 rounds of L2 latency)
     double s = 0.0;
     if ((int)threadIdx.x < per * K) {
         const int kk = threadIdx.x % K;
-        double s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        unsigned b = threadIdx.x / K;
-        for (; b + 3 * per < gridDim.x; b += 4 * per) {
-            s += __ldcg(&part[(int64_t)b * K + kk]);
-            s1 += __ldcg(&part[(int64_t)(b + per) * K + kk]);
-            s2 += __ldcg(&part[(int64_t)(b + 2 * per) * K + kk]);
-            s3 += __ldcg(&part[(int64_t)(b + 3 * per) * K + kk]);
+        for (int b = threadIdx.x / K; b < (int)gridDim.x; b += 16 * per) {
+            double u[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+                u[q] = b + q * per < (int)gridDim.x ? __ldcg(&part[(int64_t)(b + q * per) * K + kk]) : 0.0;
+#pragma unroll
+            for (int q = 0; q < 16; q += 4) s += (u[q] + u[q + 1]) + (u[q + 2] + u[q + 3]);
         }
-        for (; b < gridDim.x; b += per) s += __ldcg(&part[(int64_t)b * K + kk]);
-        s = (s + s1) + (s2 + s3);
     }
     red[threadIdx.x] = s;
     __syncthreads();
@@ -1768,34 +1784,98 @@ __device__ void grid_reduce_k(double v, int K, double *part, unsigned *counter, 
 
 struct NoPost { __device__ void operator()() const {} };
 
-__global__ void k_b_init(int n, int K, const double *b, int64_t ldb, double *x, double *r, double *p,
-                         double *part, unsigned *counter, BatchScalars *sc, double tol, int maxit) {
+// Tiles of kTG DOFs x K columns between the caller's layout (column k at
+// src + k * ld) and the interleaved one, through shared memory: both sides are
+// read and written in full rows.  (A thread per interleaved entry touched 8
+// bytes of every 32-byte sector of the caller's columns: 601 us for 32 columns
+// of the 1024^2 problem, where the bytes take 79.)
+constexpr int kTG = 64, kTT = 256;
+struct TileTr {
+    double v[kMaxBatch][kTG + 1];
+};
+// warp w loads the columns w, w + 8, ... of the DOFs [g0, g0 + kTG)
+__device__ __forceinline__ void tile_load(TileTr &t, int n, int K, const double *__restrict__ src, int64_t ld, int g0) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int u = 0; u < kMaxBatch / (kTT / 32); ++u) {
+        const int k = w + u * (kTT / 32);
+        if (k < K)
+#pragma unroll
+            for (int h = 0; h < kTG; h += 32)
+                t.v[k][h + lane] = g0 + h + lane < n ? src[(int64_t)k * ld + g0 + h + lane] : 0.0;
+    }
+}
+
+__global__ void __launch_bounds__(kTT) k_b_init(int n, int K, const double *b, int64_t ldb, double *x, double *r,
+                                                double *p, double *part, unsigned *counter, BatchScalars *sc,
+                                                double tol, int maxit) {
+    __shared__ TileTr t;
+    __shared__ bool last;
     pdl_wait();
     pdl_trigger();
-    const int k = threadIdx.x % K;
-    const int64_t nK = (int64_t)n * K;
-    double s = 0.0;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nK; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t g = e / K;
-        const double bv = b[(int64_t)k * ldb + g];
-        x[e] = 0.0;
-        r[e] = bv;
-        p[e] = 0.0;
-        s = fma(bv, bv, s);
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int NW = kTT / 32, PER = kMaxBatch / NW;
+    double s[PER] = {};                     // sums of squares of this warp's columns
+    for (int g0 = blockIdx.x * kTG; g0 < n; g0 += gridDim.x * kTG) {
+        tile_load(t, n, K, b, ldb, g0);
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int k = w + u * NW;
+            if (k < K)
+#pragma unroll
+                for (int h = 0; h < kTG; h += 32) s[u] = fma(t.v[k][h + lane], t.v[k][h + lane], s[u]);
+        }
+        __syncthreads();
+        const int cnt = min(kTG, n - g0) * K;
+        const int64_t e0 = (int64_t)g0 * K;
+        for (int q = threadIdx.x; q < cnt; q += kTT) {
+            x[e0 + q] = 0.0;
+            r[e0 + q] = t.v[q % K][q / K];
+            p[e0 + q] = 0.0;
+        }
+        __syncthreads();
     }
-    grid_reduce_k(s, K, part, counter,
-        [&](int kk, double tot) {
-            sc->bb[kk] = tot; sc->rr[kk] = tot; sc->tol2[kk] = tol * tol * tot;
-            sc->it[kk] = 0; sc->fresh[kk] = 1; sc->beta[kk] = 0.0; sc->hold[kk] = 0; sc->mx[kk] = maxit;
-            sc->conv[kk] = tot == 0.0 ? 1 : 0;
-            sc->done[kk] = tot == 0.0 ? 1 : 0;
-        },
-        [&]() {
-            sc->K = K; sc->maxit = maxit; sc->step = 0;
-            int all = 1;
-            for (int kk = 0; kk < K; ++kk) all &= sc->done[kk];
-            sc->all_done = all;
-        });
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+        const int k = w + u * NW;
+        if (lane == 0 && k < K) part[(int64_t)blockIdx.x * K + k] = s[u];
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // lane k: column k; the warps share the blocks, in a fixed order
+    double tot = 0.0;
+    if (lane < K)
+        for (int q = w; q < (int)gridDim.x; q += 8 * NW) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = q + u * NW < (int)gridDim.x ? __ldcg(&part[(int64_t)(q + u * NW) * K + lane]) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) tot += v[u];
+        }
+    t.v[w][lane] = tot;
+    __syncthreads();
+    if (w == 0 && lane < K) {
+        tot = 0.0;
+#pragma unroll
+        for (int u = 0; u < NW; ++u) tot += t.v[u][lane];
+        sc->bb[lane] = tot; sc->rr[lane] = tot; sc->tol2[lane] = tol * tol * tot;
+        sc->it[lane] = 0; sc->fresh[lane] = 1; sc->beta[lane] = 0.0; sc->hold[lane] = 0; sc->mx[lane] = maxit;
+        sc->conv[lane] = tot == 0.0 ? 1 : 0;
+        sc->done[lane] = tot == 0.0 ? 1 : 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sc->K = K; sc->maxit = maxit; sc->step = 0;
+        int all = 1;
+        for (int kk = 0; kk < K; ++kk) all &= sc->done[kk];
+        sc->all_done = all;
+        *counter = 0u;
+    }
 }
 
 // First half of a batched PCG iteration: p_new = z + beta p_old, q = A p_new
@@ -1884,7 +1964,9 @@ __global__ void k_b_dir_spmv(int nx, int K, const double *__restrict__ w, const 
         }, NoPost{});
 }
 
-// The same first half for more than kMarchMinK right-hand sides, a lane per
+// The same first half for more than kMarchMinK right-hand sides (a warp costs
+// the FP64 pipe the same for 21 lanes as for 32: 650 against 589 us for 21
+// right-hand sides on 1024^2, 652 against 856 for 32), a lane per
 // right-hand side and no tile: each warp marches up a strip of MW columns with
 // three rows of p_new in registers, so nothing meets at a barrier, and the
 // strips are cut into as many equal segments as there are resident warps (one
@@ -1894,11 +1976,9 @@ __global__ void k_b_dir_spmv(int nx, int K, const double *__restrict__ w, const 
 // end of their load phases.  Every weight read is in range (a missing
 // neighbour's p_new is zero and reads a finite weight), so the products need
 // no predicates, and their order is the tile kernel's: q is the same bit for
-// bit.
-// 32 right-hand sides: the 1024^2 three-level solve (46 iterations) 101 ->
-// 92 ms, the 512^2 FP64 solve 75.6 -> 72.5 ms, with the update kernel's loads
-// in flight.
-constexpr int MW = 8, kMarchT = 256, kMarchPerSm = 2, kMarchMinK = 16;
+// bit.  32 right-hand sides: the 1024^2 three-level solve (46 iterations)
+// 101 -> 92 ms (the kernel 856 -> 652 us), the 512^2 FP64 solve 75.6 -> 72.5 ms.
+constexpr int MW = 8, kMarchT = 256, kMarchPerSm = 2, kMarchMinK = 24;
 __global__ void __launch_bounds__(kMarchT, kMarchPerSm)
 k_b_dir_march(int nx, int K, const double *__restrict__ w, const double *__restrict__ z, double *p0, double *p1,
               double *__restrict__ q, double *part, unsigned *counter, BatchScalars *sc, double *alphas, int strips,
@@ -2025,25 +2105,7 @@ __global__ void k_b_update(int64_t nK, int K, double *__restrict__ x, double *__
     const double a = sc->alpha[k];
     double s = 0.0;
     if (live) {
-        // four entries per round: sixteen independent loads in flight
-        const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-        int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-        for (; e + 3 * stride < nK; e += 4 * stride) {
-            double pv[4], qv[4], xv[4], rv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                pv[u] = p[e + u * stride]; qv[u] = q[e + u * stride];
-                xv[u] = x[e + u * stride]; rv[u] = r[e + u * stride];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                x[e + u * stride] = fma(a, pv[u], xv[u]);
-                const double ri = fma(-a, qv[u], rv[u]);
-                r[e + u * stride] = ri;
-                s = fma(ri, ri, s);
-            }
-        }
-        for (; e < nK; e += stride) {
+        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nK; e += (int64_t)gridDim.x * blockDim.x) {
             x[e] = fma(a, p[e], x[e]);
             const double ri = fma(-a, q[e], r[e]);
             r[e] = ri;
@@ -2103,17 +2165,24 @@ __global__ void k_b_norm2(int64_t nK, int K, const double *v, double *part, unsi
 
 
 // dst[g * K + k] = src[k * ld + g] and back
-__global__ void k_b_gather(int n, int K, const double *src, int64_t ld, double *dst) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)n * K) return;
-    const int k = (int)(e % K);
-    dst[e] = src[(int64_t)k * ld + e / K];
+__global__ void __launch_bounds__(kTT) k_b_gather(int n, int K, const double *src, int64_t ld, double *dst) {
+    __shared__ TileTr t;
+    const int g0 = blockIdx.x * kTG;
+    tile_load(t, n, K, src, ld, g0);
+    __syncthreads();
+    const int cnt = min(kTG, n - g0) * K;
+    for (int q = threadIdx.x; q < cnt; q += kTT) dst[(int64_t)g0 * K + q] = t.v[q % K][q / K];
 }
-__global__ void k_b_scatter(int n, int K, const double *src, double *dst, int64_t ld) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)n * K) return;
-    const int k = (int)(e % K);
-    dst[(int64_t)k * ld + e / K] = src[e];
+__global__ void __launch_bounds__(kTT) k_b_scatter(int n, int K, const double *src, double *dst, int64_t ld) {
+    __shared__ TileTr t;
+    const int g0 = blockIdx.x * kTG, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cnt = min(kTG, n - g0) * K;
+    for (int q = threadIdx.x; q < cnt; q += kTT) t.v[q % K][q / K] = src[(int64_t)g0 * K + q];
+    __syncthreads();
+    for (int k = w; k < K; k += kTT / 32)
+#pragma unroll
+        for (int h = 0; h < kTG; h += 32)
+            if (g0 + h + lane < n) dst[(int64_t)k * ld + g0 + h + lane] = t.v[k][h + lane];
 }
 
 // A new right-hand side in slot k of a running batch.
@@ -2339,7 +2408,7 @@ template <class T, class ACC> BatchRoute route_t(const DevLevel &L, int prec) {
     // the largest bucket's layout bounds every bucket's
     const int nw_max = ((L.max_b + 1) / 2 + 3) / 4;
     const bool stream = L.bk.n > 0 && L.bperm && nw_max <= kMaxBuckets &&
-                        StreamSmemB::of<T, ACC>(L).total <= kSmemMaxB;
+                        StreamSmemB::of<T, ACC>(L, 32 * nw_max).total <= kSmemMaxB;
     const bool bg = neu_bg_smem<T, ACC>(L) <= kSmemMaxB && avg_bg_smem<T, ACC>(L) <= kSmemMaxB;
     R.dir_stream = !R.dir_staged && stream;
     R.stream_fits = stream;
@@ -2424,8 +2493,9 @@ void dir_bs_buckets(const DevLevel &L, const BatchLevel &B, const double *r, dou
         Lb.max_b = L.bk.max_b[i];
         Lb.max_ld = L.bk.max_ld[i];
         Lb.max_nG = L.bk.max_nG[i];
-        const int nt = 32 * L.bk.nw[i];
-        const size_t sm = StreamSmemB::of<T, ACC>(Lb).total;
+        // the bucket's warps are those of two rows a thread
+        const int nt = bs_rows<ACC>() == 2 ? 32 * L.bk.nw[i] : 32 * ((L.bk.nw[i] + 1) / 2);
+        const size_t sm = StreamSmemB::of<T, ACC>(Lb, nt).total;
         auto kern = k_dir_bs<T, ACC, SWZ, POST, kSBMaxT>;
         if constexpr (sizeof(ACC) == 4)       // (FP64 wants the 128 registers)
             if (nt <= kSBSmallT) kern = k_dir_bs<T, ACC, SWZ, POST, kSBSmallT>;
@@ -2767,8 +2837,10 @@ int gemm_rows(int variant, int n) {
 void launch_b_init(int n, int K, const double *b, int64_t ldb, double *x, double *r, double *p,
                    double *part, unsigned *counter, BatchScalars *sc, double tol, int maxit,
                    cudaStream_t s) {
-    const int64_t nK = (int64_t)n * K;
-    k_b_init<<<vgrid_b(nK, K), bblock(K), 0, s>>>(n, K, b, ldb, x, r, p, part, counter, sc, tol, maxit);
+    int g = (n + kTG - 1) / kTG;
+    const int cap = 8 * num_sms_b() < kMaxVecGrid ? 8 * num_sms_b() : kMaxVecGrid;
+    if (g > cap) g = cap;
+    k_b_init<<<g < 1 ? 1 : g, kTT, 0, s>>>(n, K, b, ldb, x, r, p, part, counter, sc, tol, maxit);
 }
 template <int TX, int TY> int tile_blocks(int nx) {
     const int n1 = nx - 1;
@@ -2868,12 +2940,10 @@ void launch_fp64_rate(int iters, double *out, cudaStream_t s) {
     k_fp64_rate<<<kFmaBlocksPerSm * num_sms_b(), 256, 0, s>>>(iters, 0.9999999, 1e-9, out);
 }
 void launch_b_gather(int n, int K, const double *src, int64_t ld, double *dst, cudaStream_t s) {
-    const int64_t nK = (int64_t)n * K;
-    if (nK > 0) k_b_gather<<<(int)((nK + 255) / 256), 256, 0, s>>>(n, K, src, ld, dst);
+    if (n > 0) k_b_gather<<<(n + kTG - 1) / kTG, kTT, 0, s>>>(n, K, src, ld, dst);
 }
 void launch_b_scatter(int n, int K, const double *src, double *dst, int64_t ld, cudaStream_t s) {
-    const int64_t nK = (int64_t)n * K;
-    if (nK > 0) k_b_scatter<<<(int)((nK + 255) / 256), 256, 0, s>>>(n, K, src, dst, ld);
+    if (n > 0) k_b_scatter<<<(n + kTG - 1) / kTG, kTT, 0, s>>>(n, K, src, dst, ld);
 }
 
 }  // namespace bddc
