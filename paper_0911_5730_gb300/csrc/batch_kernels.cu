@@ -453,7 +453,8 @@ template <class T, int BP> struct LaneSmem {
     }
 };
 
-template <class T, int BP, bool POST>
+// TRI: L.sub_tri
+template <class T, int BP, bool POST, bool TRI>
 __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L, BatchLevel B, const double *r, double *z,
                                                      const int *skip, RzBatch rz) {
     using ACC = float;
@@ -629,7 +630,8 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                     ACC col[BP];
                     load_vec<T, ACC, BP>(Ls + c * BP, col);
 #pragma unroll
-                    for (int q = 0; q < BP; ++q) t[q] -= col[q ^ c] * xp[c];
+                    for (int q = 0; q < BP; ++q)
+                        if (!TRI || q <= c) t[q] -= col[q ^ c] * xp[c];
                 }
             }
 #pragma unroll
@@ -667,11 +669,11 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                 for (int q = 0; q < BP; ++q) y[q] = j >= 0 ? ys[(j * BP + q) * 32 + lane] : (ACC)0;
             };
             // column dot products in four partial sums (fixed order)
-            auto dot4 = [](const ACC (&col)[BP], const ACC (&v)[BP], int c, int q0) -> ACC {
+            auto dot4 = [](const ACC (&col)[BP], const ACC (&v)[BP], int c, int q0, int q1) -> ACC {
                 ACC a[4] = {0, 0, 0, 0};
 #pragma unroll
                 for (int q = 0; q < BP; ++q)
-                    if (q >= q0) a[q & 3] += col[q ^ c] * v[q];
+                    if (q >= q0 && q < q1) a[q & 3] += col[q ^ c] * v[q];
                 return (a[0] + a[1]) + (a[2] + a[3]);
             };
             auto bstep = [&](int j, ACC (&y)[BP]) -> bool {
@@ -687,7 +689,7 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                     for (int c = 0; c < BP; ++c) {
                         ACC col[BP];
                         load_vec<T, ACC, BP>(Ls1 + c * BP, col);
-                        t[c] -= dot4(col, zn, c, 0);
+                        t[c] -= dot4(col, zn, c, 0, TRI ? c + 1 : BP);
                     }
                 }
                 const T *Li = ring + (size_t)s * 2 * BB;
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                 for (int c = 0; c < BP; ++c) {
                     ACC col[BP];
                     load_vec<T, ACC, BP>(Li + c * BP, col);
-                    zn[c] = dot4(col, t, c, c);
+                    zn[c] = dot4(col, t, c, c, BP);
                 }
                 if (POST) {
 #pragma unroll
@@ -931,16 +933,16 @@ __device__ __forceinline__ void prod(ACC (&a)[R][4], const T *M, int ldm, const 
         for (int i = F; i < E; ++i) fma4(a[i], ld<T, ACC>(at(rw[i], c)), x);
     }
 }
-// a = Linv v (lower triangular, zeros stored above) or, with COL false, its
-// transpose: rows k, k + h, ...; row i of them has its columns in [0, (i + 1) h)
-// (transposed: [i h, b)), taken in segments of h columns
-template <class T, class ACC, bool COL, bool SWZ, int R, int SEG = 0>
-__device__ __forceinline__ void prod_tri(ACC (&a)[R][4], const T *M, int ldm, const ACC *v, int h, int b,
-                                         const int (&rw)[R]) {
-    const int c1 = (SEG + 1) * h < b ? (SEG + 1) * h : b;
-    if constexpr (COL) prod<T, ACC, false, true, SWZ, SEG, R, R>(a, M, ldm, v, SEG * h, c1, rw);
-    else prod<T, ACC, false, false, SWZ, 0, SEG + 1, R>(a, M, ldm, v, SEG * h, c1, rw);
-    if constexpr (SEG + 1 < R) prod_tri<T, ACC, COL, SWZ, R, SEG + 1>(a, M, ldm, v, h, b, rw);
+// The same over all columns of an M with a triangle of zeros, for the rows k,
+// k + h, ... of a thread: M(row, c) is zero for c > row + d (LOW) or c < row - d,
+// so row i of them has its columns below (i + 1) h + d or from i h - d on, taken
+// in R segments.
+template <class T, class ACC, bool SUB, bool COL, bool SWZ, bool LOW, int R, int SEG = 0>
+__device__ __forceinline__ void prod_tri(ACC (&a)[R][4], const T *M, int ldm, const ACC *v, int h, int b, int d,
+                                         const int (&rw)[R], int c0 = 0) {
+    const int e = SEG + 1 == R ? b : LOW ? min(b, (SEG + 1) * h + d) : max(0, (SEG + 1) * h - d);
+    prod<T, ACC, SUB, COL, SWZ, LOW ? SEG : 0, LOW ? R : SEG + 1, R>(a, M, ldm, v, c0, e, rw);
+    if constexpr (SEG + 1 < R) prod_tri<T, ACC, SUB, COL, SWZ, LOW, R, SEG + 1>(a, M, ldm, v, h, b, d, rw, e);
 }
 
 template <class T, class ACC, bool SWZ, bool POST, int NT>
@@ -970,6 +972,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
         const int sub = perm[ti];
         const int nI = L.nI[sub], nG = L.nG[sub], b = L.bsz[sub], m = nI > 0 ? L.nblk[sub] : 0;
         const int mb = m * b, ldb = fld(b, SWZ), h = (b + R - 1) / R;
+        const int dz = L.sub_over[sub];   // Lsub is zero left of column row - dz
         const T *F = O.dir + L.offF[sub];
         const size_t bsq = (size_t)b * ldb;
         const int *iI = L.idxI + L.offI[sub];
@@ -1061,7 +1064,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
             }
             if (j > 0) {
                 wait_half(2 * j - 1);
-                if (colact) prod<T, ACC, true, true, SWZ, 0, R, R>(a, slot(2 * j - 1), ldb, yb, 0, b, rw);
+                if (colact) prod_tri<T, ACC, true, true, SWZ, false, R>(a, slot(2 * j - 1), ldb, yb, h, b, dz, rw);
             }
             if (colact) {
 #pragma unroll
@@ -1076,7 +1079,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
                 for (int i = 0; i < R; ++i)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) a[i][q] = 0;
-                prod_tri<T, ACC, true, SWZ, R>(a, slot(2 * j), ldb, tb, h, b, rw);
+                prod_tri<T, ACC, false, true, SWZ, true, R>(a, slot(2 * j), ldb, tb, h, b, 0, rw);   // Linv_j
 #pragma unroll
                 for (int i = 0; i < R; ++i) {
                     if (kept(i)) {
@@ -1106,7 +1109,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
             if (j < m - 1) {
                 const int s = 2 * j + 1;
                 if (s < ns - SBN) wait_half(s);
-                if (colact) prod<T, ACC, true, false, SWZ, 0, R, R>(a, slot(s), ldb, yb, 0, b, rw);
+                if (colact) prod_tri<T, ACC, true, false, SWZ, true, R>(a, slot(s), ldb, yb, h, b, dz, rw);
             }
             if (colact) {
 #pragma unroll
@@ -1121,7 +1124,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
                 for (int i = 0; i < R; ++i)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) a[i][q] = 0;
-                prod_tri<T, ACC, false, SWZ, R>(a, slot(2 * j), ldb, tb, h, b, rw);
+                prod_tri<T, ACC, false, false, SWZ, false, R>(a, slot(2 * j), ldb, tb, h, b, 0, rw);   // its transpose
 #pragma unroll
                 for (int i = 0; i < R; ++i)
                     if (kept(i)) {
@@ -2298,13 +2301,11 @@ void dir_ls(const DevLevel &L, const BatchLevel &B, bool post, const double *r, 
         const RzBatch rzv = (post && rz) ? *rz : none;
         const size_t sm = lane_smem<T, ACC>(L);
         const int grid = (L.nsub + kLSW - 1) / kLSW;
-        if (L.bp == 8) {
-            if (post) launch_plain(k_dir_ls<T, 8, true>, grid, 32 * kLSW, sm, s, L, B, r, z, skip, rzv);
-            else launch_plain(k_dir_ls<T, 8, false>, grid, 32 * kLSW, sm, s, L, B, r, z, skip, rzv);
-        } else {
-            if (post) launch_plain(k_dir_ls<T, 16, true>, grid, 32 * kLSW, sm, s, L, B, r, z, skip, rzv);
-            else launch_plain(k_dir_ls<T, 16, false>, grid, 32 * kLSW, sm, s, L, B, r, z, skip, rzv);
-        }
+        const auto k8 = L.sub_tri ? (post ? k_dir_ls<T, 8, true, true> : k_dir_ls<T, 8, false, true>)
+                                  : (post ? k_dir_ls<T, 8, true, false> : k_dir_ls<T, 8, false, false>);
+        const auto k16 = L.sub_tri ? (post ? k_dir_ls<T, 16, true, true> : k_dir_ls<T, 16, false, true>)
+                                   : (post ? k_dir_ls<T, 16, true, false> : k_dir_ls<T, 16, false, false>);
+        launch_plain(L.bp == 8 ? k8 : k16, grid, 32 * kLSW, sm, s, L, B, r, z, skip, rzv);
     } else {
         throw Error(BDDC_E_STATE, "lane Dirichlet kernel in FP64");
     }
@@ -2711,8 +2712,10 @@ void prepare_batch_kernels() {
     BDDC_SMEM_ATTR_B((k_dir_b<T, A, BPV, false>));              \
     BDDC_SMEM_ATTR_B((k_dir_b<T, A, BPV, true>));
 #define BDDC_DIR_LS(T, BPV)                                     \
-    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, false>));                \
-    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, true>));
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, false, false>));         \
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, true, false>));          \
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, false, true>));          \
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, true, true>));
     BDDC_DIR_LS(float, 8) BDDC_DIR_LS(float, 16) BDDC_DIR_LS(__nv_bfloat16, 8) BDDC_DIR_LS(__nv_bfloat16, 16)
 #undef BDDC_DIR_LS
     BDDC_DIR_B(double, double, 8) BDDC_DIR_B(double, double, 16) BDDC_DIR_B(double, double, 32)

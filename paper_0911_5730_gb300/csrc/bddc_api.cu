@@ -535,6 +535,13 @@ void setup_level(bddc_ctx *C, LevelData &LD, const double *emat, const std::vect
         D.max_nI = std::max(D.max_nI, nI[s]); D.max_nG = std::max(D.max_nG, nG[s]);
         D.max_b = std::max(D.max_b, bsz[s]); D.max_m = std::max(D.max_m, nblk[s]);
     }
+    std::vector<int> over(ns);
+    D.sub_tri = 1;
+    for (int s = 0; s < ns; ++s) {
+        over[s] = std::max(0, bw[s] - bsz[s]);
+        if (over[s]) D.sub_tri = 0;
+    }
+    D.sub_over = A.upload(over, st);
     std::vector<int64_t> szY(ns);
     for (int s = 0; s < ns; ++s) szY[s] = (int64_t)nblk[s] * bsz[s];
     auto oI = prefix(nI), oF = prefix(szF), oN = prefix(szN), oCOO = prefix(cooCnt), oY = prefix(szY);

@@ -114,6 +114,11 @@ struct DevLevel {
     int nc = 0;           // coarse DOFs (= DOFs of the next level)
     int max_nI = 0, max_nG = 0, max_nc = 0, max_b = 0, max_m = 0, max_coo = 0;
     int max_ld = 0;            // largest leading dimension of a factor block
+    // entry (r, c) of every Lsub of substructure s is zero for c < r - sub_over[s]
+    // (its interior's bandwidth less its block size, at least 0); sub_tri: all
+    // are 0, Lsub is upper triangular.  The batch Dirichlet kernels skip the zeros.
+    const int *sub_over = nullptr;
+    int sub_tri = 0;
     // the batch autotuner's route per precision index p (FP64 0, FP32 1,
     // BF16 2): bit 2p: the streaming Dirichlet kernel where the staged one
     // also fits; bit 2p+1: the chunked Neumann / averaging kernels likewise;
