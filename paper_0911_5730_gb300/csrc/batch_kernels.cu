@@ -413,57 +413,68 @@ __global__ void __launch_bounds__(32 * lanes_per_rhs<BP>()) k_dir_b(DevLevel L, 
 }
 
 // The Dirichlet corrections with a lane per right-hand side, streamed
-// (blocks of up to 16 rows, FP32 accumulation).  A block of kLSW warps takes
-// kLSW substructures, one per warp, so every warp of the SM runs sweeps and
-// little shared memory is needed per substructure: the factor blocks come
-// through a ring of kLSRing slots (block j in slot j % kLSRing, copied
-// kLSRing steps ahead; the backward sweep starts from the blocks left in the
-// ring and refills the slot of block j+1 after step j), the right-hand side
-// rows of block j are loaded into registers two steps ahead, and the forward
-// sweep's y_j go to the sweep scratch (same thread writes and reads them
-// back, two steps ahead).  Each lane holds all rows of its right-hand side's
+// (blocks of up to 16 rows).  A block takes as many substructures as it has
+// warps, one per warp, so every warp of the SM runs sweeps and little shared
+// memory is needed per substructure: the factor blocks come through a ring of
+// slots (unit u in slot u mod the slots, copied that many units ahead; the
+// backward sweep starts from the units left in the ring), the right-hand side
+// rows of block j are loaded into registers two steps ahead (FP64: one), and
+// the forward sweep's y_j go to the sweep scratch (same thread writes and
+// reads them back, as far ahead).  Each lane holds all rows of its right-hand side's
 // block: a factor column is a broadcast read feeding BP multiply-adds per
 // lane and no value crosses lanes.  The coupling entries A_{I Gamma} (post:
 // b_I -= A_{I Gamma} u_B; pre: the product A_{Gamma I} x_I) are grouped by
 // the block of their interior row at the start (a stable counting sort by
-// ballots), so each step applies only its own.
-constexpr int kLSW = 4, kLSRing = 4;
+// ballots), so each step applies only its own.  The blocks' zero triangles are
+// skipped exactly (TRI: those of L_{j,j-1} too), which a block's warps that
+// share rows can do only by halves.
+// The ring's unit is a block in FP32, half a block (the sequence Linv_0, Lsub_1,
+// Linv_1, ...) in FP64.  There the double pipe bounds the kernel and a
+// substructure of the 16 x 16-element kind takes 30 KB with three half blocks:
+// seven of them share an SM, one wave of 1024 substructures: 436 us before and
+// 462 us after the coarse solve for 32 right-hand sides, where the streaming
+// kernel takes 535 and 594 (with two whole blocks in the ring six share an SM,
+// and the second wave brought it to 598 and 649).
+template <class ACC> __host__ __device__ constexpr int ls_ring() { return sizeof(ACC) == 4 ? 4 : 3; }
+template <class ACC, int BP> __host__ __device__ constexpr int ls_max_warps() { return sizeof(ACC) == 8 && BP == 16 ? 7 : 4; }
 // Rows of u_B (and half as many of r and z) in flight outside the sweeps, and
 // blocks per SM: with blocks of 8 rows the registers of 32 rows in flight
 // (166 a thread) left twelve warps per SM.  With half of them 24 warps: 16384
 // substructures, post 291 -> 279 us, 1024^2 FP32 solve of 32 91.7 -> 84.5 ms.
-__host__ __device__ constexpr int ls_rows(int bp) { return bp == 8 ? 16 : 32; }
-__host__ __device__ constexpr int ls_blocks(int bp) { return bp == 8 ? 6 : 0; }
+template <class ACC> __host__ __device__ constexpr int ls_rows(int bp) { return bp == 8 || sizeof(ACC) == 8 ? 16 : 32; }
+template <class ACC> __host__ __device__ constexpr int ls_blocks(int bp) { return bp == 8 && sizeof(ACC) == 4 ? 6 : 0; }
 
-template <class T, int BP> struct LaneSmem {
-    size_t slot, ring, bsm, vg, rec, srt, bst, bars, warp, total;
-    __host__ __device__ static LaneSmem of(const DevLevel &L) {
+template <class T, class ACC, int BP> struct LaneSmem {
+    size_t unit, ring, bsm, vg, rec, srt, bst, bars, warp, total;
+    __host__ __device__ static LaneSmem of(const DevLevel &L, int warps) {
         LaneSmem m;
-        m.slot = al16(2 * (size_t)BP * BP * sizeof(T));
-        m.ring = kLSRing * m.slot;
-        m.bsm = al16(sizeof(float) * BP * 32);
-        m.vg = al16(sizeof(float) * (size_t)(L.max_nG > 0 ? L.max_nG : 1) * 32);
+        m.unit = (sizeof(ACC) == 4 ? 2 : 1) * (size_t)BP * BP * sizeof(T);
+        m.ring = ls_ring<ACC>() * m.unit;
+        m.bsm = al16(sizeof(ACC) * BP * 32);
+        m.vg = al16(sizeof(ACC) * (size_t)(L.max_nG > 0 ? L.max_nG : 1) * 32);
         m.rec = al16((size_t)L.max_irec);
         m.srt = al16(2 * (size_t)(L.max_coo > 0 ? L.max_coo : 1));
         m.bst = al16(2 * (size_t)(L.max_m + 2));
-        m.bars = al16(8 * (kLSRing + 1));
+        m.bars = al16(8 * (ls_ring<ACC>() + 1));
         m.warp = m.ring + m.bsm + m.vg + m.rec + m.srt + m.bst + m.bars;
-        m.total = kLSW * m.warp + al16(8 * 32 * kLSW + 16);
+        m.total = warps * m.warp + al16(8 * 32 * warps + 16);
         return m;
     }
 };
 
 // TRI: L.sub_tri
-template <class T, int BP, bool POST, bool TRI>
-__global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L, BatchLevel B, const double *r, double *z,
-                                                     const int *skip, RzBatch rz) {
-    using ACC = float;
-    constexpr int BB = BP * BP;
+template <class T, class ACC, int BP, bool POST, bool TRI>
+__global__ void __launch_bounds__(32 * ls_max_warps<ACC, BP>(), ls_blocks<ACC>(BP))
+k_dir_ls(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, RzBatch rz) {
+    constexpr int NS = ls_ring<ACC>(), BB = BP * BP;
+    constexpr bool HALF = sizeof(ACC) == 8;
+    constexpr int UE = HALF ? BB : 2 * BB;   // elements of a ring unit
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem_ls[];
-    const LaneSmem<T, BP> ly = LaneSmem<T, BP>::of(L);
+    const int nwb = blockDim.x >> 5;
+    const LaneSmem<T, ACC, BP> ly = LaneSmem<T, ACC, BP>::of(L, nwb);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int sub = blockIdx.x * kLSW + warp;
+    const int sub = blockIdx.x * nwb + warp;
     const bool live = sub < L.nsub;
     const int K = B.K;
     const bool act = lane < K;
@@ -475,56 +486,63 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
     unsigned short *srt = reinterpret_cast<unsigned short *>(p);   p += ly.srt;
     unsigned short *bst = reinterpret_cast<unsigned short *>(p);   p += ly.bst;
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(p);   // ring slots, then the record
-    double *red = reinterpret_cast<double *>(smem_ls + (size_t)kLSW * ly.warp);   // [kLSW][32]
-    int *flag = reinterpret_cast<int *>(red + 32 * kLSW);
+    double *red = reinterpret_cast<double *>(smem_ls + (size_t)nwb * ly.warp);   // [nwb][32]
+    int *flag = reinterpret_cast<int *>(red + 32 * nwb);
 
     const int nI = live ? L.nI[sub] : 0, nG = live ? L.nG[sub] : 0, m = live ? L.nblk[sub] : 0;
     const int ncoo = live ? L.ncoo[sub] : 0, nown = live ? L.nown[sub] : 0;
     const IRecLayout lay(nI, nG, ncoo, nown);
-    const unsigned slot_bytes = 2u * BB * (unsigned)sizeof(T);
+    const unsigned unit_bytes = (unsigned)(UE * sizeof(T));
+    const int nu = HALF ? 2 * m - 1 : m;
     const T *F = live ? Ops<T>::get(L).dir + L.offF[sub] : nullptr;
     unsigned ph = 0, pend = 0;      // per ring slot: parity of its next completion, a copy in flight
     bool ok = true;
     double acc = 0.0;               // post: r.z over the entries of z this substructure writes
+    auto refill = [&](int u) {      // unit u into its slot, which every lane is done with
+        const int s = u % NS;
+        if (lane == 0) {
+            const T *src = HALF ? F + (size_t)((u + 1) / 2 * 2 + (u & 1)) * BB : F + (size_t)u * UE;
+            mbar_expect(&bars[s], unit_bytes);
+            bulk_copy(ring + (size_t)s * UE, src, unit_bytes, &bars[s]);
+        }
+        pend |= 1u << s;
+    };
+    auto unit = [&](int u) -> const T * { return ring + (size_t)(u % NS) * UE; };
     if (live) {
         if (lane == 0) {
-            for (int s = 0; s <= kLSRing; ++s) mbar_init(&bars[s]);
-            mbar_expect(&bars[kLSRing], (unsigned)lay.bytes);
-            bulk_copy(rec, L.irec + L.irecOff[sub], (unsigned)lay.bytes, &bars[kLSRing]);
+            for (int s = 0; s <= NS; ++s) mbar_init(&bars[s]);
+            mbar_expect(&bars[NS], (unsigned)lay.bytes);
+            bulk_copy(rec, L.irec + L.irecOff[sub], (unsigned)lay.bytes, &bars[NS]);
         }
         __syncwarp();
-        for (int j = 0; j < m && j < kLSRing; ++j) {
-            if (lane == 0) {
-                mbar_expect(&bars[j], slot_bytes);
-                bulk_copy(ring + (size_t)j * 2 * BB, F + (size_t)j * 2 * BB, slot_bytes, &bars[j]);
-            }
-            pend |= 1u << j;
-        }
+        for (int u = 0; u < nu && u < NS; ++u) refill(u);
     }
     pdl_wait();
     pdl_trigger();
-    if (live) ok = __all_sync(0xffffffffu, mbar_wait(&bars[kLSRing], 0));
+    if (live) ok = __all_sync(0xffffffffu, mbar_wait(&bars[NS], 0));
     if (live && ok) {
         const double *gC = reinterpret_cast<const double *>(rec + lay.cv);
         const int *gI = reinterpret_cast<const int *>(rec + lay.iI);
         const int *gGi = reinterpret_cast<const int *>(rec + lay.iG);
         const int *gP = reinterpret_cast<const int *>(rec + lay.pr);
         const int *gO = reinterpret_cast<const int *>(rec + lay.ow);
-        float *ys = reinterpret_cast<float *>(B.ys) + L.offY[sub] * 32;
+        ACC *ys = reinterpret_cast<ACC *>(B.ys) + L.offY[sub] * 32;
         // post: the first UV rows of u_B in flight while the entries are sorted
-        constexpr int UV = ls_rows(BP);
+        constexpr int UV = ls_rows<ACC>(BP);
         double uv[UV];
         if (POST) {
 #pragma unroll
             for (int u = 0; u < UV; ++u) uv[u] = (u < nG && act) ? B.uB[(int64_t)gGi[u] * K + lane] : 0.0;
         }
-        // the coupling values narrowed in place: entry e's binary32 in the
+        // FP32: the coupling values narrowed in place, entry e's binary32 in the
         // first half of its binary64 slot (read and written by one lane)
+        constexpr int CS = 8 / sizeof(ACC);
         ACC *cvs = reinterpret_cast<ACC *>(rec + lay.cv);
-        for (int e = lane; e < ncoo; e += 32) {
-            const double v = gC[e];
-            cvs[2 * e] = from_f64<ACC>(v);
-        }
+        if (CS > 1)
+            for (int e = lane; e < ncoo; e += 32) {
+                const double v = gC[e];
+                cvs[CS * e] = from_f64<ACC>(v);
+            }
         {
             // entries by the block of their interior row, in entry order
             // within a block: counts (shared atomics), their prefix sums, then
@@ -581,6 +599,7 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
         }
         __syncwarp();
 
+        constexpr int AH = sizeof(ACC) == 4 ? 2 : 1;   // blocks of rows in flight
         auto load_rows = [&](double (&d)[BP], int j) {
 #pragma unroll
             for (int q = 0; q < BP; ++q) {
@@ -588,18 +607,12 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                 d[q] = (j >= 0 && j < m && row < nI && act) ? r[(int64_t)gI[row] * K + lane] : 0.0;
             }
         };
-        auto wait_slot = [&](int s) -> bool {
+        auto wait_unit = [&](int u) -> bool {
+            const int s = u % NS;
             const bool w = __all_sync(0xffffffffu, mbar_wait(&bars[s], (ph >> s) & 1u));
             ph ^= 1u << s;
             pend &= ~(1u << s);
             return w;
-        };
-        auto refill = [&](int s, int blk) {   // after __syncwarp: every lane is done with slot s
-            if (lane == 0) {
-                mbar_expect(&bars[s], slot_bytes);
-                bulk_copy(ring + (size_t)s * 2 * BB, F + (size_t)blk * 2 * BB, slot_bytes, &bars[s]);
-            }
-            pend |= 1u << s;
         };
 
         // forward sweep: y_j = Linv_j (b_j - L_{j,j-1} y_{j-1})
@@ -609,22 +622,21 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
         auto fstep = [&](int j, double (&d)[BP]) -> bool {
 #pragma unroll
             for (int q = 0; q < BP; ++q) bsm[q * 32 + lane] = from_f64<ACC>(d[q]);
-            load_rows(d, j + 2);
+            load_rows(d, j + AH);
             if (POST) {
                 const int e1 = bst[j + 1];
                 for (int e = bst[j]; e < e1; ++e) {
                     const int k = srt[e], pr = gP[k];
-                    bsm[((pr & 0xffff) - j * BP) * 32 + lane] -= cvs[2 * k] * vG[(pr >> 16) * 32 + lane];
+                    bsm[((pr & 0xffff) - j * BP) * 32 + lane] -= cvs[CS * k] * vG[(pr >> 16) * 32 + lane];
                 }
             }
             ACC t[BP];
 #pragma unroll
             for (int q = 0; q < BP; ++q) t[q] = bsm[q * 32 + lane];
-            const int s = j % kLSRing;
-            if (!wait_slot(s)) return false;
-            const T *Li = ring + (size_t)s * 2 * BB;
-            const T *Ls = Li + BB;
+            if (!HALF && !wait_unit(j)) return false;
             if (j > 0) {
+                if (HALF && !wait_unit(2 * j - 1)) return false;
+                const T *Ls = HALF ? unit(2 * j - 1) : unit(j) + BB;
 #pragma unroll
                 for (int c = 0; c < BP; ++c) {
                     ACC col[BP];
@@ -633,7 +645,13 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                     for (int q = 0; q < BP; ++q)
                         if (!TRI || q <= c) t[q] -= col[q ^ c] * xp[c];
                 }
+                if (HALF) {
+                    __syncwarp();
+                    if (2 * j - 1 + NS < nu) refill(2 * j - 1 + NS);
+                }
             }
+            if (HALF && !wait_unit(2 * j)) return false;
+            const T *Li = unit(HALF ? 2 * j : j);
 #pragma unroll
             for (int q = 0; q < BP; ++q) xp[q] = 0;
 #pragma unroll
@@ -646,16 +664,21 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
 #pragma unroll
             for (int q = 0; q < BP; ++q) ys[(j * BP + q) * 32 + lane] = xp[q];
             __syncwarp();
-            if (j + kLSRing < m) refill(s, j + kLSRing);
+            if (const int u = (HALF ? 2 * j : j) + NS; u < nu) refill(u);
             return true;
         };
         {
-            double da[BP], db[BP];
+            double da[BP];
             load_rows(da, 0);
-            load_rows(db, 1);
-            for (int j = 0; j < m && ok; j += 2) {
-                ok = fstep(j, da);
-                if (ok && j + 1 < m) ok = fstep(j + 1, db);
+            if constexpr (AH == 2) {
+                double db[BP];
+                load_rows(db, 1);
+                for (int j = 0; j < m && ok; j += 2) {
+                    ok = fstep(j, da);
+                    if (ok && j + 1 < m) ok = fstep(j + 1, db);
+                }
+            } else {
+                for (int j = 0; j < m && ok; ++j) ok = fstep(j, da);
             }
         }
 
@@ -680,19 +703,24 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                 ACC t[BP];
 #pragma unroll
                 for (int q = 0; q < BP; ++q) t[q] = y[q];
-                load_y(y, j - 2);
-                const int s = j % kLSRing;
-                if (j < m - kLSRing && !wait_slot(s)) return false;
+                load_y(y, j - AH);
+                if (!HALF && j < nu - NS && !wait_unit(j)) return false;
                 if (j < m - 1) {
-                    const T *Ls1 = ring + (size_t)((j + 1) % kLSRing) * 2 * BB + BB;
+                    if (HALF && 2 * j + 1 < nu - NS && !wait_unit(2 * j + 1)) return false;
+                    const T *Ls1 = HALF ? unit(2 * j + 1) : unit(j + 1) + BB;
 #pragma unroll
                     for (int c = 0; c < BP; ++c) {
                         ACC col[BP];
                         load_vec<T, ACC, BP>(Ls1 + c * BP, col);
                         t[c] -= dot4(col, zn, c, 0, TRI ? c + 1 : BP);
                     }
+                    if (HALF) {
+                        __syncwarp();
+                        if (2 * j + 1 >= NS) refill(2 * j + 1 - NS);
+                    }
                 }
-                const T *Li = ring + (size_t)s * 2 * BB;
+                if (HALF && 2 * j < nu - NS && !wait_unit(2 * j)) return false;
+                const T *Li = unit(HALF ? 2 * j : j);
 #pragma unroll
                 for (int c = 0; c < BP; ++c) {
                     ACC col[BP];
@@ -712,26 +740,35 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
                     const int e1 = bst[j + 1];
                     for (int e = bst[j]; e < e1; ++e) {
                         const int k = srt[e], pr = gP[k];
-                        vG[(pr >> 16) * 32 + lane] += cvs[2 * k] * bsm[((pr & 0xffff) - j * BP) * 32 + lane];
+                        vG[(pr >> 16) * 32 + lane] += cvs[CS * k] * bsm[((pr & 0xffff) - j * BP) * 32 + lane];
                     }
                 }
                 __syncwarp();
-                if (j <= m - 2 && j + 1 - kLSRing >= 0) refill((j + 1) % kLSRing, j + 1 - kLSRing);
+                if (HALF) {
+                    if (2 * j >= NS) refill(2 * j - NS);
+                } else if (j <= m - 2 && j + 1 >= NS) {
+                    refill(j + 1 - NS);
+                }
                 return true;
             };
-            ACC ya[BP], yb[BP];
+            ACC ya[BP];
             load_y(ya, m - 1);
-            load_y(yb, m - 2);
-            for (int j = m - 1; j >= 0 && ok; j -= 2) {
-                ok = bstep(j, ya);
-                if (ok && j - 1 >= 0) ok = bstep(j - 1, yb);
+            if constexpr (AH == 2) {
+                ACC yb[BP];
+                load_y(yb, m - 2);
+                for (int j = m - 1; j >= 0 && ok; j -= 2) {
+                    ok = bstep(j, ya);
+                    if (ok && j - 1 >= 0) ok = bstep(j - 1, yb);
+                }
+            } else {
+                for (int j = m - 1; j >= 0 && ok; --j) ok = bstep(j, ya);
             }
         }
         if (ok && POST && rz.sc && act) {
             // r.z over the interior entries just written (read back by the
             // lane that wrote them), in four partial sums
             double a4[4] = {0.0, 0.0, 0.0, 0.0};
-            constexpr int RU = ls_rows(BP) / 2 * (BP == 8 ? 1 : 2);
+            constexpr int RU = BP == 8 ? 8 : ls_rows<ACC>(BP);
             for (int i0 = 0; i0 < nI; i0 += RU) {
                 double rv[RU], zv[RU];
 #pragma unroll
@@ -774,9 +811,9 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
     }
     if (live && !ok) {
         if (lane == 0) atomicExch(L.err, 1);
-        for (int s = 0; s < kLSRing; ++s)   // bounded: copies in flight land before the warp exits
+        for (int s = 0; s < NS; ++s)   // bounded: copies in flight land before the warp exits
             if ((pend >> s) & 1u) mbar_wait(&bars[s], (ph >> s) & 1u);
-        mbar_wait(&bars[kLSRing], 0);
+        mbar_wait(&bars[NS], 0);
     }
     if (POST && rz.sc) {
         // per-block partials (the warps' in a fixed order), summed over the
@@ -785,8 +822,7 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
         __syncthreads();
         if (warp == 0) {
             double t = 0.0;
-#pragma unroll
-            for (int w = 0; w < kLSW; ++w) t += red[w * 32 + lane];
+            for (int w = 0; w < nwb; ++w) t += red[w * 32 + lane];
             if (act) rz.part[(int64_t)blockIdx.x * K + lane] = t;
             __threadfence();
         }
@@ -797,22 +833,22 @@ __global__ void __launch_bounds__(32 * kLSW, ls_blocks(BP)) k_dir_ls(DevLevel L,
         __threadfence();
         double t = 0.0;
         if (act) {
+            constexpr int PU = 16;
             int sb = warp;
-            for (; sb + 7 * kLSW < (int)gridDim.x; sb += 8 * kLSW) {
-                double v[8];
+            for (; sb + (PU - 1) * nwb < (int)gridDim.x; sb += PU * nwb) {
+                double v[PU];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = __ldcg(&rz.part[(int64_t)(sb + u * kLSW) * K + lane]);
+                for (int u = 0; u < PU; ++u) v[u] = __ldcg(&rz.part[(int64_t)(sb + u * nwb) * K + lane]);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) t += v[u];
+                for (int u = 0; u < PU; ++u) t += v[u];
             }
-            for (; sb < (int)gridDim.x; sb += kLSW) t += __ldcg(&rz.part[(int64_t)sb * K + lane]);
+            for (; sb < (int)gridDim.x; sb += nwb) t += __ldcg(&rz.part[(int64_t)sb * K + lane]);
         }
         red[warp * 32 + lane] = t;
         __syncthreads();
         if (warp == 0 && act) {
             double tot = 0.0;
-#pragma unroll
-            for (int w = 0; w < kLSW; ++w) tot += red[w * 32 + lane];
+            for (int w = 0; w < nwb; ++w) tot += red[w * 32 + lane];
             BatchScalars *sc = rz.sc;
             if (!sc->done[lane]) {
                 const double beta = sc->fresh[lane] ? 0.0 : tot / sc->rho[lane];
@@ -2284,31 +2320,37 @@ void dir_b(const DevLevel &L, const BatchLevel &B, bool post, const double *r, d
     else dir_b_launch<T, ACC, 32>(L, B, post, r, z, skip, s, rz);
 }
 
-// The lane-per-right-hand-side kernel (k_dir_ls) takes FP32 accumulation and
-// uniform blocks of 8 or 16 rows.
+// The lane-per-right-hand-side kernel (k_dir_ls) takes uniform blocks of 8 or
+// 16 rows.
+template <class T, class ACC> size_t lane_total(const DevLevel &L, int w) {
+    return L.bp == 8 ? LaneSmem<T, ACC, 8>::of(L, w).total : LaneSmem<T, ACC, 16>::of(L, w).total;
+}
+// Warps of a block: one wave of blocks, up to the most that the kernel and
+// the shared memory take.
+template <class T, class ACC> int lane_warps(const DevLevel &L) {
+    const int most = L.bp == 8 ? ls_max_warps<ACC, 8>() : ls_max_warps<ACC, 16>();
+    int w = std::min(most, std::max(1, (L.nsub + num_sms_b() - 1) / num_sms_b()));
+    while (w > 1 && lane_total<T, ACC>(L, w) > kSmemMaxB) --w;
+    return w;
+}
 template <class T, class ACC> size_t lane_smem(const DevLevel &L) {
-    if (!std::is_same<ACC, float>::value || !(L.bp == 8 || L.bp == 16) || !L.irec) return 0;
+    if (!(L.bp == 8 || L.bp == 16) || !L.irec) return 0;
     if (L.max_m + 1 > 32 * L.bp) return 0;   // the sort's block counts live in the block buffer
-    return L.bp == 8 ? LaneSmem<T, 8>::of(L).total : LaneSmem<T, 16>::of(L).total;
+    return lane_total<T, ACC>(L, lane_warps<T, ACC>(L));
 }
 
 template <class T, class ACC>
 void dir_ls(const DevLevel &L, const BatchLevel &B, bool post, const double *r, double *z, const int *skip,
             cudaStream_t s, const RzBatch *rz = nullptr) {
-    if constexpr (std::is_same<ACC, float>::value) {
-        if (!B.ys) throw Error(BDDC_E_STATE, "lane Dirichlet kernel without its scratch");
-        const RzBatch none{nullptr, nullptr, nullptr, nullptr};
-        const RzBatch rzv = (post && rz) ? *rz : none;
-        const size_t sm = lane_smem<T, ACC>(L);
-        const int grid = (L.nsub + kLSW - 1) / kLSW;
-        const auto k8 = L.sub_tri ? (post ? k_dir_ls<T, 8, true, true> : k_dir_ls<T, 8, false, true>)
-                                  : (post ? k_dir_ls<T, 8, true, false> : k_dir_ls<T, 8, false, false>);
-        const auto k16 = L.sub_tri ? (post ? k_dir_ls<T, 16, true, true> : k_dir_ls<T, 16, false, true>)
-                                   : (post ? k_dir_ls<T, 16, true, false> : k_dir_ls<T, 16, false, false>);
-        launch_plain(L.bp == 8 ? k8 : k16, grid, 32 * kLSW, sm, s, L, B, r, z, skip, rzv);
-    } else {
-        throw Error(BDDC_E_STATE, "lane Dirichlet kernel in FP64");
-    }
+    if (!B.ys) throw Error(BDDC_E_STATE, "lane Dirichlet kernel without its scratch");
+    const RzBatch none{nullptr, nullptr, nullptr, nullptr};
+    const RzBatch rzv = (post && rz) ? *rz : none;
+    const int W = lane_warps<T, ACC>(L);
+    const auto k8 = L.sub_tri ? (post ? k_dir_ls<T, ACC, 8, true, true> : k_dir_ls<T, ACC, 8, false, true>)
+                              : (post ? k_dir_ls<T, ACC, 8, true, false> : k_dir_ls<T, ACC, 8, false, false>);
+    const auto k16 = L.sub_tri ? (post ? k_dir_ls<T, ACC, 16, true, true> : k_dir_ls<T, ACC, 16, false, true>)
+                               : (post ? k_dir_ls<T, ACC, 16, true, false> : k_dir_ls<T, ACC, 16, false, false>);
+    launch_plain(L.bp == 8 ? k8 : k16, (L.nsub + W - 1) / W, 32 * W, lane_smem<T, ACC>(L), s, L, B, r, z, skip, rzv);
 }
 
 template <class T, class ACC>
@@ -2443,7 +2485,7 @@ bool batch_path(const DevLevel &L, int prec) { return route(L, prec).ok; }
 
 bool batch_lane(const DevLevel &L) {
     auto fits = [](size_t b) { return b > 0 && b <= kSmemMaxB; };
-    return fits(lane_smem<float, float>(L)) || fits(lane_smem<__nv_bfloat16, float>(L));
+    return fits(lane_smem<float, float>(L)) || fits(lane_smem<__nv_bfloat16, float>(L)) || fits(lane_smem<double, double>(L));
 }
 
 bool batch_streams(const DevLevel &L) {
@@ -2544,13 +2586,20 @@ void dir_bs(const DevLevel &L, const BatchLevel &B, bool post, const double *r, 
     }
 }
 
+// In FP64 the lane kernel pays for 32 right-hand sides whatever K is, the
+// streaming kernel for each 16 (a warp's column groups): 512^2 problem, both
+// corrections, 974 us streaming at 16 and 1628 at 17, 1175 with a lane each.
+template <class ACC> bool lane_wide(const BatchRoute &R, const BatchLevel &B) {
+    return sizeof(ACC) == 4 || B.K > 16 || !R.stream_fits;
+}
+
 template <class T, class ACC>
 void pre_b(const DevLevel &L, const BatchLevel &B, int prec, const double *r, const int *skip, cudaStream_t s,
            cudaEvent_t *ev) {
     const BatchRoute R = route_t<T, ACC>(L, prec);
     if (ev) cudaEventRecord(ev[0], s);
     if (R.pre_tc) tc_dir_b(L, B, prec, false, r, nullptr, skip, nullptr, s);
-    else if (R.dir_lane) dir_ls<T, ACC>(L, B, false, r, nullptr, skip, s);
+    else if (R.dir_lane && lane_wide<ACC>(R, B)) dir_ls<T, ACC>(L, B, false, r, nullptr, skip, s);
     else if (R.dir_staged) dir_b<T, ACC>(L, B, false, r, nullptr, skip, s);
     else dir_bs<T, ACC>(L, B, false, r, nullptr, skip, nullptr, s);
     if (ev) cudaEventRecord(ev[1], s);
@@ -2568,7 +2617,7 @@ void post_b(const DevLevel &L, const BatchLevel &B, int prec, const double *r, d
     else avg_bg<T, ACC>(L, B, prec, skip, s);
     if (ev) cudaEventRecord(ev[1], s);
     if (R.post_tc) tc_dir_b(L, B, prec, true, r, z, skip, rz, s);
-    else if (R.dir_lane) dir_ls<T, ACC>(L, B, true, r, z, skip, s, rz);
+    else if (R.dir_lane && lane_wide<ACC>(R, B)) dir_ls<T, ACC>(L, B, true, r, z, skip, s, rz);
     else if (R.dir_staged) dir_b<T, ACC>(L, B, true, r, z, skip, s, rz);
     else dir_bs<T, ACC>(L, B, true, r, z, skip, rz, s);
     if (ev) cudaEventRecord(ev[2], s);
@@ -2711,12 +2760,14 @@ void prepare_batch_kernels() {
 #define BDDC_DIR_B(T, A, BPV)                                   \
     BDDC_SMEM_ATTR_B((k_dir_b<T, A, BPV, false>));              \
     BDDC_SMEM_ATTR_B((k_dir_b<T, A, BPV, true>));
-#define BDDC_DIR_LS(T, BPV)                                     \
-    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, false, false>));         \
-    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, true, false>));          \
-    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, false, true>));          \
-    BDDC_SMEM_ATTR_B((k_dir_ls<T, BPV, true, true>));
-    BDDC_DIR_LS(float, 8) BDDC_DIR_LS(float, 16) BDDC_DIR_LS(__nv_bfloat16, 8) BDDC_DIR_LS(__nv_bfloat16, 16)
+#define BDDC_DIR_LS(T, ACC, BPV)                                     \
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, ACC, BPV, false, false>));         \
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, ACC, BPV, true, false>));          \
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, ACC, BPV, false, true>));          \
+    BDDC_SMEM_ATTR_B((k_dir_ls<T, ACC, BPV, true, true>));
+    BDDC_DIR_LS(double, double, 8) BDDC_DIR_LS(double, double, 16)
+    BDDC_DIR_LS(float, float, 8) BDDC_DIR_LS(float, float, 16)
+    BDDC_DIR_LS(__nv_bfloat16, float, 8) BDDC_DIR_LS(__nv_bfloat16, float, 16)
 #undef BDDC_DIR_LS
     BDDC_DIR_B(double, double, 8) BDDC_DIR_B(double, double, 16) BDDC_DIR_B(double, double, 32)
     BDDC_DIR_B(float, float, 8) BDDC_DIR_B(float, float, 16) BDDC_DIR_B(float, float, 32)

@@ -326,7 +326,7 @@ struct RzBatch {
 // Whether a level's operators fit the batched kernels' shared-memory slices.
 bool batch_path(const DevLevel &L, int prec);
 bool batch_streams(const DevLevel &L);   // some precision can take the streaming Dirichlet kernel
-bool batch_lane(const DevLevel &L);      // FP32 / BF16 can take the lane-per-right-hand-side Dirichlet kernel
+bool batch_lane(const DevLevel &L);      // some precision can take the lane-per-right-hand-side Dirichlet kernel
 void batch_prepare_level(const DevLevel &L);   // launch shapes of the streaming kernel, before any capture
 // Autotuning of one level's batch kernels on the problem's own operators
 // (CUDA events, three launches after one untimed): for every precision,
