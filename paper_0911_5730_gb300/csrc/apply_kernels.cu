@@ -1763,9 +1763,9 @@ void avg_launch(const DevLevel &L, int prec, const int *skip, cudaStream_t s) {
 // Interiors beyond the records of warp_path in FP32 / BF16 with a power-of-two
 // block size: the warp Dirichlet kernel in class 3 where there are warps for
 // every SM and a wave of them fits; the block-per-substructure kernels
-// (k_dir_s) otherwise.  576 elasticity substructures of 450 interior
-// DOFs: 28 + 24 us, where the block-per-substructure kernels took 40 + 35; a handful of substructures runs
-// faster with a block each.
+// (k_dir_s) otherwise.  576 elasticity substructures of 450 interior DOFs:
+// 28 + 24 us, where the block-per-substructure kernels took 40 + 35; a handful
+// of substructures runs faster with a block each.
 bool warp_dir_large(const DevLevel &L, int prec) {
     if (prec == BDDC_PREC_FP64 || force_generic_dir()) return false;
     if (!(L.bp == 8 || L.bp == 16 || L.bp == 32) || !L.irec || dir_class(L) != 3 || L.max_m * L.bp > 65535) return false;

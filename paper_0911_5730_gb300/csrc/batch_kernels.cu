@@ -2703,13 +2703,19 @@ void tune_route_t(DevLevel &L, BatchLevel &B, int prec, const double *r, double 
     }
 }
 
-template <class T, class ACC> void tune_t(const DevLevel &L, BatchLevel &B, int prec, const double *r, cudaStream_t s) {
+template <class T, class ACC> void tune_t(const DevLevel &L, BatchLevel &B, int prec, const double *r, double *z,
+                                       cudaStream_t s) {
     const BatchRoute R = route_t<T, ACC>(L, prec);
-    if (R.dir_stream && !R.pre_tc && L.bk.n > 1 && B.fork && B.ys) {
+    // The streaming kernel's buckets, for the correction that takes it (FP32
+    // levels with a tensor-core pre-correction stream the post-correction only;
+    // sixteen large level-2 substructures in three buckets: 318 us one after
+    // another, 128 the longest).
+    const bool bs_pre = R.dir_stream && !R.pre_tc, bs_post = R.dir_stream && !R.post_tc;
+    if ((bs_pre || bs_post) && L.bk.n > 1 && B.fork && B.ys) {
         double t[2];
         for (int par = 0; par < 2; ++par) {
             B.bucket_par = par;
-            t[par] = time3(s, [&] { dir_bs<T, ACC>(L, B, false, r, nullptr, nullptr, nullptr, s); });
+            t[par] = time3(s, [&] { dir_bs<T, ACC>(L, B, !bs_pre, r, z, nullptr, nullptr, s); });
         }
         B.bucket_par = t[1] < t[0] ? 1 : 0;
         if (const char *e = std::getenv("BDDC_BUCKETS")) {   // "serial" or "parallel"
@@ -2741,9 +2747,9 @@ void tune_level_b(DevLevel &L, BatchLevel &B, int prec, const double *r, double 
     tune_route_t<double, double>(L, B, BDDC_PREC_FP64, r, z, s);
     tune_route_t<float, float>(L, B, BDDC_PREC_FP32, r, z, s);
     tune_route_t<__nv_bfloat16, float>(L, B, BDDC_PREC_BF16, r, z, s);
-    if (prec == BDDC_PREC_FP64) tune_t<double, double>(L, B, prec, r, s);
-    else if (prec == BDDC_PREC_FP32) tune_t<float, float>(L, B, prec, r, s);
-    else tune_t<__nv_bfloat16, float>(L, B, prec, r, s);
+    if (prec == BDDC_PREC_FP64) tune_t<double, double>(L, B, prec, r, z, s);
+    else if (prec == BDDC_PREC_FP32) tune_t<float, float>(L, B, prec, r, z, s);
+    else tune_t<__nv_bfloat16, float>(L, B, prec, r, z, s);
     BDDC_CUDA_TRY(cudaStreamSynchronize(s));
 }
 
