@@ -2664,10 +2664,16 @@ void tune_route_t(DevLevel &L, BatchLevel &B, int prec, const double *r, double 
         L.route_pref &= ~(sbit | lbit);
         const BatchRoute R0 = route_t<T, ACC>(L, prec);
         if (R0.dir_staged && !(R0.pre_tc && R0.post_tc)) {
-            int cand[3] = {0, 0, 0}, nc = 1;
-            if (R0.lane_fits && B.ys) cand[nc++] = lbit;
+            // (FP64 with a substructure for every SM: the staged kernel takes
+            // 1200 us a sweep of 1024 substructures, a lane each 450, and is not
+            // timed beside it, which keeps the first use of a problem as short
+            // as without the lane kernel)
+            int cand[3] = {0, 0, 0}, nc = 0;
+            const bool lane = R0.lane_fits && B.ys;
+            if (!(prec == BDDC_PREC_FP64 && lane && L.nsub >= num_sms_b())) cand[nc++] = 0;
+            if (lane) cand[nc++] = lbit;
             if (R0.stream_fits && B.ys) cand[nc++] = sbit;
-            int pick = 0;
+            int pick = forced ? 0 : cand[0];
             if (forced) {
                 if (forced[0] == 's' && forced[1] == 't' && forced[2] == 'r' && R0.stream_fits && B.ys) pick = sbit;
             } else if (nc > 1) {
