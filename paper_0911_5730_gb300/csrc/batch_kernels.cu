@@ -14,6 +14,7 @@
 // converged keeps its state while the others iterate.
 #include "internal.h"
 #include "device_util.cuh"
+#include "rules.h"
 
 #include <algorithm>
 #include <cstdlib>
@@ -976,7 +977,7 @@ __device__ __forceinline__ void prod(ACC (&a)[R][4], const T *M, int ldm, const 
 template <class T, class ACC, bool SUB, bool COL, bool SWZ, bool LOW, int R, int SEG = 0>
 __device__ __forceinline__ void prod_tri(ACC (&a)[R][4], const T *M, int ldm, const ACC *v, int h, int b, int d,
                                          const int (&rw)[R], int c0 = 0) {
-    const int e = SEG + 1 == R ? b : LOW ? min(b, (SEG + 1) * h + d) : max(0, (SEG + 1) * h - d);
+    const int e = tri_segment_end(SEG, R, h, b, d, LOW);
     prod<T, ACC, SUB, COL, SWZ, LOW ? SEG : 0, LOW ? R : SEG + 1, R>(a, M, ldm, v, c0, e, rw);
     if constexpr (SEG + 1 < R) prod_tri<T, ACC, SUB, COL, SWZ, LOW, R, SEG + 1>(a, M, ldm, v, h, b, d, rw, e);
 }

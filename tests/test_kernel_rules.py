@@ -1,0 +1,50 @@
+"""The kernels' rules of sizes (csrc/rules.h), compiled by the host compiler
+and checked over their whole range; no GPU."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_0911_5730_gb300", "csrc")
+
+
+@pytest.fixture
+def run(tmp_path):
+    def go(body, flags=()):
+        """Compiles a program around `body` (statements that return the number
+        of the first rule broken, 0 if none) and returns that number."""
+        src, exe = tmp_path / "t.cpp", tmp_path / "t"
+        src.write_text(body)
+        subprocess.run(["g++", "-std=c++17", "-O1", "-I" + CSRC, *flags, str(src), "-o", str(exe)], check=True)
+        p = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+        assert p.returncode == 0, p.stdout + p.stderr
+    return go
+
+
+def test_triangle_segments(run):
+    """Products with a triangle of zeros, for every block size and offset: the
+    segments stay within the block, follow one another, and every entry that
+    may be nonzero lies in a segment that serves its row."""
+    run(r"""
+#include <cstdio>
+#include <initializer_list>
+#include "rules.h"
+int main() {
+    for (int R : {2, 4}) for (int b = 1; b <= 160; ++b) for (int d = 0; d <= b; ++d) for (int low = 0; low < 2; ++low) {
+        const int h = (b + R - 1) / R;
+        int from = 0, end[4];
+        for (int s = 0; s < R; ++s) {
+            end[s] = bddc::tri_segment_end(s, R, h, b, d, low);
+            if (end[s] < from || end[s] > b) { printf("R %d b %d d %d low %d: segment %d [%d, %d)\n", R, b, d, low, s, from, end[s]); return 1; }
+            from = end[s];
+        }
+        if (end[R - 1] != b) return 2;
+        for (int r = 0; r < b; ++r) for (int c = 0; c < b; ++c) {
+            if (low ? c > r + d : c < r - d) continue;
+            int s = 0;
+            while (c >= end[s]) ++s;
+            if (low ? r / h < s : r / h > s) { printf("R %d b %d d %d low %d: (%d, %d) left out\n", R, b, d, low, r, c); return 3; }
+        }
+    }
+}
+""")
