@@ -136,8 +136,8 @@ typedef struct {
     int32_t n_interface[3];       /* interface DOFs of the level (each counted once) */
     /* tile shapes the autotuner chose for the batch kernels of this context
      * (timed on the context's own operators when its batch workspace is first
-     * used): node tile of the batched PCG stencil (x, y; batches of more than
-     * 24 columns march instead) and rows per block of
+     * used): node tile of the batched PCG stencil (x, y; timed at 24 columns,
+     * the widest batch that takes a tile: wider ones march) and rows per block of
      * the top-level product with the dense inverse, or 0 when the batched top
      * solve uses the block-tridiagonal factor (top_blocks); 0 before the first
      * batched call */

@@ -1920,7 +1920,8 @@ __global__ void __launch_bounds__(kTT) k_b_init(int n, int K, const double *b, i
 
 // First half of a batched PCG iteration: p_new = z + beta p_old, q = A p_new
 // and alpha_k = rho_k / (p_new . q).  A block owns a BT_X x BT_Y tile of nodes
-// (the tile shape is chosen per problem by the autotuner, dir_spmv_tune)
+// (the tile shape is chosen per problem by the autotuner, dir_spmv_tune, at the
+// widest K that takes a tile)
 // for all K right-hand sides; p_new is formed once per entry of the tile and
 // its halo in shared memory (the FP64 pipe is the limit), from p_old in one
 // direction buffer, and written to the other.
@@ -2018,7 +2019,7 @@ __global__ void k_b_dir_spmv(int nx, int K, const double *__restrict__ w, const 
 // no predicates, and their order is the tile kernel's: q is the same bit for
 // bit.  32 right-hand sides: the 1024^2 three-level solve (46 iterations)
 // 101 -> 92 ms (the kernel 856 -> 652 us), the 512^2 FP64 solve 75.6 -> 72.5 ms.
-constexpr int MW = 8, kMarchT = 256, kMarchPerSm = 2, kMarchMinK = 24;
+constexpr int MW = 8, kMarchT = 256, kMarchPerSm = 2;
 __global__ void __launch_bounds__(kMarchT, kMarchPerSm)
 k_b_dir_march(int nx, int K, const double *__restrict__ w, const double *__restrict__ z, double *p0, double *p1,
               double *__restrict__ q, double *part, unsigned *counter, BatchScalars *sc, double *alphas, int strips,
@@ -2940,15 +2941,9 @@ void dir_spmv_v(int nx, int K, const double *w, const double *z, double *p0, dou
     launch_plain(k_b_dir_spmv<TX, TY>, tile_blocks<TX, TY>(nx), bblock(K), bt_smem(TX, TY, K), s, nx, K, w, z,
                  p0, p1, q, part, counter, sc, alphas);
 }
-void launch_b_dir_spmv(int nx, int K, const double *w, const double *z, double *p0, double *p1,
-                       double *q, double *part, unsigned *counter, BatchScalars *sc, double *alphas,
-                       cudaStream_t s, int variant) {
-    if (K > kMarchMinK && variant >= 0) {
-        const MarchShape m = march_shape(nx);
-        launch_plain(k_b_dir_march, m.blocks, kMarchT, 0, s, nx, K, w, z, p0, p1, q, part, counter, sc, alphas,
-                     m.strips, m.rows);
-        return;
-    }
+void launch_b_dir_tile(int nx, int K, const double *w, const double *z, double *p0, double *p1, double *q,
+                       double *part, unsigned *counter, BatchScalars *sc, double *alphas, cudaStream_t s,
+                       int variant) {
     switch (variant) {
     case 1: dir_spmv_v<32, 4>(nx, K, w, z, p0, p1, q, part, counter, sc, alphas, s); break;
     case 2: dir_spmv_v<32, 8>(nx, K, w, z, p0, p1, q, part, counter, sc, alphas, s); break;
@@ -2956,8 +2951,20 @@ void launch_b_dir_spmv(int nx, int K, const double *w, const double *z, double *
     default: dir_spmv_v<16, 8>(nx, K, w, z, p0, p1, q, part, counter, sc, alphas, s);
     }
 }
-int dir_spmv_tune(int nx, int K, const double *w, const double *z, double *p0, double *p1, double *q,
-                  double *part, unsigned *counter, BatchScalars *sc, double *alphas, cudaStream_t s) {
+void launch_b_dir_spmv(int nx, int K, const double *w, const double *z, double *p0, double *p1,
+                       double *q, double *part, unsigned *counter, BatchScalars *sc, double *alphas,
+                       cudaStream_t s, int variant) {
+    if (!stencil_marches(K)) {
+        launch_b_dir_tile(nx, K, w, z, p0, p1, q, part, counter, sc, alphas, s, variant);
+        return;
+    }
+    const MarchShape m = march_shape(nx);
+    launch_plain(k_b_dir_march, m.blocks, kMarchT, 0, s, nx, K, w, z, p0, p1, q, part, counter, sc, alphas,
+                 m.strips, m.rows);
+}
+int dir_spmv_tune(int nx, const double *w, const double *z, double *p0, double *p1, double *q, double *part,
+                  unsigned *counter, BatchScalars *sc, double *alphas, cudaStream_t s) {
+    static_assert(!stencil_marches(kTileTuneK), "the tiles are timed at a width that takes one");
     if (const char *e = std::getenv("BDDC_TILE_VARIANT")) {   // 0..3: this tile, no timing
         const int v = std::atoi(e);
         if (v >= 0 && v < kNTiles) return v;
@@ -2966,7 +2973,7 @@ int dir_spmv_tune(int nx, int K, const double *w, const double *z, double *p0, d
     float tb = 1e30f;
     for (int v = 0; v < kNTiles; ++v) {
         const float t = time_launches(
-            [&] { launch_b_dir_spmv(nx, K, w, z, p0, p1, q, part, counter, sc, alphas, s, v); }, 3, s);
+            [&] { launch_b_dir_tile(nx, kTileTuneK, w, z, p0, p1, q, part, counter, sc, alphas, s, v); }, 3, s);
         if (t < tb) { tb = t; best = v; }
     }
     return best;

@@ -1280,8 +1280,8 @@ BatchWs &batch_ws(bddc_ctx *C, Workspace &W) {
         if (C->tile_v < 0) {
             // (the elasticity operator has no tile to choose)
             C->tile_v = elastic(C) ? 0
-                                   : dir_spmv_tune(C->nx, KB, C->w_dev, bw->z, bw->p, bw->p1, bw->q, bw->part,
-                                                   bw->counter, scs, al, st);
+                                   : dir_spmv_tune(C->nx, C->w_dev, bw->z, bw->p, bw->p1, bw->q, bw->part, bw->counter,
+                                                   scs, al, st);
             const BatchLevel &top = bw->lv.back();
             C->gemm_v = C->Ainv ? gemm_tune(C->n_top, C->ld_top, C->Ainv, top.rcv, top.ucv, KB, W.err, st) : -1;
             if (C->Ainv && C->band) {

@@ -367,13 +367,14 @@ void launch_b_init(int n, int K, const double *b, int64_t ldb, double *x, double
 // between p0 and p1 by sc->step), q = A p_new, alpha = rho / (p_new . q).
 // part must hold launch_b_dir_spmv_blocks(nx) * K doubles.
 int launch_b_dir_spmv_blocks(int nx);
-// variant: node tile 16x8, 32x4, 32x8 or 8x16 (0..3), chosen by dir_spmv_tune
-// (which runs every variant on scratch scalars, directions and q).
+// variant: node tile 16x8, 32x4, 32x8 or 8x16 (0..3) of batches that do not
+// march (stencil_marches), chosen by dir_spmv_tune (which runs every tile on
+// scratch scalars, directions and q at the width kTileTuneK).
 void launch_b_dir_spmv(int nx, int K, const double *w, const double *z, double *p0, double *p1,
                        double *q, double *part, unsigned *counter, BatchScalars *sc, double *alphas,
                        cudaStream_t s, int variant = 0);
-int dir_spmv_tune(int nx, int K, const double *w, const double *z, double *p0, double *p1, double *q,
-                  double *part, unsigned *counter, BatchScalars *sc, double *alphas, cudaStream_t s);
+int dir_spmv_tune(int nx, const double *w, const double *z, double *p0, double *p1, double *q, double *part,
+                  unsigned *counter, BatchScalars *sc, double *alphas, cudaStream_t s);
 void dir_spmv_tile(int variant, int *tx, int *ty);
 // x += alpha p_new; r -= alpha q; rr; convergence; step += 1
 void launch_b_update(int n, int K, double *x, double *r, const double *p0, const double *p1,

@@ -21,4 +21,9 @@ BDDC_HD constexpr int tri_segment_end(int seg, int R, int h, int b, int d, bool 
     return e < 0 ? 0 : e > b ? b : e;
 }
 
+// The batched stencil: up to kMarchMinK right-hand sides take a node tile, whose
+// shape is timed at that width, the widest one that uses it; more march.
+constexpr int kMarchMinK = 24, kTileTuneK = kMarchMinK;
+BDDC_HD constexpr bool stencil_marches(int K) { return K > kMarchMinK; }
+
 }  // namespace bddc

@@ -48,3 +48,12 @@ int main() {
     }
 }
 """)
+
+
+def test_stencil_tile_is_timed_where_it_runs(run):
+    """The width at which the stencil's tiles are timed takes a tile, and no
+    wider one does."""
+    run(r"""
+#include "rules.h"
+int main() { return bddc::stencil_marches(bddc::kTileTuneK) ? 1 : !bddc::stencil_marches(bddc::kTileTuneK + 1) ? 2 : 0; }
+""")
