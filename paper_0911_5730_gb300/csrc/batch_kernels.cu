@@ -2588,11 +2588,9 @@ void dir_bs(const DevLevel &L, const BatchLevel &B, bool post, const double *r, 
     }
 }
 
-// In FP64 the lane kernel pays for 32 right-hand sides whatever K is, the
-// streaming kernel for each 16 (a warp's column groups): 512^2 problem, both
-// corrections, 974 us streaming at 16 and 1628 at 17, 1175 with a lane each.
-template <class ACC> bool lane_wide(const BatchRoute &R, const BatchLevel &B) {
-    return sizeof(ACC) == 4 || B.K > 16 || !R.stream_fits;
+// Whether a level whose route is the lane kernel uses it for this batch.
+template <class ACC> bool lane_wide(const DevLevel &L, const BatchRoute &R, const BatchLevel &B) {
+    return sizeof(ACC) == 4 || fp64_lane_at(B.K, L.bp, L.nsub, num_sms_b(), R.stream_fits);
 }
 
 template <class T, class ACC>
@@ -2601,7 +2599,7 @@ void pre_b(const DevLevel &L, const BatchLevel &B, int prec, const double *r, co
     const BatchRoute R = route_t<T, ACC>(L, prec);
     if (ev) cudaEventRecord(ev[0], s);
     if (R.pre_tc) tc_dir_b(L, B, prec, false, r, nullptr, skip, nullptr, s);
-    else if (R.dir_lane && lane_wide<ACC>(R, B)) dir_ls<T, ACC>(L, B, false, r, nullptr, skip, s);
+    else if (R.dir_lane && lane_wide<ACC>(L, R, B)) dir_ls<T, ACC>(L, B, false, r, nullptr, skip, s);
     else if (R.dir_staged) dir_b<T, ACC>(L, B, false, r, nullptr, skip, s);
     else dir_bs<T, ACC>(L, B, false, r, nullptr, skip, nullptr, s);
     if (ev) cudaEventRecord(ev[1], s);
@@ -2619,7 +2617,7 @@ void post_b(const DevLevel &L, const BatchLevel &B, int prec, const double *r, d
     else avg_bg<T, ACC>(L, B, prec, skip, s);
     if (ev) cudaEventRecord(ev[1], s);
     if (R.post_tc) tc_dir_b(L, B, prec, true, r, z, skip, rz, s);
-    else if (R.dir_lane && lane_wide<ACC>(R, B)) dir_ls<T, ACC>(L, B, true, r, z, skip, s, rz);
+    else if (R.dir_lane && lane_wide<ACC>(L, R, B)) dir_ls<T, ACC>(L, B, true, r, z, skip, s, rz);
     else if (R.dir_staged) dir_b<T, ACC>(L, B, true, r, z, skip, s, rz);
     else dir_bs<T, ACC>(L, B, true, r, z, skip, rz, s);
     if (ev) cudaEventRecord(ev[2], s);
@@ -2666,18 +2664,14 @@ void tune_route_t(DevLevel &L, BatchLevel &B, int prec, const double *r, double 
         L.route_pref &= ~(sbit | lbit);
         const BatchRoute R0 = route_t<T, ACC>(L, prec);
         if (R0.dir_staged && !(R0.pre_tc && R0.post_tc)) {
-            // (FP64 with a substructure for every SM: the staged kernel takes
-            // 1200 us a sweep of 1024 substructures, a lane each 450, and is not
-            // timed beside it, which keeps the first use of a problem as short
-            // as without the lane kernel)
             int cand[3] = {0, 0, 0}, nc = 0;
-            const bool lane = R0.lane_fits && B.ys;
-            if (!(prec == BDDC_PREC_FP64 && lane && L.nsub >= num_sms_b())) cand[nc++] = 0;
+            const bool lane = R0.lane_fits && B.ys, stream = R0.stream_fits && B.ys;
+            if (prec != BDDC_PREC_FP64 || !lane || fp64_staged_timed(L.bp, L.nsub, num_sms_b(), stream)) cand[nc++] = 0;
             if (lane) cand[nc++] = lbit;
-            if (R0.stream_fits && B.ys) cand[nc++] = sbit;
+            if (stream) cand[nc++] = sbit;
             int pick = forced ? 0 : cand[0];
             if (forced) {
-                if (forced[0] == 's' && forced[1] == 't' && forced[2] == 'r' && R0.stream_fits && B.ys) pick = sbit;
+                if (forced[0] == 's' && forced[1] == 't' && forced[2] == 'r' && stream) pick = sbit;
             } else if (nc > 1) {
                 double best = 1e30;
                 for (int i = 0; i < nc; ++i) {

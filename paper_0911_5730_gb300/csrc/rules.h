@@ -26,4 +26,29 @@ BDDC_HD constexpr int tri_segment_end(int seg, int R, int h, int b, int d, bool 
 constexpr int kMarchMinK = 24, kTileTuneK = kMarchMinK;
 BDDC_HD constexpr bool stencil_marches(int K) { return K > kMarchMinK; }
 
+// The FP64 batch Dirichlet kernels on levels of uniform blocks of bp rows where
+// the lane-per-right-hand-side kernel fits; us for both corrections (m = 15
+// blocks of 16 rows, 7 of 8 rows; 152 SMs; the streaming kernel and the staged
+// one take the same within 5 % for fewer columns unless given):
+//   blocks of 16 rows        169 subs.  256   576   1024
+//     staged                       678   684  1373   2396
+//     streaming, 17 to 32          544   556   848   1456
+//     streaming, up to 16          543   545   596    809
+//     lane                         755   758   776   1175
+//   blocks of 8 rows         169 subs.  256  1024   4096  16384
+//     staged                        95    98   307   1017   3986
+//     streaming                    177   180   223    761   2664
+//     lane                         136   136   216    677   2526
+// Whether the staged kernel is timed beside the others: not where it lost
+// wherever it was measured, which keeps the first use of a large problem short.
+BDDC_HD constexpr bool fp64_staged_timed(int bp, int nsub, int sms, bool stream) {
+    return bp == 16 ? !(stream && nsub >= sms) : nsub < 6 * sms;
+}
+// Whether K columns take the lane kernel where it was the fastest for 32: it
+// costs the same for any K, and so does the streaming kernel with blocks of 8
+// rows; with blocks of 16 rows that one is the faster up to 16 columns.
+BDDC_HD constexpr bool fp64_lane_at(int K, int bp, int nsub, int sms, bool stream) {
+    return K > 16 || !(bp == 16 && nsub >= sms && stream);
+}
+
 }  // namespace bddc
