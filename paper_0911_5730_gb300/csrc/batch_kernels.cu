@@ -2158,6 +2158,7 @@ __global__ void k_b_update(int64_t nK, int K, double *__restrict__ x, double *__
             if (sc->done[kk] || sc->hold[kk]) return;
             sc->rr[kk] = tot;
             sc->it[kk] += 1;
+            sc->last[kk] = sc->step;
             if (tot <= sc->tol2[kk]) { sc->conv[kk] = 1; sc->done[kk] = 1; }
             if (sc->it[kk] >= sc->mx[kk]) sc->done[kk] = 1;
         },
@@ -2252,6 +2253,11 @@ __global__ void k_b_admit(int n, int K, int k, const double *__restrict__ b, dou
 __global__ void k_b_column(int n, int K, int k, const double *x, double *dst) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g < n) dst[g] = x[(int64_t)g * K + k];
+}
+
+__global__ void k_b_move_column(int n, int K, int k, const double *src, double *dst) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < n) dst[(int64_t)g * K + k] = src[(int64_t)g * K + k];
 }
 
 // Both integer-operation conversions against the hardware ones, bit for bit
@@ -3000,6 +3006,9 @@ void launch_b_admit(int n, int K, int k, const double *b, double *x, double *r, 
 }
 void launch_b_column(int n, int K, int k, const double *x, double *dst, cudaStream_t s) {
     if (n > 0) k_b_column<<<(n + 255) / 256, 256, 0, s>>>(n, K, k, x, dst);
+}
+void launch_b_move_column(int n, int K, int k, const double *src, double *dst, cudaStream_t s) {
+    if (n > 0) k_b_move_column<<<(n + 255) / 256, 256, 0, s>>>(n, K, k, src, dst);
 }
 void launch_selftest_convert(const double *d, int64_t n, unsigned long long *bad, cudaStream_t s) {
     if (n > 0) k_selftest_convert<<<(int)((n + 255) / 256), 256, 0, s>>>(d, n, bad);

@@ -1,6 +1,7 @@
 // bddc_api.cu - setup orchestration, the apply recursion, the PCG driver and
 // the C entry points of libbddc.so.
 #include "internal.h"
+#include "rules.h"
 #include "partition.h"
 
 #include <algorithm>
@@ -1347,6 +1348,14 @@ void set_batch_width(BatchWs &BW, int K) {
     for (auto &B : BW.lv) B.K = K;
 }
 
+// Column k resumes after steps that it sat out: its direction, written at step
+// last[k], to the buffer that the next step with it (`next`) reads.
+void resume_direction(BatchWs &BW, int n, int K, int k, int next, cudaStream_t st) {
+    const int from = direction_written(BW.hsc->last[k]), to = direction_read(next);
+    double *const p[2] = {BW.p, BW.p1};
+    if (from != to) launch_b_move_column(n, K, k, p[from], p[to], st);
+}
+
 cudaGraphExec_t batch_graph(bddc_ctx *C, Workspace &W, BatchWs &BW, int prec, int K) {
     const int key = prec * 64 + K;
     auto it = BW.graphs.find(key);
@@ -1412,6 +1421,7 @@ int pcg_batch(bddc_ctx *C, Workspace &W, int prec, const double *b, int64_t ldb,
                 // from the same iterate, residual and direction (the apply
                 // below gives its z, rho and beta; the others stay done)
                 h.done[k] = 0; h.conv[k] = 0;
+                resume_direction(BW, n, K, k, h.step, st);
                 again = true;
             }
         }
@@ -2680,6 +2690,7 @@ void engine_loop(bddc_server *S, Engine *E) {
                     // keeps iterating from the same state: it sits out the next
                     // direction update and rejoins at that iteration's apply
                     h.done[k] = 0; h.conv[k] = 0; h.hold[k] = 1;
+                    resume_direction(BW, n, K, k, h.step + 1, st);
                     resume = true;
                 } else {
                     out.push_back(k);

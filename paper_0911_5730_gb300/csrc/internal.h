@@ -312,6 +312,7 @@ struct BatchScalars {
     // out the next direction/update half and joins at that iteration's apply
     int hold[kMaxBatch];
     int mx[kMaxBatch];     // iteration limit of each right-hand side
+    int last[kMaxBatch];   // the step that wrote its latest direction
     int K, maxit, all_done;
     int step;      // lockstep iterations run (selects the direction buffer)
 };
@@ -379,6 +380,8 @@ void dir_spmv_tile(int variant, int *tx, int *ty);
 // x += alpha p_new; r -= alpha q; rr; convergence; step += 1
 void launch_b_update(int n, int K, double *x, double *r, const double *p0, const double *p1,
                      const double *q, double *part, unsigned *counter, BatchScalars *sc, cudaStream_t s);
+// p of column k from buffer src to buffer dst ([n][K] each)
+void launch_b_move_column(int n, int K, int k, const double *src, double *dst, cudaStream_t s);
 void launch_b_residual(int nx, int K, const double *w, const double *b, int64_t ldb, const double *x,
                        double *res, cudaStream_t s);
 void launch_b_norm2(int n, int K, const double *v, double *part, unsigned *counter, double *out,

@@ -51,4 +51,10 @@ BDDC_HD constexpr bool fp64_lane_at(int K, int bp, int nsub, int sms, bool strea
     return K > 16 || !(bp == 16 && nsub >= sms && stream);
 }
 
+// The two direction buffers of a batch: lockstep step `step` reads one and
+// writes the other, for the columns that iterate.  A column that sat out steps
+// may find its latest direction in the one that its next step would write.
+BDDC_HD constexpr int direction_read(int step) { return step & 1; }
+BDDC_HD constexpr int direction_written(int step) { return 1 - (step & 1); }
+
 }  // namespace bddc

@@ -79,3 +79,27 @@ int main() {
     }
 }
 """)
+
+
+def test_direction_buffers_of_a_resumed_column(run):
+    """A column that stops at a step, sits out any number of steps and resumes
+    finds the direction that it wrote last."""
+    run(r"""
+#include "rules.h"
+using namespace bddc;
+int main() {
+    for (int stop = 0; stop < 8; ++stop) for (int missed = 0; missed < 8; ++missed) {
+        int buf[2] = {-1, -2}, last = -1, step = 0;
+        for (; step <= stop; ++step) {
+            if (step > 0 && buf[direction_read(step)] != last) return 1;
+            last = step;
+            buf[direction_written(step)] = step;
+        }
+        step += missed;
+        const int from = direction_written(last), to = direction_read(step);
+        if (from != to) buf[to] = buf[from];
+        if (buf[direction_read(step)] != stop) return 2;
+        if (direction_read(step) == direction_written(step)) return 3;
+    }
+}
+""")
