@@ -2669,7 +2669,7 @@ void engine_loop(bddc_server *S, Engine *E) {
                 const Request &R = *slot[k].R;
                 BDDC_CUDA_TRY(cudaMemcpyAsync(BW.bcol + (size_t)k * n, R.b.data() + (size_t)slot[k].j * n,
                                               sizeof(double) * n, cudaMemcpyHostToDevice, st));
-                launch_b_admit(n, K, k, BW.bcol + (size_t)k * n, BW.x, BW.r, BW.part, BW.counter, BW.sc,
+                launch_b_admit(n, K, k, BW.bcol + (size_t)k * n, BW.x, BW.r, BW.p, BW.p1, BW.part, BW.counter, BW.sc,
                                R.rtol, std::min(R.maxit, W->maxit_cap), st);
             }
             cudaGraphExec_t g = batch_graph(C, *W, BW, E->prec, K);
