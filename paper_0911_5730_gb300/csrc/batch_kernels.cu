@@ -1330,21 +1330,21 @@ template <class T, class ACC> __host__ inline size_t neu_bg_smem(const DevLevel 
 
 template <class T, class ACC, int RT>
 __global__ void __launch_bounds__(32 * kNBW, RT == 1 ? 4 : 3) k_neu_bg(DevLevel L, BatchLevel B, int pidx, const double *r,
-                                                      const int *skip) {
+                                                      const int *skip, int chunk) {
     extern __shared__ __align__(16) unsigned char smem_ng[];
     if (skip && *skip) return;
     const int sub = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
     const int K = B.K;
     const bool act = lane < K;
     const int nG = L.nG[sub], nc = L.ncl[sub];
-    const NeuSmem ly = NeuSmem::of<T, ACC>(L, B.chunk);
+    const NeuSmem ly = NeuSmem::of<T, ACC>(L, chunk);
     const NRecLayout lay(nG, nc, (int)sizeof(T));
     unsigned char *head = smem_ng;
     ACC *f = reinterpret_cast<ACC *>(smem_ng + ly.head);
     unsigned char *ring = smem_ng + ly.head + ly.f;
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem_ng + ly.total - 32);   // stages, head
     const unsigned char *rec = L.nrec[pidx] + L.nrecOff[pidx][sub];
-    const int ldn = lay.ld, CH = neu_chunk_rows<T>(nG, B.chunk);
+    const int ldn = lay.ld, CH = neu_chunk_rows<T>(nG, chunk);
     const int ntile = ldn >> 3, nch = nG > 0 ? (nG + CH - 1) / CH : 0;
     // N streams once per pass of nw * RT tiles; step s is chunk s % nch of pass s / nch
     const int npass = (ntile + nw * RT - 1) / (nw * RT), nstep = npass * nch;
@@ -2392,14 +2392,22 @@ int neu_warps(const DevLevel &L) {
     const int t = (L.max_nG + 7) / 8;
     return t < 1 ? 1 : (t > kNBW ? kNBW : t);
 }
+// The chunk of a launch: the one asked for (tuned, in the context's precision
+// then) where the level fits with it in this precision, else the largest of
+// 32, 16 and 8 KB that fits; 0: none does.
+template <class T, class ACC> __host__ inline int neu_chunk(const DevLevel &L, int asked) {
+    for (int c : {asked, kChunkBytes, kChunkBytes / 2, kChunkBytes / 4})
+        if (c > 0 && neu_bg_smem<T, ACC>(L, c) <= kSmemMaxB) return c;
+    return 0;
+}
 template <class T, class ACC>
 void neu_bg(const DevLevel &L, const BatchLevel &B, int prec, const double *r, const int *skip, cudaStream_t s) {
     const int nw = neu_warps(L), rt = ((L.max_nG + 7) / 8 + nw - 1) / nw;
-    const size_t sm = neu_bg_smem<T, ACC>(L, B.chunk);
-    const int pi = pidx_b(prec);
-    if (rt <= 1) launch_plain(k_neu_bg<T, ACC, 1>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip);
-    else if (rt == 2 || sizeof(ACC) == 8) launch_plain(k_neu_bg<T, ACC, 2>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip);
-    else launch_plain(k_neu_bg<T, ACC, 3>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip);
+    const int chunk = neu_chunk<T, ACC>(L, B.chunk), pi = pidx_b(prec);
+    const size_t sm = neu_bg_smem<T, ACC>(L, chunk);
+    if (rt <= 1) launch_plain(k_neu_bg<T, ACC, 1>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip, chunk);
+    else if (rt == 2 || sizeof(ACC) == 8) launch_plain(k_neu_bg<T, ACC, 2>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip, chunk);
+    else launch_plain(k_neu_bg<T, ACC, 3>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip, chunk);
 }
 template <class T, class ACC>
 void avg_bg(const DevLevel &L, const BatchLevel &B, int prec, const int *skip, cudaStream_t s) {
@@ -2463,7 +2471,7 @@ template <class T, class ACC> BatchRoute route_t(const DevLevel &L, int prec) {
     const int nw_max = ((L.max_b + 1) / 2 + 3) / 4;
     const bool stream = L.bk.n > 0 && L.bperm && nw_max <= kMaxBuckets &&
                         StreamSmemB::of<T, ACC>(L, 32 * nw_max).total <= kSmemMaxB;
-    const bool bg = neu_bg_smem<T, ACC>(L) <= kSmemMaxB && avg_bg_smem<T, ACC>(L) <= kSmemMaxB;
+    const bool bg = neu_chunk<T, ACC>(L, 0) > 0 && avg_bg_smem<T, ACC>(L) <= kSmemMaxB;
     R.dir_stream = !R.dir_staged && stream;
     R.stream_fits = stream;
     R.bg_fits = bg;
@@ -2734,7 +2742,7 @@ template <class T, class ACC> void tune_t(const DevLevel &L, BatchLevel &B, int 
             if (e[0] == 'p') B.bucket_par = 1;
         }
     }
-    if (!R.neu_staged && neu_bg_smem<T, ACC>(L) <= kSmemMaxB) {
+    if (!R.neu_staged) {
         const int cand[3] = {16 * 1024, 32 * 1024, 64 * 1024};
         double best = 1e30;
         int pick = 0;
