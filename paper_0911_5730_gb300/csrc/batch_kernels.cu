@@ -1310,11 +1310,11 @@ template <class T> __host__ __device__ inline int neu_chunk_rows(int nG, int chu
 }
 struct NeuSmem {
     size_t head, f, stage, total;
-    template <class T, class ACC> __host__ __device__ static NeuSmem of(const DevLevel &L, int chunk) {
+    template <class T, class ACC> __host__ __device__ static NeuSmem of(const DevLevel &L, int chunk, bool head = true) {
         NeuSmem m;
         const size_t mg = L.max_nG > 0 ? L.max_nG : 1, mc = L.max_nc > 0 ? L.max_nc : 1;
         const size_t row = sizeof(T) * ((mg + 7) & ~size_t(7));
-        m.head = (size_t)NRecLayout((int)mg, (int)mc, (int)sizeof(T)).N;
+        m.head = head ? (size_t)NRecLayout((int)mg, (int)mc, (int)sizeof(T)).N : 0;
         m.f = al16(sizeof(ACC) * ((mg + 7) & ~size_t(7)) * 32);
         const size_t cb = chunk > 0 ? (size_t)chunk : (size_t)kChunkBytes;
         // one stage when the whole operator fits in it and one pass covers its rows, else two
@@ -1324,11 +1324,14 @@ struct NeuSmem {
         return m;
     }
 };
-template <class T, class ACC> __host__ inline size_t neu_bg_smem(const DevLevel &L, int chunk_bytes = 0) {
-    return NeuSmem::of<T, ACC>(L, chunk_bytes).total;
+template <class T, class ACC> __host__ inline size_t neu_bg_smem(const DevLevel &L, int chunk_bytes, bool head = true) {
+    return NeuSmem::of<T, ACC>(L, chunk_bytes, head).total;
 }
 
-template <class T, class ACC, int RT>
+// HEAD: the record ahead of N is staged; else it is read where it lies (levels
+// whose Psi leaves no room for N's stages: FP64 interfaces of 512 DOFs with 19
+// coarse ones or more).
+template <class T, class ACC, int RT, bool HEAD>
 __global__ void __launch_bounds__(32 * kNBW, RT == 1 ? 4 : 3) k_neu_bg(DevLevel L, BatchLevel B, int pidx, const double *r,
                                                       const int *skip, int chunk) {
     extern __shared__ __align__(16) unsigned char smem_ng[];
@@ -1337,13 +1340,13 @@ __global__ void __launch_bounds__(32 * kNBW, RT == 1 ? 4 : 3) k_neu_bg(DevLevel 
     const int K = B.K;
     const bool act = lane < K;
     const int nG = L.nG[sub], nc = L.ncl[sub];
-    const NeuSmem ly = NeuSmem::of<T, ACC>(L, chunk);
+    const NeuSmem ly = NeuSmem::of<T, ACC>(L, chunk, HEAD);
     const NRecLayout lay(nG, nc, (int)sizeof(T));
-    unsigned char *head = smem_ng;
+    const unsigned char *rec = L.nrec[pidx] + L.nrecOff[pidx][sub];
+    const unsigned char *head = HEAD ? smem_ng : rec;
     ACC *f = reinterpret_cast<ACC *>(smem_ng + ly.head);
     unsigned char *ring = smem_ng + ly.head + ly.f;
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem_ng + ly.total - 32);   // stages, head
-    const unsigned char *rec = L.nrec[pidx] + L.nrecOff[pidx][sub];
     const int ldn = lay.ld, CH = neu_chunk_rows<T>(nG, chunk);
     const int ntile = ldn >> 3, nch = nG > 0 ? (nG + CH - 1) / CH : 0;
     // N streams once per pass of nw * RT tiles; step s is chunk s % nch of pass s / nch
@@ -1355,11 +1358,11 @@ __global__ void __launch_bounds__(32 * kNBW, RT == 1 ? 4 : 3) k_neu_bg(DevLevel 
     };
     if (tid == 0) {
         for (int s = 0; s < 3; ++s) mbar_init(&bars[s]);
-        if (lay.N > 0) bulk_load(head, rec, (unsigned)lay.N, &bars[2]);
+        if (HEAD && lay.N > 0) bulk_load(smem_ng, rec, (unsigned)lay.N, &bars[2]);
         for (int s = 0; s < 2 && s < nstep; ++s) issue(s);
     }
     __syncthreads();
-    bool ok = lay.N == 0 || mbar_wait(&bars[2], 0);
+    bool ok = !HEAD || lay.N == 0 || mbar_wait(&bars[2], 0);
     int waited = 0;                          // steps waited for
     if (__syncthreads_and(ok)) {
         const T *Ps = reinterpret_cast<const T *>(head + lay.psi);
@@ -1446,7 +1449,7 @@ __global__ void __launch_bounds__(32 * kNBW, RT == 1 ? 4 : 3) k_neu_bg(DevLevel 
     // a wait gave up: flag it, and let the copies in flight land (bounded)
     if (tid == 0) {
         atomicExch(L.err, 1);
-        if (lay.N > 0) mbar_wait(&bars[2], 0);
+        if (HEAD && lay.N > 0) mbar_wait(&bars[2], 0);
         const int s0 = waited > 0 ? waited - 1 : 0;          // in flight: the step that failed and the next
         for (int s = s0; s < s0 + 2 && s < nstep; ++s) mbar_wait(&bars[s & 1], (unsigned)(s >> 1) & 1u);
     }
@@ -2392,22 +2395,27 @@ int neu_warps(const DevLevel &L) {
     const int t = (L.max_nG + 7) / 8;
     return t < 1 ? 1 : (t > kNBW ? kNBW : t);
 }
-// The chunk of a launch: the one asked for (tuned, in the context's precision
+// The form of a launch: the chunk asked for (tuned, in the context's precision
 // then) where the level fits with it in this precision, else the largest of
-// 32, 16 and 8 KB that fits; 0: none does.
-template <class T, class ACC> __host__ inline int neu_chunk(const DevLevel &L, int asked) {
-    for (int c : {asked, kChunkBytes, kChunkBytes / 2, kChunkBytes / 4})
-        if (c > 0 && neu_bg_smem<T, ACC>(L, c) <= kSmemMaxB) return c;
-    return 0;
+// 32, 16 and 8 KB that fits, with the record staged if possible; chunk 0: none.
+struct NeuForm { int chunk; bool head; };
+template <class T, class ACC> NeuForm neu_form(const DevLevel &L, int asked) {
+    for (bool head : {true, false})
+        for (int c : {head ? asked : 0, kChunkBytes, kChunkBytes / 2, kChunkBytes / 4})
+            if (c > 0 && neu_bg_smem<T, ACC>(L, c, head) <= kSmemMaxB) return {c, head};
+    return {0, false};
 }
 template <class T, class ACC>
 void neu_bg(const DevLevel &L, const BatchLevel &B, int prec, const double *r, const int *skip, cudaStream_t s) {
     const int nw = neu_warps(L), rt = ((L.max_nG + 7) / 8 + nw - 1) / nw;
-    const int chunk = neu_chunk<T, ACC>(L, B.chunk), pi = pidx_b(prec);
-    const size_t sm = neu_bg_smem<T, ACC>(L, chunk);
-    if (rt <= 1) launch_plain(k_neu_bg<T, ACC, 1>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip, chunk);
-    else if (rt == 2 || sizeof(ACC) == 8) launch_plain(k_neu_bg<T, ACC, 2>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip, chunk);
-    else launch_plain(k_neu_bg<T, ACC, 3>, L.nsub, 32 * nw, sm, s, L, B, pi, r, skip, chunk);
+    const NeuForm F = neu_form<T, ACC>(L, B.chunk);
+    // without the staged record, interfaces that need all tiles of a warp only
+    constexpr int most = sizeof(ACC) == 8 ? 2 : 3;
+    const auto kern = !F.head                     ? k_neu_bg<T, ACC, most, false>
+                      : rt <= 1                   ? k_neu_bg<T, ACC, 1, true>
+                      : rt == 2 || most == 2      ? k_neu_bg<T, ACC, 2, true>
+                                                  : k_neu_bg<T, ACC, 3, true>;
+    launch_plain(kern, L.nsub, 32 * nw, neu_bg_smem<T, ACC>(L, F.chunk, F.head), s, L, B, pidx_b(prec), r, skip, F.chunk);
 }
 template <class T, class ACC>
 void avg_bg(const DevLevel &L, const BatchLevel &B, int prec, const int *skip, cudaStream_t s) {
@@ -2471,7 +2479,7 @@ template <class T, class ACC> BatchRoute route_t(const DevLevel &L, int prec) {
     const int nw_max = ((L.max_b + 1) / 2 + 3) / 4;
     const bool stream = L.bk.n > 0 && L.bperm && nw_max <= kMaxBuckets &&
                         StreamSmemB::of<T, ACC>(L, 32 * nw_max).total <= kSmemMaxB;
-    const bool bg = neu_chunk<T, ACC>(L, 0) > 0 && avg_bg_smem<T, ACC>(L) <= kSmemMaxB;
+    const bool bg = neu_form<T, ACC>(L, 0).chunk > 0 && avg_bg_smem<T, ACC>(L) <= kSmemMaxB;
     R.dir_stream = !R.dir_staged && stream;
     R.stream_fits = stream;
     R.bg_fits = bg;
@@ -2823,9 +2831,10 @@ void prepare_batch_kernels() {
 #undef BDDC_DIR_BS_SMALL
 #undef BDDC_DIR_BS
 #define BDDC_NEU_BG(T, A)                                       \
-    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 1>));                      \
-    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 2>));                      \
-    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 3>));
+    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 1, true>));                \
+    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 2, true>));                \
+    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, 3, true>));                \
+    BDDC_SMEM_ATTR_B((k_neu_bg<T, A, sizeof(A) == 8 ? 2 : 3, false>));
     BDDC_NEU_BG(double, double) BDDC_NEU_BG(float, float) BDDC_NEU_BG(__nv_bfloat16, float)
 #undef BDDC_NEU_BG
     BDDC_SMEM_ATTR_B((k_avg_bg<double, double>)); BDDC_SMEM_ATTR_B((k_avg_bg<float, float>));

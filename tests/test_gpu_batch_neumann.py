@@ -77,3 +77,15 @@ def test_small_chunk(lib):
         _check(P, wl, "fp64", 1e-10)
     finally:
         P.close()
+
+
+@pytest.mark.parametrize("per_side,prec,tol", [(6, "fp64", 1e-10), (19, "fp32", 1e-5)])
+def test_record_not_staged(lib, per_side, prec, tol):
+    """502 DOFs with 22 (FP64) and 74 (FP32) coarse ones: the record leaves no
+    room for the smallest chunks."""
+    wl = _flanked(252, per_side)
+    P = lib.Problem.from_workload(wl)
+    try:
+        _check(P, wl, prec, tol)
+    finally:
+        P.close()
