@@ -26,6 +26,7 @@
 //    A_II^{-1} (r_I - A_{I Gamma} u_B,Gamma) and its interface is u_B.
 #include "internal.h"
 #include "device_util.cuh"
+#include "rules.h"
 
 namespace bddc {
 
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, 
     const int ldb = fld(b, swz);
     const size_t bsq = (size_t)b * ldb;
     const int ns = 2 * m - 1;
-    unsigned par = 0, pend = 0;           // bit q: parity of slot q's next phase; a copy in flight (thread 0)
+    RingSlots slots;                      // copies in flight: thread 0's
     bool ok = true;
     // half s (2 j: Linv_j, 2 j - 1: Lsub_j): its bytes rounded out to 16-byte
     // boundaries, and where it starts in its slot
@@ -210,19 +211,14 @@ __global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, 
         const uintptr_t ae = (a + bsq * sizeof(T) + 15) & ~uintptr_t(15);
         mbar_expect(&bars[q], (unsigned)(ae - al));
         bulk_copy(smem_s + (size_t)q * ly.stage, reinterpret_cast<const void *>(al), (unsigned)(ae - al), &bars[q]);
-        pend |= 1u << q;
+        slots.issued(q);
     };
     auto slot = [&](int s) {
         const uintptr_t a = reinterpret_cast<uintptr_t>(half_of(s));
         return reinterpret_cast<const T *>(smem_s + (size_t)(s % ring) * ly.stage + (a & 15));
     };
     auto wait_half = [&](int s) {         // every thread sees the copy's completion itself
-        const int q = s % ring;
-        if (ok) {
-            ok = mbar_wait(&bars[q], (par >> q) & 1u);
-            if (ok) pend &= ~(1u << q);
-        }
-        par ^= 1u << q;
+        ok = ok && slots.wait(s % ring, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
     };
     if (tid == 0) {
         for (int q = 0; q < ring; ++q) mbar_init(&bars[q]);
@@ -306,9 +302,8 @@ __global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, 
     }
     if (!__syncthreads_and(ok)) {
         if (tid == 0) {
-            atomicExch(L.err, 1);
-            for (int q = 0; q < ring; ++q)                // bounded: copies in flight land first
-                if ((pend >> q) & 1u) mbar_wait(&bars[q], (par >> q) & 1u);
+            atomicExch(L.err, 1);                         // bounded: copies in flight land first
+            slots.drain(ring, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
         }
         return;
     }

@@ -610,7 +610,7 @@ k_dir_ls(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
         };
         auto wait_unit = [&](int u) -> bool {
             const int s = u % NS;
-            const bool w = __all_sync(0xffffffffu, mbar_wait(&bars[s], (ph >> s) & 1u));
+            const bool w = warp_wait_copy(&bars[s], nullptr, lane, (ph >> s) & 1u);   // waits twice for a late copy
             ph ^= 1u << s;
             pend &= ~(1u << s);
             return w;
@@ -1003,7 +1003,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
     if (tid == 0)
         for (int s2 = 0; s2 < SBN; ++s2) mbar_init(&bars[s2]);
     __syncthreads();
-    unsigned par = 0, pend = 0;           // bit s: parity of slot s's next phase; a copy in flight (thread 0)
+    RingSlots slots;                      // copies in flight: thread 0's
     bool ok = true;                       // false once a wait of this thread gave up: it waits no more
     for (int ti = blockIdx.x; ti < count; ti += gridDim.x) {
         const int sub = perm[ti];
@@ -1035,19 +1035,14 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
             mbar_expect(&bars[s % SBN], (unsigned)(ae - al));
             bulk_copy(ring + (size_t)(s % SBN) * ly.stage, reinterpret_cast<const void *>(al),
                       (unsigned)(ae - al), &bars[s % SBN]);
-            pend |= 1u << (s % SBN);
+            slots.issued(s % SBN);
         };
         auto slot = [&](int s) {
             const uintptr_t a = reinterpret_cast<uintptr_t>(half_of(s));
             return reinterpret_cast<const T *>(ring + (size_t)(s % SBN) * ly.stage + (a & 15));
         };
         auto wait_half = [&](int s) {     // every thread sees the copy's completion itself
-            const int q = s % SBN;
-            if (ok) {
-                ok = mbar_wait(&bars[q], (par >> q) & 1u);
-                if (ok) pend &= ~(1u << q);
-            }
-            par ^= 1u << q;
+            ok = ok && slots.wait(s % SBN, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
         };
         if (tid == 0 && ok)
             for (int s = 0; s < SBN && s < ns; ++s) issue(s);
@@ -1284,8 +1279,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
     }
     if (!ok) atomicExch(L.err, 1);
     if (tid == 0)                         // bounded: copies in flight land before the block exits
-        for (int s2 = 0; s2 < SBN; ++s2)
-            if ((pend >> s2) & 1u) mbar_wait(&bars[s2], (par >> s2) & 1u);
+        slots.drain(SBN, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
 }
 
 // (6)-(9) for K right-hand sides, a block of up to kNBW warps per

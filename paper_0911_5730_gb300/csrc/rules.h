@@ -57,4 +57,27 @@ BDDC_HD constexpr bool fp64_lane_at(int K, int bp, int nsub, int sms, bool strea
 BDDC_HD constexpr int direction_read(int step) { return step & 1; }
 BDDC_HD constexpr int direction_written(int step) { return 1 - (step & 1); }
 
+// One thread's view of a ring of shared-memory slots filled by bulk copies, a
+// barrier each (barrier s completes once per copy into slot s, with alternating
+// parity).  wait_for(s, parity) polls barrier s a bounded number of times.  A
+// thread whose wait gave up (false) waits and issues no more: the slot still
+// counts as in flight.
+struct RingSlots {
+    unsigned parity = 0;    // bit s: parity of the next completion of slot s
+    unsigned pending = 0;   // bit s: a copy that this thread issued is in flight
+
+    BDDC_HD void issued(int s) { pending |= 1u << s; }
+    template <class F> BDDC_HD bool wait(int s, F &&wait_for) {
+        if (!wait_for(s, (parity >> s) & 1u)) return false;
+        parity ^= 1u << s;
+        pending &= ~(1u << s);
+        return true;
+    }
+    // before the block exits: the copies in flight land
+    template <class F> BDDC_HD void drain(int slots, F &&wait_for) const {
+        for (int s = 0; s < slots; ++s)
+            if ((pending >> s) & 1u) wait_for(s, (parity >> s) & 1u);
+    }
+};
+
 }  // namespace bddc
