@@ -8,6 +8,7 @@
 // constraint rows of eq. (14), and the constrained Neumann operator with the
 // coarse basis (Sec. 2.1).  The dense top-level factorization closes the file.
 #include "internal.h"
+#include "rules.h"
 
 #include <cmath>
 
@@ -54,12 +55,14 @@ __device__ bool cta_cholesky(double *A, int n, int lda) {
 }
 
 // The same for a matrix that may be semidefinite to rounding: a pivot that is
-// not positive gives a zero column.
-__device__ void cta_cholesky_semi(double *A, int n, int lda) {
+// not above the rounding of its diagonal entry (d0[n]: scratch for those) gives
+// a zero column.
+__device__ void cta_cholesky_semi(double *A, int n, int lda, double *d0) {
+    for (int j = threadIdx.x; j < n; j += blockDim.x) d0[j] = A[(int64_t)j * lda + j];
     for (int j = 0; j < n; ++j) {
         __syncthreads();
         const double d = A[(int64_t)j * lda + j];
-        const double l = d > 0.0 ? sqrt(d) : 0.0;
+        const double l = semi_pivot(d, d0[j], n) ? sqrt(d) : 0.0;
         __syncthreads();
         if (threadIdx.x == 0) A[(int64_t)j * lda + j] = l;
         for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x)
@@ -614,7 +617,7 @@ __global__ void __launch_bounds__(128) k_edge_eig(SetupLevel S, EdgeBatch E, dou
         Wk[q] = sum;
     }
     __syncthreads();
-    cta_cholesky_semi(Wk, ne, ne);
+    cta_cholesky_semi(Wk, ne, ne, lamv);
     for (int q = threadIdx.x; q < ne * ne; q += blockDim.x) {  // P = Xd Lg
         const int i = q / ne, j = q % ne;
         double sum = 0.0;

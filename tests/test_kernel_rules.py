@@ -138,3 +138,50 @@ int main() {
     }
 }
 """)
+
+
+def test_semidefinite_pivots(run):
+    """Cholesky factors of Gram matrices of half rank: L L^T is the matrix up to
+    n dropped pivots, each worth the root of its threshold."""
+    run(r"""
+#include <cmath>
+#include <cstdio>
+#include <random>
+#include <vector>
+#include "rules.h"
+int main() {
+    for (int n : {8, 16, 31}) {
+        const int r = n / 2;
+        std::mt19937_64 gen(1);
+        for (int t = 0; t < 20000; ++t) {
+            std::vector<double> B(n * r), G(n * n), A;
+            for (auto &v : B) v = (double)(gen() >> 11) * 0x1p-52 - 1.0;
+            double mx = 0.0;
+            for (int i = 0; i < n; ++i)
+                for (int j = 0; j < n; ++j) {
+                    double s = 0.0;
+                    for (int k = 0; k < r; ++k) s += B[i * r + k] * B[j * r + k];
+                    G[i * n + j] = s;
+                    if (i == j) mx = std::max(mx, s);
+                }
+            A = G;
+            for (int j = 0; j < n; ++j) {
+                const double d = A[j * n + j], l = bddc::semi_pivot(d, G[j * n + j], n) ? std::sqrt(d) : 0.0;
+                A[j * n + j] = l;
+                for (int i = j + 1; i < n; ++i) A[i * n + j] = l > 0.0 ? A[i * n + j] / l : 0.0;
+                for (int i = j + 1; i < n; ++i)
+                    for (int k = j + 1; k <= i; ++k) A[i * n + k] -= A[i * n + j] * A[k * n + j];
+            }
+            for (int i = 0; i < n; ++i)
+                for (int j = 0; j <= i; ++j) {
+                    double s = 0.0;
+                    for (int k = 0; k <= j; ++k) s += A[i * n + k] * A[j * n + k];
+                    if (!(std::fabs(s - G[i * n + j]) <= n * std::sqrt(n * 0x1p-52) * mx)) {
+                        printf("n %d matrix %d: off by %g of %g\n", n, t, s - G[i * n + j], mx);
+                        return 1;
+                    }
+                }
+        }
+    }
+}
+""", ["-O2"])
