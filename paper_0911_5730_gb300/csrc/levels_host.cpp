@@ -5,18 +5,14 @@
 // interior ordering with its block structure, and the flattened per-
 // substructure index maps uploaded to the device.  No floating-point work of
 // the method happens here.
+#include "for_each_sub.h"
 #include "levels_host.h"
 
 #include <algorithm>
-#include <atomic>
-#include <exception>
 #include <map>
-#include <mutex>
 #include <numeric>
 #include <queue>
 #include <stdexcept>
-#include <system_error>
-#include <thread>
 
 namespace bddc {
 
@@ -34,39 +30,6 @@ struct DSU {
         if (a != b) { if (a < b) p[b] = a; else p[a] = b; }
     }
 };
-
-// f(s) for every substructure s < n, shared out to the host's cores (the calls
-// touch disjoint data); few substructures stay on the calling thread.  The
-// first exception is rethrown after all threads have stopped.  (The orderings
-// of the 512^2 channel problem's 1024 substructures were 55 of the 130 ms of
-// its setup and solve.)
-template <class F> void for_each_sub(int n, F &&f) {
-    constexpr int kChunk = 16, kMostThreads = 16;
-    std::atomic<int> next{0};
-    std::exception_ptr first;
-    std::mutex mu;
-    auto work = [&] {
-        try {
-            for (int s0 = next.fetch_add(kChunk); s0 < n; s0 = next.fetch_add(kChunk))
-                for (int s = s0; s < std::min(n, s0 + kChunk); ++s) f(s);
-        } catch (...) {
-            std::lock_guard<std::mutex> lk(mu);
-            if (!first) first = std::current_exception();
-            next = n;
-        }
-    };
-    const int cores = (int)std::thread::hardware_concurrency();
-    const int want = std::min(std::min(cores, kMostThreads), n / (4 * kChunk));
-    std::vector<std::thread> pool;
-    try {
-        for (int t = 1; t < want; ++t) pool.emplace_back(work);
-    } catch (const std::system_error &) {
-        // no more threads to be had: those that started and this one do it
-    }
-    work();
-    for (auto &t : pool) t.join();
-    if (first) std::rethrow_exception(first);
-}
 
 // Bandwidth of an ordering (ord[k] = node) on an undirected graph.
 int bandwidth(const std::vector<std::vector<int>> &adj, const std::vector<int> &ord) {
