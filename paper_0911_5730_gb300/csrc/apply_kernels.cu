@@ -200,7 +200,6 @@ __global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, 
     const size_t bsq = (size_t)b * ldb;
     const int ns = 2 * m - 1;
     RingSlots slots;                      // copies in flight: thread 0's
-    bool ok = true;
     // half s (2 j: Linv_j, 2 j - 1: Lsub_j): its bytes rounded out to 16-byte
     // boundaries, and where it starts in its slot
     auto half_of = [&](int s) { return F + ((size_t)(s + 1) / 2 * 2 + (s & 1)) * bsq; };
@@ -218,7 +217,7 @@ __global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, 
         return reinterpret_cast<const T *>(smem_s + (size_t)(s % ring) * ly.stage + (a & 15));
     };
     auto wait_half = [&](int s) {         // every thread sees the copy's completion itself
-        ok = ok && slots.wait(s % ring, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
+        slots.wait(s % ring, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
     };
     if (tid == 0) {
         for (int q = 0; q < ring; ++q) mbar_init(&bars[q]);
@@ -273,12 +272,12 @@ __global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, 
         }
         wait_half(2 * j);
         __syncthreads();
-        if (tid == 0 && ok && j > 0 && 2 * j - 1 + ring < ns) issue(2 * j - 1 + ring);
+        if (tid == 0 && slots.ok && j > 0 && 2 * j - 1 + ring < ns) issue(2 * j - 1 + ring);
         const T *Li = slot(2 * j);
         rows([&](int rr, int c) { return ld<T, ACC>(Li + fpos(rr, c, ldb, swz)); }, tmp, zero, next,
              [&](int rr, ACC a) { xj[rr] = a; });
         __syncthreads();
-        if (tid == 0 && ok && 2 * j + ring < ns) issue(2 * j + ring);
+        if (tid == 0 && slots.ok && 2 * j + ring < ns) issue(2 * j + ring);
     }
     for (int j = m - 1; j >= 0; --j) {
         ACC *xj = x + j * b;
@@ -293,14 +292,14 @@ __global__ void __launch_bounds__(kSBWide) k_dir_s(DevLevel L, const double *r, 
         }
         if (2 * j < ns - ring) wait_half(2 * j);
         __syncthreads();
-        if (tid == 0 && ok && j < m - 1 && 2 * j + 1 - ring >= 0) issue(2 * j + 1 - ring);
+        if (tid == 0 && slots.ok && j < m - 1 && 2 * j + 1 - ring >= 0) issue(2 * j + 1 - ring);
         const T *Li = slot(2 * j);
         rows([&](int rr, int c) { return ld<T, ACC>(Li + fpos(c, rr, ldb, swz)); }, tmp, self, all,
              [&](int rr, ACC a) { xj[rr] = a; });
         __syncthreads();
-        if (tid == 0 && ok && 2 * j - ring >= 0) issue(2 * j - ring);
+        if (tid == 0 && slots.ok && 2 * j - ring >= 0) issue(2 * j - ring);
     }
-    if (!__syncthreads_and(ok)) {
+    if (!__syncthreads_and(slots.ok)) {
         if (tid == 0) {
             atomicExch(L.err, 1);                         // bounded: copies in flight land first
             slots.drain(ring, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });

@@ -1004,7 +1004,6 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
         for (int s2 = 0; s2 < SBN; ++s2) mbar_init(&bars[s2]);
     __syncthreads();
     RingSlots slots;                      // copies in flight: thread 0's
-    bool ok = true;                       // false once a wait of this thread gave up: it waits no more
     for (int ti = blockIdx.x; ti < count; ti += gridDim.x) {
         const int sub = perm[ti];
         const int nI = L.nI[sub], nG = L.nG[sub], b = L.bsz[sub], m = nI > 0 ? L.nblk[sub] : 0;
@@ -1042,9 +1041,9 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
             return reinterpret_cast<const T *>(ring + (size_t)(s % SBN) * ly.stage + (a & 15));
         };
         auto wait_half = [&](int s) {     // every thread sees the copy's completion itself
-            ok = ok && slots.wait(s % SBN, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
+            slots.wait(s % SBN, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
         };
-        if (tid == 0 && ok)
+        if (tid == 0 && slots.ok)
             for (int s = 0; s < SBN && s < ns; ++s) issue(s);
         {
             // the right-hand side into the scratch, a lane per column, four
@@ -1105,7 +1104,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
             }
             wait_half(2 * j);
             __syncthreads();
-            if (tid == 0 && ok && j > 0 && 2 * j - 1 + SBN < ns) issue(2 * j - 1 + SBN);
+            if (tid == 0 && slots.ok && j > 0 && 2 * j - 1 + SBN < ns) issue(2 * j - 1 + SBN);
             if (colact) {
 #pragma unroll
                 for (int i = 0; i < R; ++i)
@@ -1124,7 +1123,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
                 }
             }
             __syncthreads();
-            if (tid == 0 && ok && 2 * j + SBN < ns) issue(2 * j + SBN);
+            if (tid == 0 && slots.ok && 2 * j + SBN < ns) issue(2 * j + SBN);
         }
         // backward: x_j = Linv_j^T (y_j - Lsub_{j+1}^T x_{j+1}); halves ns-1 ..
         // ns-SBN are still in the ring
@@ -1150,7 +1149,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
             }
             if (2 * j < ns - SBN) wait_half(2 * j);
             __syncthreads();
-            if (tid == 0 && ok && j < m - 1 && 2 * j + 1 - SBN >= 0) issue(2 * j + 1 - SBN);
+            if (tid == 0 && slots.ok && j < m - 1 && 2 * j + 1 - SBN >= 0) issue(2 * j + 1 - SBN);
             if (colact) {
 #pragma unroll
                 for (int i = 0; i < R; ++i)
@@ -1165,9 +1164,9 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
                     }
             }
             __syncthreads();
-            if (tid == 0 && ok && 2 * j - SBN >= 0) issue(2 * j - SBN);
+            if (tid == 0 && slots.ok && 2 * j - SBN >= 0) issue(2 * j - SBN);
         }
-        if (!__syncthreads_and(ok)) break;
+        if (!__syncthreads_and(slots.ok)) break;
         // every issued half has been waited for: the ring is idle from here
         if (!POST) {
             // r_B -= A_{Gamma I} x (Gamma entry q: warp q mod nw, lane: column;
@@ -1277,7 +1276,7 @@ k_dir_bs(DevLevel L, BatchLevel B, const double *r, double *z, const int *skip, 
         }
         __syncthreads();                  // red is free for the next substructure
     }
-    if (!ok) atomicExch(L.err, 1);
+    if (!slots.ok) atomicExch(L.err, 1);
     if (tid == 0)                         // bounded: copies in flight land before the block exits
         slots.drain(SBN, [&](int q, unsigned parity) { return mbar_wait(&bars[q], parity); });
 }

@@ -59,19 +59,19 @@ BDDC_HD constexpr int direction_written(int step) { return 1 - (step & 1); }
 
 // One thread's view of a ring of shared-memory slots filled by bulk copies, a
 // barrier each (barrier s completes once per copy into slot s, with alternating
-// parity).  wait_for(s, parity) polls barrier s a bounded number of times.  A
-// thread whose wait gave up (false) waits and issues no more: the slot still
-// counts as in flight.
+// parity).  wait_for(s, parity) polls barrier s a bounded number of times.
 struct RingSlots {
     unsigned parity = 0;    // bit s: parity of the next completion of slot s
     unsigned pending = 0;   // bit s: a copy that this thread issued is in flight
+    bool ok = true;         // false once a wait gave up: the thread waits and issues no more
 
     BDDC_HD void issued(int s) { pending |= 1u << s; }
-    template <class F> BDDC_HD bool wait(int s, F &&wait_for) {
-        if (!wait_for(s, (parity >> s) & 1u)) return false;
-        parity ^= 1u << s;
-        pending &= ~(1u << s);
-        return true;
+    template <class F> BDDC_HD void wait(int s, F &&wait_for) {
+        if (ok) {
+            ok = wait_for(s, (parity >> s) & 1u);
+            if (ok) pending &= ~(1u << s);
+        }
+        parity ^= (unsigned)ok << s;    // (a slot whose copy did not land keeps its parity for the drain)
     }
     // before the block exits: the copies in flight land
     template <class F> BDDC_HD void drain(int slots, F &&wait_for) const {

@@ -106,8 +106,9 @@ int main() {
 
 
 def test_ring_drains_what_is_in_flight(run):
-    """A ring whose copy number `late` does not land within a wait: the drain
-    waits for every copy in flight, the late one among them."""
+    """A ring whose copy number `late` does not land within a wait: the thread
+    waits and issues no more, and the drain waits for every copy in flight, the
+    late one among them."""
     run(r"""
 #include <initializer_list>
 #include "rules.h"
@@ -115,26 +116,29 @@ using namespace bddc;
 int main() {
     for (int n : {2, 3, 4, 6}) for (int units = 1; units <= 14; ++units) for (int late = -1; late < units; ++late) {
         RingSlots R;
-        bool ok = true;
         unsigned done[8] = {0};                 // completions of each barrier
         bool flight[8] = {false};
-        int copy[8];
+        int copy[8], polls = 0;
         bool slow = true;                       // the late copy lands after the first wait for it
         auto wait_for = [&](int s, unsigned parity) {
+            ++polls;
             if ((done[s] & 1u) != parity) return true;     // that phase has completed: no time passes
-            if (flight[s] && !(copy[s] == late && slow)) { ++done[s]; flight[s] = false; }
+            if (flight[s] && copy[s] == late && slow) { slow = false; return false; }
+            if (flight[s]) { ++done[s]; flight[s] = false; }
             return (done[s] & 1u) != parity;
         };
         auto issue = [&](int u) { flight[u % n] = true; copy[u % n] = u; R.issued(u % n); };
         for (int u = 0; u < n && u < units; ++u) issue(u);
         for (int u = 0; u < units; ++u) {
-            ok = ok && R.wait(u % n, wait_for);
-            if (ok != (late < 0 || u < late)) return 1;
-            if (ok && u + n < units) issue(u + n);
+            const int before = polls;
+            const bool had = R.ok;
+            R.wait(u % n, wait_for);
+            if (!had && polls != before) return 1;
+            if (R.ok != (late < 0 || u < late)) return 2;
+            if (R.ok && u + n < units) issue(u + n);
         }
-        slow = false;
         R.drain(n, wait_for);
-        for (int s = 0; s < n; ++s) if (flight[s]) return 2;
+        for (int s = 0; s < n; ++s) if (flight[s]) return 3;
     }
 }
 """)
