@@ -35,14 +35,14 @@ BDDC_HD constexpr bool stencil_marches(int K) { return K > kMarchMinK; }
 //     streaming, 17 to 32          544   556   848   1456
 //     streaming, up to 16          543   545   596    809
 //     lane                         755   758   776   1175
-//   blocks of 8 rows         169 subs.  256  1024   4096  16384
-//     staged                        95    98   307   1017   3986
-//     streaming                    177   180   223    761   2664
-//     lane                         136   136   216    677   2526
+//   blocks of 8 rows         169 subs.  256   400   484   625   784  1024   4096  16384
+//     staged                        95    98   132   166   204   243   307   1017   3986
+//     streaming                    177   180   183   186   189   202   223    761   2664
+//     lane                         136   136   137   141   206   214   216    677   2526
 // Whether the staged kernel is timed beside the others: not where it lost
 // wherever it was measured, which keeps the first use of a large problem short.
 BDDC_HD constexpr bool fp64_staged_timed(int bp, int nsub, int sms, bool stream) {
-    return bp == 16 ? !(stream && nsub >= sms) : nsub < 6 * sms;
+    return bp == 16 ? !(stream && nsub >= sms) : nsub < 3 * sms;
 }
 // Whether K columns take the lane kernel where it was the fastest for 32: it
 // costs the same for any K, and so does the streaming kernel with blocks of 8
