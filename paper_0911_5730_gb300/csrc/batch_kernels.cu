@@ -2223,17 +2223,17 @@ __global__ void __launch_bounds__(kTT) k_b_scatter(int n, int K, const double *s
             if (g0 + h + lane < n) dst[(int64_t)k * ld + g0 + h + lane] = t.v[k][h + lane];
 }
 
-// A new right-hand side in slot k of a running batch.  Its directions start at
-// zero: the slot's last one is multiplied by beta = 0, which would keep a NaN.
-__global__ void k_b_admit(int n, int K, int k, const double *__restrict__ b, double *x, double *r,
-                          double *p0, double *p1, double *part, unsigned *counter, BatchScalars *sc, double tol, int maxit) {
+// A new right-hand side in slot k of a running batch.  p: the direction buffer
+// that the slot reads when it joins, cleared if the slot's last right-hand side
+// may have left a NaN there (beta = 0 would keep it), else null.
+__global__ void k_b_admit(int n, int K, int k, const double *__restrict__ b, double *x, double *r, double *p,
+                          double *part, unsigned *counter, BatchScalars *sc, double tol, int maxit) {
     double s = 0.0;
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < n; g += gridDim.x * blockDim.x) {
         const double v = b[g];
         x[(int64_t)g * K + k] = 0.0;
         r[(int64_t)g * K + k] = v;
-        p0[(int64_t)g * K + k] = 0.0;
-        p1[(int64_t)g * K + k] = 0.0;
+        if (p) p[(int64_t)g * K + k] = 0.0;
         s = fma(v, v, s);
     }
     grid_reduce_k(s, 1, part, counter,
@@ -3011,11 +3011,11 @@ void launch_b_norm2(int n, int K, const double *v, double *part, unsigned *count
     const int64_t nK = (int64_t)n * K;
     k_b_norm2<<<vgrid_b(nK, K), bblock(K), 0, s>>>(nK, K, v, part, counter, out);
 }
-void launch_b_admit(int n, int K, int k, const double *b, double *x, double *r, double *p0, double *p1,
-                    double *part, unsigned *counter, BatchScalars *sc, double tol, int maxit, cudaStream_t s) {
+void launch_b_admit(int n, int K, int k, const double *b, double *x, double *r, double *p, double *part,
+                    unsigned *counter, BatchScalars *sc, double tol, int maxit, cudaStream_t s) {
     int g = (n + kRB - 1) / kRB;
     if (g > 4 * num_sms_b()) g = 4 * num_sms_b();
-    k_b_admit<<<g, kRB, 0, s>>>(n, K, k, b, x, r, p0, p1, part, counter, sc, tol, maxit);
+    k_b_admit<<<g, kRB, 0, s>>>(n, K, k, b, x, r, p, part, counter, sc, tol, maxit);
 }
 void launch_b_column(int n, int K, int k, const double *x, double *dst, cudaStream_t s) {
     if (n > 0) k_b_column<<<(n + 255) / 256, 256, 0, s>>>(n, K, k, x, dst);

@@ -2639,6 +2639,7 @@ void engine_loop(bddc_server *S, Engine *E) {
         launch_b_init(n, K, BW.bcol, n, BW.x, BW.r, BW.p, BW.part, BW.counter, BW.sc, 1e-8, 1, st);
         BDDC_CUDA_TRY(cudaMemsetAsync(BW.rzcounter, 0, sizeof(unsigned), st));
         BatchScalars &h = *BW.hsc;
+        std::vector<char> spoiled(K, 0);   // the slot's last direction may be NaN or infinite
         std::vector<double> hal, hbe;
         for (;;) {
             std::vector<int> admitted;
@@ -2669,8 +2670,11 @@ void engine_loop(bddc_server *S, Engine *E) {
                 const Request &R = *slot[k].R;
                 BDDC_CUDA_TRY(cudaMemcpyAsync(BW.bcol + (size_t)k * n, R.b.data() + (size_t)slot[k].j * n,
                                               sizeof(double) * n, cudaMemcpyHostToDevice, st));
-                launch_b_admit(n, K, k, BW.bcol + (size_t)k * n, BW.x, BW.r, BW.p, BW.p1, BW.part, BW.counter, BW.sc,
-                               R.rtol, std::min(R.maxit, W->maxit_cap), st);
+                // (it sits out the step h.step and joins at the next one)
+                double *clear = !spoiled[k] ? nullptr : direction_read(h.step + 1) ? BW.p1 : BW.p;
+                launch_b_admit(n, K, k, BW.bcol + (size_t)k * n, BW.x, BW.r, clear, BW.part, BW.counter, BW.sc, R.rtol,
+                               std::min(R.maxit, W->maxit_cap), st);
+                spoiled[k] = 0;
             }
             cudaGraphExec_t g = batch_graph(C, *W, BW, E->prec, K);
             for (int c = 0; c < 2; ++c) BDDC_CUDA_TRY(cudaGraphLaunch(g, st));
@@ -2740,6 +2744,7 @@ void engine_loop(bddc_server *S, Engine *E) {
                     I.kappa_est = lmin > 0 ? lmax / lmin : 0.0;
                     if (status != BDDC_OK && !R.done) R.status = status;
                     if (--R.remaining == 0) finish_request(S, R);
+                    spoiled[k] = !(h.conv[k] && std::isfinite(h.rr[k]));
                     slot[k].R.reset();
                     slot[k].j = -1;
                 }

@@ -387,9 +387,10 @@ void launch_b_residual(int nx, int K, const double *w, const double *b, int64_t 
 void launch_b_norm2(int n, int K, const double *v, double *part, unsigned *counter, double *out,
                     cudaStream_t s);
 // Slot k of a running batch takes a new right-hand side b (device [n]):
-// x(:, k) = p(:, k) = 0, r(:, k) = b, its scalars reset, hold set; all_done cleared.
-void launch_b_admit(int n, int K, int k, const double *b, double *x, double *r, double *p0, double *p1,
-                    double *part, unsigned *counter, BatchScalars *sc, double tol, int maxit, cudaStream_t s);
+// x(:, k) = 0, r(:, k) = b, p(:, k) = 0 (unless p is null), its scalars reset,
+// hold set; all_done cleared.
+void launch_b_admit(int n, int K, int k, const double *b, double *x, double *r, double *p, double *part,
+                    unsigned *counter, BatchScalars *sc, double tol, int maxit, cudaStream_t s);
 // dst[g] = x(g, k)
 void launch_b_column(int n, int K, int k, const double *x, double *dst, cudaStream_t s);
 // mismatches of the integer-operation binary32/binary64 conversions against
