@@ -2002,8 +2002,8 @@ __global__ void k_b_dir_spmv(int nx, int K, const double *__restrict__ w, const 
 }
 
 // The same first half for more than kMarchMinK right-hand sides (a warp costs
-// the FP64 pipe the same for 21 lanes as for 32: 650 against 589 us for 21
-// right-hand sides on 1024^2, 652 against 856 for 32), a lane per
+// the FP64 pipe the same for 21 lanes as for 32: 650 against the tile's 531 us
+// for 21 right-hand sides on 1024^2, 652 against 856 for 32), a lane per
 // right-hand side and no tile: each warp marches up a strip of MW columns with
 // three rows of p_new in registers, so nothing meets at a barrier, and the
 // strips are cut into as many equal segments as there are resident warps (one
